@@ -6,10 +6,10 @@ next frame, the result buffers) is made by ``prepare``; ``run`` is the call per
 frame.  Meshes are voxel bodies cut into tetrahedra: a unit-cube bar, and a capsule
 figure with 15 joints (or more, subdivided) posed by forward kinematics.
 
-The mixed-precision cases fix the SpMV to one thread per row, as a program does that
-wants the same pose to give the same bits on every run: the solver's own timing of
-that shape may otherwise split a row's sum.  Its rows per block stay the solver's
-choice.
+The SpMV is fixed to one thread per row, and in FP64 to 128 rows per block, as a
+program does that wants the same pose to give the same bits on every run: the solver's
+own timing of that shape may otherwise split a row's sum (and, in FP64, order the sums
+of the tiles) in another way each time.
 """
 from __future__ import annotations
 
@@ -276,9 +276,9 @@ def _forces(case, asset, rng):
 
 def _context(case, asset, poses, **over):
     mu, lam = _material(case)
-    opts = dict(precision=case["precision"], rotation=case["rotation"], max_batch=max(1, poses))
-    if case["precision"] == "mixed":
-        opts["spmv_split"] = 1
+    opts = dict(precision=case["precision"], rotation=case["rotation"], max_batch=max(1, poses), spmv_split=1)
+    if case["precision"] == "fp64":
+        opts["tile_rows"] = 128
     if case["penalty"]:
         opts.update(constraint="penalty", k_s=_stiffness(case))
     opts.update(over)
