@@ -51,7 +51,8 @@ __host__ __device__ __forceinline__ T* rec_field(T* rec, size_t np, int f, size_
 }
 
 // Problem states (PCG)
-enum : int { kIdle = 0, kActive = 1, kConverged = 2, kMaxIter = 3 };
+// (kFault: a bounded wait of the resident kernel ran out)
+enum : int { kIdle = 0, kActive = 1, kConverged = 2, kMaxIter = 3, kFault = 4 };
 
 // Per-problem scalars.  Tickets are reset to 0 by the tile that completes them.
 struct ProbScal {

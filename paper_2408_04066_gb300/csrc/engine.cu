@@ -21,6 +21,8 @@ constexpr double kLsNoise = 1.0e-10; // predicted decrease below this * |E|: tak
 constexpr int kPcgTiles[3] = {64, 128, 256};   // PCG rows per block the autotuner times
 constexpr int kPcgChunk = 16;                   // PCG iterations enqueued between convergence checks (no history)
 constexpr int kPcgChunkMin = 16, kPcgChunkMax = 64;   // bounds of a predicted chunk (multiples of 8)
+constexpr int kResStages = 2;                   // 32 KB chunks of A_c^{-1} the resident kernel's ring holds
+constexpr int kResWaves = 2;                    // waves of clusters it may take
 constexpr int kPcgHistSteps = 16;               // Newton steps remembered per slot
 constexpr double kPredTol = 3e-3;   // PCG target of the co-rotational predictor step (at most cg_tol)
 constexpr double kEwGamma = 0.9;    // forcing rule where the Newton model is trusted (see advance)
@@ -94,7 +96,7 @@ mfem_status upload(mfem_ctx* c, U** dst, const U* src, size_t count) {
 
 void free_slots(mfem_ctx* c) {
     SlotDev& S = c->slot;
-    void* ptrs[] = {S.xf, S.xf_prev, S.xpred, S.dcorr, S.tol2, S.coarse_on, S.rcp, S.ec, S.rcs, S.aggq, S.bsplit,
+    void* ptrs[] = {S.xf, S.xf_prev, S.xpred, S.dcorr, S.tol2, S.coarse_on, S.rcp, S.ec, S.rcs, S.aggq, S.bsplit, S.epart, S.rbar,
                     S.x, S.xff, S.qff, S.xprev, S.xp,
                     S.g, S.ge, S.Ke, S.val, S.dinv, S.vec, S.part, S.sc, S.active, S.alpha, S.outbuf};
     for (void* p : ptrs)
@@ -120,9 +122,9 @@ size_t bytes_per_slot(const mfem_ctx* c) {
     return H * 12 * 8 + 4 * n * 3 * 8 + (kt == 4 ? n * 3 * 8 + H * 9 * 8 : 0) + m * 12 * 8 + m * kKe * kt + slots * 9 * kt +
            9 * npad32((int)n) * kt +
            kVecStride * npad32((int)n) * kt + (size_t)part_tiles_for(c) * 4 * 8 + sizeof(ProbScal) + 4 + 8 + 8 +
-           H * 12 * 8 + (c->opt.init == MFEM_INIT_WARM ? 2 * n * 3 * 8 : 0) + 4 + (line_search(c) ? n * 3 * 8 : 0) +
+           H * 12 * 8 + 128 + (c->opt.init == MFEM_INIT_WARM ? 2 * n * 3 * 8 : 0) + 4 + (line_search(c) ? n * 3 * 8 : 0) +
            (c->mesh.coarse_n > 0 ? ((n + 255) / 256) * 24 * 4 + (coarse_ks(c) + 1) * c->mesh.coarse_n * 4 + 128 +
-                                        (size_t)c->mesh.n_agg * 9 * 4 +
+                                        (size_t)c->mesh.n_agg * 9 * 4 + (size_t)4 * coarse_ld(c->mesh.coarse_n) * 4 +
                                         coarse_b_bytes(c->mesh.coarse_n, kCoarseGroupSlots) / kCoarseGroupSlots
                                   : 0);
 }
@@ -167,6 +169,7 @@ mfem_status alloc_slots(mfem_ctx* c, int B) {
     AL(S.alpha, B * sizeof(double));
     AL(S.tol2, B * sizeof(double));
     AL(S.coarse_on, B * sizeof(int));
+    AL(S.rbar, B * (size_t)128);
     if (c->mesh.coarse_n > 0) {
         S.rcp_stride = (((size_t)n + 255) / 256) * (256 / kCoarseRows) * 6;
         AL(S.rcp, B * S.rcp_stride * sizeof(float));
@@ -174,6 +177,7 @@ mfem_status alloc_slots(mfem_ctx* c, int B) {
         S.rcs_stride = ((size_t)c->mesh.coarse_n + 31) & ~(size_t)31;
         AL(S.rcs, B * S.rcs_stride * sizeof(float));
         AL(S.aggq, B * (size_t)c->mesh.n_agg * 9 * sizeof(float));
+        AL(S.epart, B * (size_t)4 * coarse_ld(c->mesh.coarse_n) * sizeof(float));
         AL(S.bsplit, coarse_b_bytes(c->mesh.coarse_n, B));
         CK(cudaMemset(S.bsplit, 0, coarse_b_bytes(c->mesh.coarse_n, B)));   // columns past N stay zero
     }
@@ -198,7 +202,7 @@ mfem_status alloc_slots(mfem_ctx* c, int B) {
     CK(cudaMallocHost((void**)&c->alpha_host, B * sizeof(double)));
     CK(cudaMallocHost((void**)&c->alpha_ring, (size_t)kStageRing * B * sizeof(double)));
     c->ring_pos = 0;
-    size_t dcap = 2 * B * std::max(sizeof(PcgDesc<float>), sizeof(PcgDesc<double>));
+    size_t dcap = 2 * B * (std::max(sizeof(PcgDesc<float>), sizeof(PcgDesc<double>)) + sizeof(ResJob));
     if (dcap > c->descs_cap) {
         if (c->descs_dev) cudaFree(c->descs_dev);
         if (c->descs_host) cudaFreeHost(c->descs_host);
@@ -286,7 +290,7 @@ double element_bytes(const mfem_ctx* c) {
 
 template <typename T>
 void build_descs(std::vector<Group>& gs, int tile, int prec, std::vector<PcgDesc<T>>& out, int& units, int& units_u,
-                 std::vector<CoarseJob>* jobs = nullptr) {
+                 std::vector<CoarseJob>* jobs = nullptr, std::vector<mfem_ctx*>* owner = nullptr) {
     units = 0;
     units_u = 0;
     for (auto& g : gs) {
@@ -338,6 +342,7 @@ void build_descs(std::vector<Group>& gs, int tile, int prec, std::vector<PcgDesc
             units += d.n_tiles;
             units_u += d.n_tiles_u;
             out.push_back(d);
+            if (owner) owner->push_back(c);
         }
         if (jobs && !jobs->empty() && jobs->back().d0 == first && jobs->back().key == c)
             jobs->back().nd = (int)out.size() - first;
@@ -449,6 +454,82 @@ mfem_status launch_chunk(mfem_ctx* c, const PcgDesc<T>* dst, int nd, int units, 
     return MFEM_OK;
 }
 
+// Layout of the resident kernel (k_pcg_resident.cu) for the table, or false if
+// its problems do not fit the chip at once: every problem gets CTAs enough for
+// its rows (kResUnits units of 64 each, whole reduction tiles).  If 16 CTAs
+// hold each problem's rows and matrix, one cluster per problem; else the SMs
+// are shared out in proportion to the rows.
+template <typename T>
+bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vector<mfem_ctx*>& owner, int tile,
+                   ResShape& sh, std::vector<ResJob>& jobs) {
+    const ResLimits& lim = c->res_lim;
+    if (lim.sms <= 0) return false;
+    sh = ResShape{};
+    sh.rtile = sizeof(T) == 8 ? tile : kCoarseRows;
+    const int per_cta = kResUnits * kCoarseRows / sh.rtile;   // tiles a CTA can own
+    const size_t np = d.size();
+    std::vector<int> tiles(np), g(np);
+    std::vector<size_t> bytes(np);
+    int need = 0, most = 0;
+    for (size_t i = 0; i < np; ++i) {
+        if (owner[i]->opt.spmv_split == 2 || (d[i].coarse && !d[i].ctc)) return false;
+        tiles[i] = (d[i].n_rows + sh.rtile - 1) / sh.rtile;
+        bytes[i] = (size_t)owner[i]->plan.slice_ptr.back() * (9 * sizeof(T) + 4);
+        g[i] = (tiles[i] + per_cta - 1) / per_cta;
+        need += g[i];
+        most = std::max(most, g[i]);
+        if (d[i].coarse) sh.b_chunks = std::max(sh.b_chunks, res_part_chunks(d[i].coarse_n));
+    }
+    // chunks of A_c^{-1} a CTA streams per iteration
+    auto ring = [&](const std::vector<int>& gg) {
+        int n_a = 0;
+        for (size_t i = 0; i < np; ++i)
+            if (d[i].coarse)
+                n_a = std::max(n_a, (res_coarse_units(d[i].coarse_n) + gg[i] - 1) / gg[i] * res_part_chunks(d[i].coarse_n));
+        return std::min(n_a, kResStages);
+    };
+    sh.smem = res_smem_max();
+    if (most <= 16) {
+        for (int k = 0, cl = 1; k < kResClusterSizes; ++k, cl *= 2) {
+            std::vector<int> gc(np, cl);
+            sh.stages = ring(gc);
+            sh.v_bytes = sh.smem - res_smem_coarse(sh.stages, sh.b_chunks);
+            bool fits = cl >= most && lim.clusters[k] > 0;
+            for (size_t i = 0; i < np; ++i) fits = fits && bytes[i] <= (size_t)cl * sh.v_bytes;
+            if (!fits || (int)np > kResWaves * lim.clusters[k]) continue;
+            sh.cluster = cl;
+            sh.grid = cl * (int)np;
+            g = gc;
+            break;
+        }
+    }
+    if (sh.cluster == 0) {
+        if (need > lim.sms) return false;
+        for (int left = lim.sms - need; left > 0; --left) {
+            size_t at = np;
+            for (size_t i = 0; i < np; ++i)
+                if (g[i] < tiles[i] && (at == np || (int64_t)tiles[i] * g[at] > (int64_t)tiles[at] * g[i])) at = i;
+            if (at == np) break;
+            ++g[at];
+        }
+        sh.grid = 0;
+        for (int x : g) sh.grid += x;
+        sh.stages = ring(g);
+        sh.v_bytes = sh.smem - res_smem_coarse(sh.stages, sh.b_chunks);
+    }
+    sh.v_bytes &= ~127;
+    jobs.clear();
+    int at = 0;
+    for (size_t i = 0; i < np; ++i) {
+        const mfem_ctx* o = owner[i];
+        const size_t b = d[i].bslot;
+        jobs.push_back(ResJob{at, g[i], o->slot.epart ? o->slot.epart + b * 4 * coarse_ld(o->mesh.coarse_n) : nullptr,
+                              o->slot.rbar + b * 32, o->mesh.Abf});
+        at += g[i];
+    }
+    return true;
+}
+
 template <typename T>
 mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, int split, int max_iters, bool count,
                     bool one_chunk = false, bool slopes = false, bool per_request = false) {
@@ -456,12 +537,17 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
     std::vector<PcgDesc<T>> d;
     std::vector<CoarseJob> jobs;
     int units = 0, units_u = 0;
-    build_descs<T>(gs, tile, prec, d, units, units_u, &jobs);
+    std::vector<mfem_ctx*> owner;
+    build_descs<T>(gs, tile, prec, d, units, units_u, &jobs, &owner);
     if (d.empty()) return MFEM_OK;
+    ResShape rsh;
+    std::vector<ResJob> rjobs;
+    bool resident = max_iters <= 0 && one_chunk && plan_resident<T>(c, d, owner, tile, rsh, rjobs);
     const int nj = (int)jobs.size();
     double coarse_bytes = 0.0;   // A_c^{-1} streamed once per iteration per mesh
     for (const auto& j : jobs) coarse_bytes += j.Abf ? 2.0 * j.N * j.N : 4.0 * j.N * coarse_ld(j.N);
-    const size_t bytes = d.size() * sizeof(PcgDesc<T>);
+    const size_t dbytes = d.size() * sizeof(PcgDesc<T>);
+    const size_t bytes = dbytes + rjobs.size() * sizeof(ResJob);
     if (2 * bytes > c->descs_cap) {   // grow: wait until no copy reads the old buffers
         CK(cudaStreamSynchronize(c->stream));
         if (c->descs_dev) cudaFree(c->descs_dev);
@@ -475,7 +561,8 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
     const size_t off = (size_t)prec * (c->descs_cap / 2);
     char* hst = (char*)c->descs_host + off;
     const PcgDesc<T>* dst = (const PcgDesc<T>*)((char*)c->descs_dev + off);
-    std::memcpy(hst, d.data(), bytes);
+    std::memcpy(hst, d.data(), dbytes);
+    if (!rjobs.empty()) std::memcpy(hst + dbytes, rjobs.data(), bytes - dbytes);
     CK(cudaMemcpyAsync((void*)dst, hst, bytes, cudaMemcpyHostToDevice, c->stream));
     c->grid_blocks = units;
     if (max_iters > 0) {
@@ -510,6 +597,9 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
             }
         }
         chunk = std::min(kPcgChunkMax, std::max(per_request ? kPcgChunkMin : 8, (best + 7) / 8 * 8));
+        // resident: every problem of a batch call runs to its own end (none waits
+        // for another inside the launch); served requests keep the round's length
+        if (resident && !per_request) chunk = cap;
     }
     for (int done = 0; done < cap; done += chunk) {
         const int n_it = std::min(chunk, cap - done);
@@ -520,9 +610,29 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
                     for (int b = 0; b < g.B; ++b)
                         if (g.ph[b].active && g.ph[b].in_pcg) g.ph[b].pcg_launched += n_it;
         int pe = count ? c->prof.begin(2, c->stream) : -1;
-        mfem_status lst = launch_chunk<T>(c, dst, (int)d.size(), units, units_u, tile, split, n_it, jobs);
-        if (lst != MFEM_OK) return lst;
-        if (count) {
+        if (resident) {
+            rsh.iters = n_it;
+            if (rsh.cluster == 0)
+                for (auto& g : gs)
+                    if (g.ctx->slot.prec == prec)
+                        CK(cudaMemsetAsync(g.ctx->slot.rbar, 0, (size_t)128 * g.ctx->slot.cap, c->stream));
+            if (launch_pcg_resident<T>(dst, reinterpret_cast<const ResJob*>((const char*)dst + dbytes), (int)d.size(),
+                                       rsh, c->stream) != cudaSuccess) {
+                cudaGetLastError();
+                c->res_lim.sms = 0;   // the device cannot hold it: streamed kernels from now on
+                resident = false;
+                chunk = kPcgChunk;
+            }
+        }
+        if (!resident) {
+            mfem_status lst = launch_chunk<T>(c, dst, (int)d.size(), units, units_u, tile, split,
+                                              std::min(n_it, kPcgChunkMax), jobs);
+            if (lst != MFEM_OK) return lst;
+        }
+        if (resident && count) {
+            c->prof.end(pe, c->stream);
+            c->prof.launches++;
+        } else if (count) {
             c->prof.end(pe, c->stream);
             int cl = nj;   // coarse kernels: per job the product (fused with the correction on the tensor cores) ...
             bool cuda_core = false;
@@ -558,6 +668,7 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
                 gc->prof.launches++;
             }
         bool any = false;
+        int ran = 0;
         for (auto& g : gs)
             if (g.ctx->slot.prec == prec) {
                 mfem_status st = read_scalars(g.ctx, g.B);
@@ -569,8 +680,20 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
             if (g.ctx->slot.prec != prec) continue;
             if (g.ctx->cerr_host && *g.ctx->cerr_host)
                 return ctx_fail(c, MFEM_ECUDA, "coarse product: a bounded wait in the tensor-core kernel ran out");
-            for (int b = 0; b < g.B; ++b)
-                if (g.ph[b].active && g.ph[b].in_pcg && g.ctx->sc_host[b].state == kActive) any = true;
+            for (int b = 0; b < g.B; ++b) {
+                ProbHost& p = g.ph[b];
+                if (!p.active || !p.in_pcg) continue;
+                const ProbScal& q = g.ctx->sc_host[b];
+                if (q.state == kFault) return ctx_fail(c, MFEM_ECUDA, "PCG: a bounded wait in the resident kernel ran out");
+                any |= q.state == kActive;
+                ran = std::max(ran, q.iter - p.pcg_seen);
+                p.pcg_seen = q.iter;
+            }
+        }
+        if (resident && count) {   // the iterations it ran, counted as the streamed kernels' launch pairs
+            c->prof.pcg_launches += 2 * ran;
+            c->prof.coarse_launches += nj * ran;
+            c->prof.pcg_bytes += coarse_bytes * ran;
         }
         if (!any) break;
     }
@@ -985,6 +1108,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 if (start[b]) {
                     g.ph[b].in_pcg = 1;
                     g.ph[b].pcg_launched = 0;
+                    g.ph[b].pcg_seen = 0;
                 }
         }
     }
@@ -1157,6 +1281,7 @@ mfem_ctx* ctx_slot_clone(mfem_ctx* src, int cap, cudaStream_t stream, mfem_statu
     c->slot.prec = src->slot.prec;
     c->tile_rows = src->tile_rows;
     c->spmv_split = src->spmv_split;
+    c->res_lim = src->res_lim;
     c->owned_by_server = true;
     mfem_status s = MFEM_OK;
     if (cudaMallocHost((void**)&c->cerr_host, sizeof(unsigned)) != cudaSuccess) s = MFEM_ENOMEM;
@@ -1455,6 +1580,10 @@ mfem_status mfem_create(const double* rest_verts, int32_t n, const int32_t* tets
     if (st != MFEM_OK) {
         std::string e2 = c->err;
         return fail(st, e2);
+    }
+    if (res_init(c->res_lim) != cudaSuccess) {   // streamed PCG kernels only
+        cudaGetLastError();
+        c->res_lim = ResLimits();
     }
     if (M.coarse_n > 0 && (st = build_coarse(c)) != MFEM_OK) {
         std::string e2 = c->err;

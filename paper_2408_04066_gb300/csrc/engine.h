@@ -39,6 +39,7 @@ struct ProbHost {
     int spec = 0;
     double spec_e0 = 0.0, spec_slope = 0.0;
     int pcg_launched = 0;   // PCG iterations launched in the current solve
+    int pcg_seen = 0;       // its iteration count at the last readback
 };
 
 // Profile accumulator with a pool of CUDA events on the context stream.
@@ -108,6 +109,7 @@ struct mfem_ctx {
     // PCG chunks captured as CUDA graphs, keyed by the launch parameters
     std::map<std::string, cudaGraphExec_t> graphs;
     bool graphs_off = false;   // capture failed once (e.g. a stream that cannot capture)
+    mfem::ResLimits res_lim;   // what the device holds of the resident PCG kernel (sms = 0: not used)
     mfem_profile last_profile{};
     std::string err;
     bool owned_by_server = false;

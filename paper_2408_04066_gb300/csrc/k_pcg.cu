@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 
 #include "kernels.h"
+#include "pcg_dev.cuh"
 
 namespace mfem {
 
@@ -76,90 +77,6 @@ __device__ __forceinline__ void restrict_units(const float (&r)[3], bool valid, 
         const int k = 6 * (row0 / kCoarseRows + u) + c;   // units past the last aggregate write nothing
         if (bgrp && k < coarse_n) coarse_b_store(bgrp, bslot % kCoarseGroupSlots, k, v);
     }
-}
-
-// ---- vector access ------------------------------------------------------------
-// 3-vectors stored as aligned 4-element groups (x, y, z, 0)
-__device__ __forceinline__ void ld4(const float* p, float (&v)[3]) {
-    const float4 a = *reinterpret_cast<const float4*>(p);
-    v[0] = a.x;
-    v[1] = a.y;
-    v[2] = a.z;
-}
-
-__device__ __forceinline__ void ld4(const double* p, double (&v)[3]) {
-    const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
-    v[0] = a.x;
-    v[1] = a.y;
-    v[2] = b.x;
-}
-
-__device__ __forceinline__ void st4(float* p, float a, float b, float c) {
-    *reinterpret_cast<float4*>(p) = make_float4(a, b, c, 0.f);
-}
-
-__device__ __forceinline__ void st4(double* p, double a, double b, double c) {
-    reinterpret_cast<double2*>(p)[0] = make_double2(a, b);
-    reinterpret_cast<double2*>(p)[1] = make_double2(c, 0.0);
-}
-
-// Per-row contribution to an inner product and its warp sum: float-float in
-// the FP32 path (no FP64 instructions until one conversion per warp), plain
-// FP64 in the FP64 path.
-template <typename T>
-struct Partial;
-
-template <>
-struct Partial<float> {
-    FF v;
-    static __device__ __forceinline__ Partial zero() { return Partial{FF{0.f, 0.f}}; }
-};
-
-template <>
-struct Partial<double> {
-    double v;
-    static __device__ __forceinline__ Partial zero() { return Partial{0.0}; }
-};
-
-__device__ __forceinline__ Partial<float> dot3_partial(float a0, float a1, float a2, float b0, float b1, float b2) {
-    const float a[3] = {a0, a1, a2}, b[3] = {b0, b1, b2};
-    return Partial<float>{ff_dot3(a, b)};
-}
-
-__device__ __forceinline__ Partial<double> dot3_partial(double a0, double a1, double a2, double b0, double b1,
-                                                        double b2) {
-    return Partial<double>{a0 * b0 + a1 * b1 + a2 * b2};
-}
-
-__device__ __forceinline__ double warp_sum_partial(Partial<float> p) { return ff_warp_sum(p.v); }
-
-__device__ __forceinline__ double warp_sum_partial(Partial<double> p) {
-    double v = p.v;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// step coefficients in the kernel's precision
-__device__ __forceinline__ void coeffs(const ProbScal* sc, float& a, float& b) {
-    a = sc->alpha_f;
-    b = sc->beta_f;
-}
-__device__ __forceinline__ void coeffs(const ProbScal* sc, double& a, double& b) {
-    a = sc->alpha;
-    b = sc->beta;
-}
-
-// z_bj = D^{-1} r for one row: D^{-1} row-major 3x3, its entry e of every row
-// stored contiguously (entry e of row `row` at di[e * np + row], np = npad32(n)),
-// so a warp's load of one entry is one contiguous 32-row run
-template <typename T>
-__device__ __forceinline__ void apply_dinv(const T* __restrict__ di, size_t np, int row, const T (&r)[3], T (&z)[3]) {
-    T m[9];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) m[e] = di[e * np + row];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) z[i] = m[3 * i] * r[0] + m[3 * i + 1] * r[1] + m[3 * i + 2] * r[2];
 }
 
 // ---- PCG in single-reduction form --------------------------------------------
@@ -318,9 +235,8 @@ __global__ void __launch_bounds__(TILE * SPLIT, (sizeof(T) == 4 ? 2048 : 1024) /
         a1 += __shfl_xor_sync(0xffffffffu, a1, 16);
         a2 += __shfl_xor_sync(0xffffffffu, a2, 16);
     }
-    // epilogue at uniform control flow with short live ranges (the kernel runs
-    // at 32 registers): each partial is reduced over the warp as soon as it is
-    // formed; rows past the end and the second half of a split row add zeros
+    // epilogue at uniform control flow; rows past the end and the second half of
+    // a split row add zeros
     const bool owner = valid && half == 0;
     if (!owner) a0 = a1 = a2 = 0;
     T ur[3] = {0, 0, 0};
@@ -329,14 +245,44 @@ __global__ void __launch_bounds__(TILE * SPLIT, (sizeof(T) == 4 ? 2048 : 1024) /
         ld4(d.nb + 4 * (size_t)row, ur);
         st4(rec_field(d.rec, np, kRecW, row), a0, a1, a2);
     }
-    double v[3];
-    v[1] = warp_sum_partial(dot3_partial(a0, a1, a2, ur[0], ur[1], ur[2]));
     T r[3] = {0, 0, 0};
     if (owner) ld4(rec_field(d.rec, np, kRecR, row), r);
-    v[0] = warp_sum_partial(dot3_partial(r[0], r[1], r[2], ur[0], ur[1], ur[2]));
-    v[2] = warp_sum_partial(dot3_partial(r[0], r[1], r[2], r[0], r[1], r[2]));
-    double tot[3];
-    if (tile_commit<3>(v, d.part, tile, d.n_tiles, &sc->tk_a, 0, tot, true) && threadIdx.x == 0) {
+    const double v = warp_sums3(dot3_partial(r[0], r[1], r[2], ur[0], ur[1], ur[2]),
+                                dot3_wu(a0, a1, a2, ur[0], ur[1], ur[2]),
+                                dot3_partial(r[0], r[1], r[2], r[0], r[1], r[2]));   // value i in lane i
+    // tile partials and, in the problem's last block, the totals: the sums over
+    // the block's warps by three threads, a value each.  An FP64 instruction takes
+    // a scheduler 64 cycles, and a shuffle tree over the block's warps spends five
+    // levels of them on lanes that hold nothing (200k figure, 16 poses, 128-row
+    // tiles: 117.8 -> 114.0 us an iteration, 800k figure, 4 poses: 90.5 -> 87.1)
+    constexpr int NW = TILE * SPLIT / 32;
+    __shared__ double sm[NW * 3];
+    __shared__ int s_last;
+    if (lane < 3) sm[3 * warp + lane] = v;
+    __syncthreads();
+    if (warp == 0) {
+        if (lane < 3) d.part[4 * tile + lane] = warps_sum<NW>(sm + lane);
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();
+            s_last = atomicAdd(&sc->tk_a, 1u) == (unsigned)(d.n_tiles - 1);
+        }
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    double acc[3] = {0.0, 0.0, 0.0};
+    for (int x = threadIdx.x; x < d.n_tiles; x += TILE * SPLIT)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) acc[i] += *(volatile double*)&d.part[4 * x + i];
+    const double tv = warp_sums3(Partial<double>{acc[0]}, Partial<double>{acc[1]}, Partial<double>{acc[2]});
+    if (lane < 3) sm[3 * warp + lane] = tv;
+    __syncthreads();
+    if (threadIdx.x < 3) sm[threadIdx.x] = warps_sum<NW>(sm + threadIdx.x);   // thread i reads and writes column i
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const double tot[3] = {sm[0], sm[1], sm[2]};
+        sc->tk_a = 0u;
         const double gamma = tot[0], delta = tot[1];
         sc->rr = tot[2];
         if (!(tot[2] > sc->tol2 * sc->rr0)) {   // |r| at target: dx is the solve's result

@@ -1,0 +1,691 @@
+// PCG of problems that fit the chip: one kernel runs every iteration.
+//
+// Same recurrences, same preconditioner and the same arithmetic per row as the
+// streamed kernels (k_pcg.cu, k_coarse_tc.cu); what differs is where things
+// live.  A problem is given a group of CTAs, one per SM; a CTA owns up to
+// kResUnits units of 64 rows, a thread owns one row and keeps its r, p, s, dx,
+// zb and D^{-1} in registers, and the CTA's slices of the matrix sit in shared
+// memory as far as they fit (the rest is read from L2).  Only u, the coarse
+// residual, the coarse partial products and the inner-product partials go
+// through global memory (L2), separated by four group barriers an iteration:
+//
+//   coarse product (tcgen05, the K-range parts of k_coarse_fused as units of
+//   work)  |  u = zb + P e  |  w = K u, dots  |  alpha, beta; p, s, dx, r, zb,
+//   restriction  |
+//
+// A group of at most 16 CTAs is a thread-block cluster and uses the cluster
+// barrier; a larger one is part of a cooperative launch (every CTA resident) and
+// counts arrivals in global memory.  Groups do not wait for one another: each
+// problem ends when it converges.
+//
+// What bounds it: the latency of the barriers and of the L2 round trips between
+// them, not bytes -- these problems are the ones whose streamed iteration is
+// three dependent launches that each leave most of the chip idle.
+//
+// Every wait in global memory or on an mbarrier is bounded by the global timer;
+// one that runs out marks the problem (kFault) and the CTA leaves after its
+// copies in flight have landed and its tensor memory is freed.  A CTA that has
+// left no longer counts in the cluster barrier.
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "kernels.h"
+#include "pcg_dev.cuh"
+#include "tc_dev.cuh"
+
+namespace mfem {
+
+namespace {
+
+constexpr int kResStepB = 16 * 16 * 2;              // bytes of B per K step: 16 columns (hi, mid, lo, zeros)
+constexpr int kResChunkB = kResStepB * kTcSteps;    // 4 KB
+constexpr int kResTmemCols = 32;
+constexpr int kResMaxStages = 8;
+constexpr int kResStatic = 2048;                    // bound of the static shared memory below
+static_assert(kResThreads == 64 * kResUnits, "one thread per row");
+
+// Scalars of one problem's recurrences; every CTA of the group keeps a copy,
+// formed from the same totals.
+struct ResState {
+    double rho, alpha, beta, rr0, rr, tol2;
+    int first, iter, maxit, state;
+};
+
+template <typename T>
+struct ResShared {
+    uint64_t full[kResMaxStages], empty[kResMaxStages], done, vals;
+    uint32_t tmem;
+    int fail;
+    int voff[kResUnits];            // byte offset of a unit's values in the value area, -1: read from global memory
+    int slots[kResUnits];
+    double wsum[kResThreads / 32][3];
+    ResState st;
+    float ws[kResThreads / 32][6];
+    float qs[kResUnits][9];
+};
+static_assert(sizeof(ResShared<double>) <= kResStatic, "static shared memory");
+
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void red_release(unsigned* p) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+// four consecutive FP32 columns of this thread's TMEM lane
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
+    uint32_t r[4];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// w_i = sum over the row's slots, in slot order, NB slots at a time: column ids
+// first, then every neighbour record, then the products.
+template <typename T, int NB, bool SMEM>
+__device__ __forceinline__ void row_product(const int* cp, const T* vp, int w, const T* nb, T& a0, T& a1, T& a2) {
+    for (int k = 0; k < w; k += NB) {
+        int c[NB];
+        T q[NB][3];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) c[i] = k + i < w ? (SMEM ? cp[32 * (k + i)] : __ldg(cp + 32 * (k + i))) : -1;
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            q[i][0] = q[i][1] = q[i][2] = (T)0;
+            if (c[i] >= 0) ld4(nb + 4 * (size_t)c[i], q[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+            if (c[i] >= 0) {
+                const T* vv = vp + 288 * (k + i);
+                T m[9];
+#pragma unroll
+                for (int e = 0; e < 9; ++e) m[e] = SMEM ? vv[32 * e] : __ldg(vv + 32 * e);
+                a0 += m[0] * q[i][0] + m[1] * q[i][1] + m[2] * q[i][2];
+                a1 += m[3] * q[i][0] + m[4] * q[i][1] + m[5] * q[i][2];
+                a2 += m[6] * q[i][0] + m[7] * q[i][1] + m[8] * q[i][2];
+            }
+    }
+}
+
+template <typename T, bool CLUSTER>
+__global__ void __launch_bounds__(kResThreads, 1)
+    k_pcg_resident(const PcgDesc<T>* __restrict__ D, const ResJob* __restrict__ J, int n_probs, ResShape sh) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ ResShared<T> S;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    int p = 0;
+    {
+        int hi = n_probs - 1;
+        while (p < hi) {
+            const int mid = (p + hi + 1) >> 1;
+            if (J[mid].cta0 <= (int)blockIdx.x) p = mid;
+            else hi = mid - 1;
+        }
+    }
+    const PcgDesc<T>& d = D[p];
+    const ResJob job = J[p];
+    const int rank = (int)blockIdx.x - job.cta0, G = job.ncta;
+    ProbScal* sc = d.sc;
+    if (sc->state != kActive) return;   // the same for the whole group: its state is written only after every CTA's last barrier
+    const bool coarse = d.coarse != 0;
+    const int n = d.n_rows, N = d.coarse_n;
+    const int ashift = coarse ? d.agg_shift - 6 : 0;   // units per aggregate (log2)
+    const size_t np = npad32(n);
+
+    // this CTA's units: whole tiles of rtile rows (the reduction's granule)
+    const int gran = sh.rtile / kCoarseRows, n_units = (n + kCoarseRows - 1) / kCoarseRows;
+    const int n_tiles = (n + sh.rtile - 1) / sh.rtile;
+    const int t0 = (int)((long long)n_tiles * rank / G), t1 = (int)((long long)n_tiles * (rank + 1) / G);
+    const int u0 = t0 * gran, nu = min(n_units, t1 * gran) - u0;
+    const int ul = t / kCoarseRows, row = (u0 + ul) * kCoarseRows + (t & (kCoarseRows - 1));
+    const bool valid = ul < nu && row < n;
+
+    // coarse units: part q of the K range of row block rb
+    const int nkc = coarse ? coarse_chunks(N) : 0, c_per = coarse ? coarse_part_chunks(N) : 1;
+    const int nq = coarse ? (nkc + c_per - 1) / c_per : 0, n_cu = coarse ? row_blocks(N) * nq : 0;
+    const int ld_e = coarse_ld(N);
+    unsigned char* bmem = smem + (size_t)sh.stages * kFuChunkA;
+    unsigned char* vmem = bmem + (size_t)sh.b_chunks * kResChunkB;
+    const bool has_cu = rank < n_cu;
+
+    // ---- set-up: barriers, the unit values that fit, the first chunks of A
+    if (t == 0) {
+        for (int i = 0; i < kResMaxStages; ++i) {
+            mbar_init(&S.full[i], 1);
+            mbar_init(&S.empty[i], 1);
+        }
+        mbar_init(&S.done, 1);
+        mbar_init(&S.vals, 1);
+        S.fail = 0;
+        S.st = ResState{sc->rho, sc->alpha, sc->beta, sc->rr0, sc->rr, sc->tol2, sc->first, sc->iter, sc->maxit,
+                        sc->state};
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (t < kResUnits) {
+        int s = 0;
+        if (t < nu) {
+            const int n_slices = (n + 31) >> 5, s0 = 2 * (u0 + t);
+            s = d.slice_ptr[min(n_slices, s0 + 2)] - d.slice_ptr[s0];
+        }
+        S.slots[t] = s;
+    }
+    for (int i = t; i < kResUnits * 9; i += kResThreads) {
+        const int a = (u0 + i / 9) >> ashift;
+        S.qs[i / 9][i % 9] = coarse && i / 9 < nu ? d.aggq[9 * a + i % 9] : 0.f;
+    }
+    if (has_cu)
+        for (int i = t; i < sh.b_chunks * kResChunkB / 16; i += kResThreads)
+            reinterpret_cast<uint4*>(bmem)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    // chunks of A an iteration streams, and the loader's place in them (thread 0)
+    int n_a = 0, l_cu = rank, l_c = 0;
+    long long loaded = 0, used = 0;
+    auto chunks_of = [&](int cu) {
+        const int c_lo = (cu % nq) * c_per;
+        return min(nkc, c_lo + c_per) - c_lo;
+    };
+    auto load_next = [&]() {   // one more chunk into its stage (free by now)
+        const int s = (int)(loaded % sh.stages);
+        const int rb = l_cu / nq, c = (l_cu % nq) * c_per + l_c;
+        mbar_expect_tx(&S.full[s], kFuChunkA);
+        bulk_g2s(smem + (size_t)s * kFuChunkA,
+                 reinterpret_cast<const unsigned char*>(job.Abf) + ((size_t)rb * nkc + c) * kFuChunkA, kFuChunkA,
+                 &S.full[s]);
+        ++loaded;
+        if (++l_c >= chunks_of(l_cu)) {
+            l_c = 0;
+            l_cu += G;
+            if (l_cu >= n_cu) l_cu = rank;
+        }
+    };
+    if (t == 0) {
+        for (int cu = rank; cu < n_cu; cu += G) n_a += chunks_of(cu);
+        int off = 0;
+        uint32_t bytes = 0;
+        for (int i = 0; i < kResUnits; ++i) {
+            const int need = S.slots[i] * (9 * (int)sizeof(T) + 4);
+            const bool fits = i < nu && off + need <= sh.v_bytes;
+            S.voff[i] = fits ? off : -1;
+            if (fits) {
+                off += need;
+                bytes += need;
+            }
+        }
+        if (bytes) {
+            mbar_expect_tx(&S.vals, bytes);
+            for (int i = 0; i < nu; ++i) {
+                if (S.voff[i] < 0 || !S.slots[i]) continue;
+                const size_t base = d.slice_ptr[2 * (u0 + i)];
+                const uint32_t vb = S.slots[i] * 9 * (uint32_t)sizeof(T);
+                bulk_g2s(vmem + S.voff[i], d.val + base * 9, vb, &S.vals);
+                bulk_g2s(vmem + S.voff[i] + vb, d.col + base, S.slots[i] * 4u, &S.vals);
+            }
+        } else {
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&S.vals)) : "memory");
+        }
+        for (int i = 0; i < n_a && i < sh.stages; ++i) load_next();
+    }
+    if (has_cu && warp == 0) {
+        __syncwarp();
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem)),
+                     "r"(kResTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+
+    // ---- the row's state
+    T r[3] = {0, 0, 0}, pp[3] = {0, 0, 0}, ss[3] = {0, 0, 0}, dx[3] = {0, 0, 0}, zb[3] = {0, 0, 0}, di[9];
+    float4 off = make_float4(0.f, 0.f, 0.f, 0.f);
+    int base = 0, w = 0;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) di[e] = 0;
+    if (valid) {
+        ld4(rec_field(d.rec, np, kRecR, row), r);
+        ld4(rec_field(d.rec, np, kRecP, row), pp);
+        ld4(rec_field(d.rec, np, kRecS, row), ss);
+        ld4(rec_field(d.rec, np, kRecDX, row), dx);
+        ld4(rec_field(d.rec, np, kRecZB, row), zb);
+#pragma unroll
+        for (int e = 0; e < 9; ++e) di[e] = d.dinv[e * np + row];
+        if (coarse) off = d.crel[row];
+        const int s = row >> 5;
+        base = __ldg(d.slice_ptr + s);
+        w = (__ldg(d.slice_ptr + s + 1) - base) >> 5;
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = has_cu ? S.tmem : 0u;
+    const int voff = ul < kResUnits ? S.voff[ul] : -1;
+    // value and column pointers of the row's first slot
+    const T* vsm = nullptr;
+    const int* csm = nullptr;
+    if (valid && voff >= 0) {
+        const int rel = base - __ldg(d.slice_ptr + 2 * (u0 + ul));   // slots of the unit before the row's slice
+        vsm = reinterpret_cast<const T*>(vmem + voff) + (size_t)rel * 9 + lane;
+        csm = reinterpret_cast<const int*>(vmem + voff + (size_t)S.slots[ul] * 9 * sizeof(T)) + rel + lane;
+    }
+    if (!mbar_wait(&S.vals, 0)) S.fail = 1;
+    const bool landed = !__syncthreads_or(S.fail);
+
+    unsigned bar_n = 0;
+    uint32_t done_ph = 0;
+    // every write of the group's CTAs before it is visible to their reads after it
+    auto barrier = [&]() {
+        if (CLUSTER) {
+            __syncwarp();
+            asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+            return;
+        }
+        __syncthreads();
+        ++bar_n;
+        if (t == 0) {
+            __threadfence();
+            red_release(job.bar);
+            const unsigned target = bar_n * (unsigned)G;
+            const uint64_t ts = global_ns();
+            while (ld_acquire(job.bar) < target)
+                if (global_ns() - ts > kTcWaitNs) {
+                    S.fail = 1;
+                    break;
+                }
+            __threadfence();
+        }
+        __syncthreads();
+    };
+
+    bool active = true;
+    for (int it = 0; landed && it < sh.iters; ++it) {
+        T u[3] = {zb[0], zb[1], zb[2]};
+        if (coarse) {
+            // ---- coarse product: this CTA's units
+            for (int cu = rank; cu < n_cu; cu += G) {
+                const int rb = cu / nq, q = cu % nq, c_lo = q * c_per, nch = chunks_of(cu);
+                // B: r_c of the part's columns as three BF16 rows, eight columns (one core-matrix row) a thread
+                for (int g = t; g < nch * (kTcKC / 8); g += kResThreads) {
+                    const int k = c_lo * kTcKC + 8 * g;
+                    float v[8];
+                    if (ashift == 0) {
+                        if (k + 7 < N) {
+                            const float4 x = *reinterpret_cast<const float4*>(d.rcp + k);
+                            const float4 y = *reinterpret_cast<const float4*>(d.rcp + k + 4);
+                            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+                            v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) v[e] = k + e < N ? d.rcp[k + e] : 0.f;
+                        }
+                    } else {
+                        for (int e = 0; e < 8; ++e) {
+                            float s = 0.f;
+                            if (k + e < N) {
+                                const int a = (k + e) / 6, comp = (k + e) - 6 * a, e1 = min(n_units, (a + 1) << ashift);
+                                for (int x = a << ashift; x < e1; ++x) s += d.rcp[6 * (size_t)x + comp];
+                            }
+                            v[e] = s;
+                        }
+                    }
+                    uint32_t h[4], m[4], l[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        uint32_t hh[2], mm[2], ll[2];
+#pragma unroll
+                        for (int f = 0; f < 2; ++f) {
+                            const float x = v[2 * e + f];
+                            const __nv_bfloat16 b0 = __float2bfloat16_rn(x);
+                            const float r1 = x - __bfloat162float(b0);
+                            const __nv_bfloat16 b1 = __float2bfloat16_rn(r1);
+                            const __nv_bfloat16 b2 = __float2bfloat16_rn(r1 - __bfloat162float(b1));
+                            hh[f] = __bfloat16_as_ushort(b0);
+                            mm[f] = __bfloat16_as_ushort(b1);
+                            ll[f] = __bfloat16_as_ushort(b2);
+                        }
+                        h[e] = hh[0] | (hh[1] << 16);
+                        m[e] = mm[0] | (mm[1] << 16);
+                        l[e] = ll[0] | (ll[1] << 16);
+                    }
+                    unsigned char* o = bmem + (g >> 4) * kResChunkB + ((g & 15) >> 1) * kResStepB + (g & 1) * 128;
+                    *reinterpret_cast<uint4*>(o) = make_uint4(h[0], h[1], h[2], h[3]);
+                    *reinterpret_cast<uint4*>(o + 16) = make_uint4(m[0], m[1], m[2], m[3]);
+                    *reinterpret_cast<uint4*>(o + 32) = make_uint4(l[0], l[1], l[2], l[3]);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncthreads();
+                if (t == 0) {
+                    constexpr uint32_t idesc = umma_idesc_bf16(kTcM, 16);
+                    const uint32_t a_base = smem_u32(smem), b_base = smem_u32(bmem);
+                    const bool keep = n_a <= sh.stages;   // every chunk stays in its stage
+                    for (int c = 0; c < nch; ++c, ++used) {
+                        const int s = (int)((keep ? used % n_a : used) % sh.stages);
+                        if (!mbar_wait(&S.full[s], keep ? 0u : (uint32_t)(used / sh.stages) & 1u)) {
+                            S.fail = 1;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint32_t a0 = a_base + s * kFuChunkA, b0 = b_base + c * kResChunkB;
+                        for (int k = 0; k < kTcSteps; ++k)
+                            umma_bf16(tmem, umma_desc(a0 + k * kFuStepA, 128, 256),
+                                      umma_desc(b0 + k * kResStepB, 128, 256), idesc, (c > 0 || k > 0) ? 1u : 0u);
+                        if (keep) continue;
+                        umma_commit(&S.empty[s]);
+                        // refill the stage before this one, whose products were issued a chunk ago
+                        if (used > 0 && loaded < used + sh.stages) {
+                            const long long prev = loaded - sh.stages;
+                            if (!mbar_wait(&S.empty[prev % sh.stages], (uint32_t)(prev / sh.stages) & 1u)) {
+                                S.fail = 1;
+                                break;
+                            }
+                            load_next();
+                        }
+                    }
+                    umma_commit(&S.done);
+                }
+                if (!mbar_wait(&S.done, done_ph)) S.fail = 1;
+                done_ph ^= 1u;
+                tc_fence_after();
+                if (warp < kTcM / 32) {
+                    float v[4];
+                    tmem_ld4(tmem + ((uint32_t)(warp * 32) << 16), v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    const int lr = warp * 32 + lane, er = 6 * kFuAggsBlk * rb + lr;
+                    if (lr < 6 * kFuAggsBlk && er < N) job.epart[(size_t)q * ld_e + er] = (v[0] + v[1]) + v[2];
+                }
+                tc_fence_before();
+                __syncthreads();
+                if (S.fail) break;
+            }
+            // the last chunk's stage, for the next iteration
+            if (t == 0 && has_cu && n_a > sh.stages && !S.fail)
+                while (loaded < used + sh.stages) {
+                    const long long prev = loaded - sh.stages;
+                    if (!mbar_wait(&S.empty[prev % sh.stages], (uint32_t)(prev / sh.stages) & 1u)) {
+                        S.fail = 1;
+                        break;
+                    }
+                    load_next();
+                }
+            barrier();
+            if (S.fail) break;
+            // ---- u = zb + Q_a P_i e_a, the parts of e_a added in part order
+            float ev = 0.f;
+            if (lane < 6 && ul < nu) {
+                const int a = (u0 + ul) >> ashift;
+                const float* ep = job.epart + 6 * a + lane;
+                float x[kFuSplit];
+#pragma unroll
+                for (int q = 0; q < kFuSplit; ++q) x[q] = q < nq ? ep[(size_t)q * ld_e] : 0.f;
+#pragma unroll
+                for (int q = 0; q < kFuSplit; ++q) ev += x[q];
+            }
+            const float e0 = __shfl_sync(0xffffffffu, ev, 0), e1 = __shfl_sync(0xffffffffu, ev, 1);
+            const float e2 = __shfl_sync(0xffffffffu, ev, 2), e3 = __shfl_sync(0xffffffffu, ev, 3);
+            const float e4 = __shfl_sync(0xffffffffu, ev, 4), e5 = __shfl_sync(0xffffffffu, ev, 5);
+            if (off.w != 0.f) {
+                const float l0 = e0 + (e4 * off.z - e5 * off.y);
+                const float l1 = e1 + (e5 * off.x - e3 * off.z);
+                const float l2 = e2 + (e3 * off.y - e4 * off.x);
+                const float* Q = S.qs[ul];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) u[i] += (T)(Q[3 * i] * l0 + Q[3 * i + 1] * l1 + Q[3 * i + 2] * l2);
+            }
+        }
+        if (valid) st4(d.nb + 4 * (size_t)row, u[0], u[1], u[2]);
+        barrier();
+        if (S.fail) break;
+        // ---- w = K u and the three inner products
+        T a0 = 0, a1 = 0, a2 = 0;
+        if (vsm) row_product<T, sizeof(T) == 4 ? 8 : 4, true>(csm, vsm, w, d.nb, a0, a1, a2);
+        else if (valid)
+            row_product<T, sizeof(T) == 4 ? 4 : 2, false>(d.col + base + lane, d.val + (size_t)base * 9 + lane, w, d.nb,
+                                                          a0, a1, a2);
+        if (!valid) u[0] = u[1] = u[2] = 0;
+        {
+            const double v1 = warp_sum_partial(dot3_partial(a0, a1, a2, u[0], u[1], u[2]));
+            const double v0 = warp_sum_partial(dot3_partial(r[0], r[1], r[2], u[0], u[1], u[2]));
+            const double v2 = warp_sum_partial(dot3_partial(r[0], r[1], r[2], r[0], r[1], r[2]));
+            if (lane == 0) {
+                S.wsum[warp][0] = v0;
+                S.wsum[warp][1] = v1;
+                S.wsum[warp][2] = v2;
+            }
+        }
+        __syncthreads();
+        {   // a tile's warps in the order of the streamed kernel's block sum
+            const int nt = t1 - t0, nw = sh.rtile / 32;
+            if (t < 3 * nt) {
+                const int tl = t / 3, i = t - 3 * tl;
+                double v[8];
+#pragma unroll
+                for (int x = 0; x < 8; ++x) v[x] = x < nw ? S.wsum[(tl * nw + x) & (kResThreads / 32 - 1)][i] : 0.0;
+                d.part[4 * (size_t)(t0 + tl) + i] =
+                    ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+            }
+        }
+        barrier();
+        if (S.fail) break;
+        {   // totals: FP64 in the streamed kernel's order (rtile threads), FP32 by every thread
+            const int nthr = sizeof(T) == 8 ? sh.rtile : kResThreads;
+            double acc[3] = {0.0, 0.0, 0.0};
+            if (t < nthr)
+                for (int x = t; x < n_tiles; x += nthr)
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) acc[i] += d.part[4 * (size_t)x + i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int i = 0; i < 3; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+            if (lane == 0)
+#pragma unroll
+                for (int i = 0; i < 3; ++i) S.wsum[warp][i] = acc[i];
+            __syncthreads();
+            if (warp == 0) {
+                const int nw = nthr / 32;
+#pragma unroll
+                for (int i = 0; i < 3; ++i) acc[i] = lane < nw ? S.wsum[lane & (kResThreads / 32 - 1)][i] : 0.0;
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+                if (lane == 0) {
+                    ResState& q = S.st;
+                    const double gamma = acc[0], delta = acc[1];
+                    q.rr = acc[2];
+                    if (!(acc[2] > q.tol2 * q.rr0)) {
+                        q.state = kConverged;
+                    } else if (q.iter >= q.maxit) {
+                        q.state = kMaxIter;
+                    } else {
+                        double beta = 0.0, den = delta;
+                        if (!q.first) {
+                            beta = gamma / q.rho;
+                            den = delta - beta * gamma / q.alpha;
+                        }
+                        if (gamma > 0.0 && den > 0.0 && isfinite(gamma) && isfinite(den)) {
+                            q.alpha = gamma / den;
+                            q.beta = beta;
+                            q.rho = gamma;
+                            q.first = 0;
+                            q.iter = q.iter + 1;
+                        } else {
+                            q.alpha = 0.0;
+                            q.beta = 0.0;
+                            q.state = kConverged;
+                        }
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        if (S.st.state != kActive) {
+            active = false;
+            break;
+        }
+        // ---- the update and the restriction of the new residual
+        const T alpha = (T)S.st.alpha, beta = (T)S.st.beta;
+        const T ww[3] = {a0, a1, a2};
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            pp[i] = fma(beta, pp[i], u[i]);
+            ss[i] = fma(beta, ss[i], ww[i]);
+            dx[i] = fma(alpha, pp[i], dx[i]);
+            r[i] = fma(-alpha, ss[i], r[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) zb[i] = di[3 * i] * r[0] + di[3 * i + 1] * r[1] + di[3 * i + 2] * r[2];
+        if (coarse) {
+            float y[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            if (off.w != 0.f) {
+                const float r32[3] = {(float)r[0], (float)r[1], (float)r[2]};
+                const float* Qt = S.qs[ul];
+                const float q0 = Qt[0] * r32[0] + Qt[3] * r32[1] + Qt[6] * r32[2];
+                const float q1 = Qt[1] * r32[0] + Qt[4] * r32[1] + Qt[7] * r32[2];
+                const float q2 = Qt[2] * r32[0] + Qt[5] * r32[1] + Qt[8] * r32[2];
+                y[0] = q0;
+                y[1] = q1;
+                y[2] = q2;
+                y[3] = off.y * q2 - off.z * q1;
+                y[4] = off.z * q0 - off.x * q2;
+                y[5] = off.x * q1 - off.y * q0;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int c = 0; c < 6; ++c) y[c] += __shfl_xor_sync(0xffffffffu, y[c], o);
+            if (lane == 0)
+#pragma unroll
+                for (int c = 0; c < 6; ++c) S.ws[warp][c] = y[c];
+            __syncthreads();
+            if (t < 6 * nu) {
+                const int x = t / 6, c = t - 6 * x;
+                d.rcp[6 * (size_t)(u0 + x) + c] = S.ws[2 * x][c] + S.ws[2 * x + 1][c];
+            }
+            barrier();
+            if (S.fail) break;
+        }
+    }
+
+    // ---- write back: the increment; the other vectors only if the solve goes on
+    if (valid) {
+        st4(rec_field(d.rec, np, kRecDX, row), dx[0], dx[1], dx[2]);
+        if (active) {
+            st4(rec_field(d.rec, np, kRecR, row), r[0], r[1], r[2]);
+            st4(rec_field(d.rec, np, kRecP, row), pp[0], pp[1], pp[2]);
+            st4(rec_field(d.rec, np, kRecS, row), ss[0], ss[1], ss[2]);
+            st4(rec_field(d.rec, np, kRecZB, row), zb[0], zb[1], zb[2]);
+        }
+    }
+    if (t == 0) {
+        if (S.fail) {
+            sc->state = kFault;
+        } else if (rank == 0) {
+            sc->rho = S.st.rho;
+            sc->alpha = S.st.alpha;
+            sc->beta = S.st.beta;
+            sc->alpha_f = (float)S.st.alpha;
+            sc->beta_f = (float)S.st.beta;
+            sc->rr = S.st.rr;
+            sc->first = S.st.first;
+            sc->iter = S.st.iter;
+            sc->state = S.st.state;
+        }
+        // copies in flight land before the memory is released
+        const bool keep = n_a <= sh.stages;
+        if (keep) {
+            for (int i = 0; i < n_a; ++i) mbar_wait(&S.full[i], 0);
+        } else {
+            for (long long i = used; i < loaded; ++i)
+                mbar_wait(&S.full[i % sh.stages], (uint32_t)(i / sh.stages) & 1u);
+        }
+    }
+    __syncthreads();
+    if (has_cu && warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kResTmemCols)
+                     : "memory");
+}
+
+template <typename T, bool CLUSTER>
+cudaError_t res_attr(int smem) {
+    cudaError_t e = cudaFuncSetAttribute(k_pcg_resident<T, CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess && CLUSTER)
+        e = cudaFuncSetAttribute(k_pcg_resident<T, CLUSTER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
+
+template <typename T>
+void res_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, const ResShape& sh, cudaStream_t s) {
+    cfg = cudaLaunchConfig_t{};
+    if (sh.cluster > 0) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = sh.cluster;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+    } else {
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+    }
+    cfg.gridDim = dim3(sh.grid);
+    cfg.blockDim = dim3(kResThreads);
+    cfg.dynamicSmemBytes = sh.smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+}
+
+}  // namespace
+
+int res_smem_max() { return 227 * 1024 - kResStatic; }
+int res_smem_coarse(int stages, int b_chunks) { return stages * kFuChunkA + b_chunks * kResChunkB; }
+int res_part_chunks(int N) { return coarse_part_chunks(N); }
+int res_coarse_units(int N) {
+    const int nkc = coarse_chunks(N), c_per = coarse_part_chunks(N);
+    return row_blocks(N) * ((nkc + c_per - 1) / c_per);
+}
+
+cudaError_t res_init(ResLimits& lim) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim.sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = res_attr<float, true>(res_smem_max());
+    if (e == cudaSuccess) e = res_attr<float, false>(res_smem_max());
+    if (e == cudaSuccess) e = res_attr<double, true>(res_smem_max());
+    if (e == cudaSuccess) e = res_attr<double, false>(res_smem_max());
+    if (e != cudaSuccess) return e;
+    for (int i = 0, c = 1; i < kResClusterSizes; ++i, c *= 2) {   // clusters of 1, 2, 4, 8, 16 CTAs resident at once
+        ResShape sh{};
+        sh.grid = c;
+        sh.cluster = c;
+        sh.smem = res_smem_max();
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr[1];
+        res_config<double>(cfg, attr, sh, nullptr);
+        int nf = 0, nd = 0;
+        if (cudaOccupancyMaxActiveClusters(&nf, k_pcg_resident<float, true>, &cfg) != cudaSuccess) nf = 0;
+        if (cudaOccupancyMaxActiveClusters(&nd, k_pcg_resident<double, true>, &cfg) != cudaSuccess) nd = 0;
+        cudaGetLastError();
+        lim.clusters[i] = nf < nd ? nf : nd;
+    }
+    return cudaSuccess;
+}
+
+template <typename T>
+cudaError_t launch_pcg_resident(const PcgDesc<T>* descs, const ResJob* jobs, int n_probs, const ResShape& sh,
+                                cudaStream_t s) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    res_config<T>(cfg, attr, sh, s);
+    if (sh.cluster > 0) return cudaLaunchKernelEx(&cfg, k_pcg_resident<T, true>, descs, jobs, n_probs, sh);
+    return cudaLaunchKernelEx(&cfg, k_pcg_resident<T, false>, descs, jobs, n_probs, sh);
+}
+
+template cudaError_t launch_pcg_resident<float>(const PcgDesc<float>*, const ResJob*, int, const ResShape&, cudaStream_t);
+template cudaError_t launch_pcg_resident<double>(const PcgDesc<double>*, const ResJob*, int, const ResShape&,
+                                                 cudaStream_t);
+
+}  // namespace mfem

@@ -78,6 +78,8 @@ struct SlotDev {
     float* rcs = nullptr;    // [B][rcs_stride] per-aggregate coarse residual (aggregates over 64 rows)
     float* aggq = nullptr;   // [B][n_agg][9] rotation of each aggregate's coarse modes for the current solve
     uint16_t* bsplit = nullptr;  // tensor-core coarse product: B operand, [ceil(B/16)][chunks][48 x 256] BF16
+    float* epart = nullptr;  // [B][4][coarse_ld(coarse_n)] partial coarse products of the resident PCG
+    unsigned* rbar = nullptr;   // [B][32] group barriers of the resident PCG (one word per 128 bytes)
     size_t rcs_stride = 0;
     size_t rcp_stride = 0;
     double* outbuf = nullptr;  // [B][n][3] caller-order staging
@@ -168,6 +170,36 @@ template <typename T>
 cudaError_t launch_pcg_iters(const PcgDesc<T>* descs_dev, int n_probs, int n_units, int n_units_u, int tile_rows,
                              int split, int iters, const CoarseJob* jobs, int n_jobs, cudaStream_t s);
 bool pcg_tile_supported(int tile_rows);
+
+// PCG of problems that fit the chip (k_pcg_resident.cu): problem i of the
+// descriptor table runs on CTAs cta0 .. cta0 + ncta - 1 of one launch.
+constexpr int kResUnits = 8;                   // units of 64 rows a CTA may own
+constexpr int kResThreads = 64 * kResUnits;    // one thread per row
+constexpr int kResClusterSizes = 5;            // cluster sizes 1, 2, 4, 8, 16
+struct ResJob {
+    int cta0, ncta;
+    float* epart;      // [4][coarse_ld(N)] partial coarse products
+    unsigned* bar;     // arrivals of the group's global barrier, zero at the launch
+    const void* Abf;   // packed BF16 rows of the mesh's A_c^{-1}
+};
+struct ResShape {
+    int grid, cluster;   // CTAs; CTAs per cluster (every group's size), 0: cooperative launch
+    int rtile;           // rows per reduction tile: a CTA owns whole tiles
+    int iters;           // most iterations of this launch
+    int stages, b_chunks, v_bytes, smem;   // shared memory: A ring, B chunks, matrix values, all
+};
+struct ResLimits {
+    int sms = 0;
+    int clusters[kResClusterSizes] = {0, 0, 0, 0, 0};   // clusters of each size resident at once
+};
+cudaError_t res_init(ResLimits& lim);   // kernel attributes and limits of the current device
+int res_smem_max();
+int res_smem_coarse(int stages, int b_chunks);
+int res_part_chunks(int N);    // chunks of the K range a coarse unit takes (b_chunks)
+int res_coarse_units(int N);   // coarse units of one product
+template <typename T>
+cudaError_t launch_pcg_resident(const PcgDesc<T>* descs, const ResJob* jobs, int n_probs, const ResShape& sh,
+                                cudaStream_t s);
 
 // Coarse space set-up: A_c = P^T K P of the assembled matrix `val` (problem 0 of
 // a slot, precision prec) and its FP32 inverse into Ainv (coarse_n rows of
