@@ -21,7 +21,7 @@ constexpr double kLsNoise = 1.0e-10; // predicted decrease below this * |E|: tak
 constexpr int kPcgTiles[3] = {64, 128, 256};   // PCG rows per block the autotuner times
 constexpr int kPcgChunk = 16;                   // PCG iterations enqueued between convergence checks (no history)
 constexpr int kPcgChunkMin = 16, kPcgChunkMax = 64;   // bounds of a predicted chunk (multiples of 8)
-constexpr int kResStages = 2;                   // 32 KB chunks of A_c^{-1} the resident kernel's ring holds
+constexpr int kResStages = 4;                   // 32 KB chunks of A_c^{-1} the resident kernel's ring holds
 constexpr int kResWaves = 2;                    // waves of clusters it may take
 constexpr int kPcgHistSteps = 16;               // Newton steps remembered per slot
 constexpr double kPredTol = 3e-3;   // PCG target of the co-rotational predictor step (at most cg_tol)
@@ -456,7 +456,7 @@ mfem_status launch_chunk(mfem_ctx* c, const PcgDesc<T>* dst, int nd, int units, 
 
 // Layout of the resident kernel (k_pcg_resident.cu) for the table, or false if
 // its problems do not fit the chip at once: every problem gets CTAs enough for
-// its rows (kResUnits units of 64 each, whole reduction tiles).  If 16 CTAs
+// its rows (kResUnits units of 64 each).  If 16 CTAs
 // hold each problem's rows and matrix, one cluster per problem; else the SMs
 // are shared out in proportion to the rows.
 template <typename T>
@@ -465,17 +465,16 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
     const ResLimits& lim = c->res_lim;
     if (lim.sms <= 0) return false;
     sh = ResShape{};
-    sh.rtile = sizeof(T) == 8 ? tile : kCoarseRows;
-    const int per_cta = kResUnits * kCoarseRows / sh.rtile;   // tiles a CTA can own
+    sh.rtile = tile;
     const size_t np = d.size();
-    std::vector<int> tiles(np), g(np);
+    std::vector<int> units(np), g(np);
     std::vector<size_t> bytes(np);
     int need = 0, most = 0;
     for (size_t i = 0; i < np; ++i) {
         if (owner[i]->opt.spmv_split == 2 || (d[i].coarse && !d[i].ctc)) return false;
-        tiles[i] = (d[i].n_rows + sh.rtile - 1) / sh.rtile;
+        units[i] = (d[i].n_rows + kCoarseRows - 1) / kCoarseRows;
         bytes[i] = (size_t)owner[i]->plan.slice_ptr.back() * (9 * sizeof(T) + 4);
-        g[i] = (tiles[i] + per_cta - 1) / per_cta;
+        g[i] = (units[i] + kResUnits - 1) / kResUnits;
         need += g[i];
         most = std::max(most, g[i]);
         if (d[i].coarse) sh.b_chunks = std::max(sh.b_chunks, res_part_chunks(d[i].coarse_n));
@@ -486,21 +485,27 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
         for (size_t i = 0; i < np; ++i)
             if (d[i].coarse)
                 n_a = std::max(n_a, (res_coarse_units(d[i].coarse_n) + gg[i] - 1) / gg[i] * res_part_chunks(d[i].coarse_n));
-        return std::min(n_a, kResStages);
+        return std::min(std::max(0, n_a - res_tmem_chunks()), kResStages);   // the first ones stay in tensor memory
     };
     sh.smem = res_smem_max();
     if (most <= 16) {
-        for (int k = 0, cl = 1; k < kResClusterSizes; ++k, cl *= 2) {
+        // the largest cluster size that leaves no CTA without rows and runs every
+        // problem at once: a smaller one halves the SMs that read a problem's matrix
+        // (11k tets, 47 units: 16 us an iteration on 8 CTAs, 11 on 16)
+        int least = 0;
+        for (size_t i = 0; i < np; ++i) least = i ? std::min(least, units[i]) : units[i];
+        for (int k = kResClusterSizes - 1, cl = 16; k >= 0 && sh.cluster == 0; --k, cl /= 2) {
+            if (cl < most || lim.clusters[k] <= 0 || (cl >= 2 * least && cl > most)) continue;
+            if ((int)np > lim.clusters[k] && cl / 2 >= most) continue;
             std::vector<int> gc(np, cl);
             sh.stages = ring(gc);
             sh.v_bytes = sh.smem - res_smem_coarse(sh.stages, sh.b_chunks);
-            bool fits = cl >= most && lim.clusters[k] > 0;
+            bool fits = (int)np <= kResWaves * lim.clusters[k];
             for (size_t i = 0; i < np; ++i) fits = fits && bytes[i] <= (size_t)cl * sh.v_bytes;
-            if (!fits || (int)np > kResWaves * lim.clusters[k]) continue;
+            if (!fits) break;
             sh.cluster = cl;
             sh.grid = cl * (int)np;
             g = gc;
-            break;
         }
     }
     if (sh.cluster == 0) {
@@ -508,7 +513,7 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
         for (int left = lim.sms - need; left > 0; --left) {
             size_t at = np;
             for (size_t i = 0; i < np; ++i)
-                if (g[i] < tiles[i] && (at == np || (int64_t)tiles[i] * g[at] > (int64_t)tiles[at] * g[i])) at = i;
+                if (g[i] < units[i] && (at == np || (int64_t)units[i] * g[at] > (int64_t)units[at] * g[i])) at = i;
             if (at == np) break;
             ++g[at];
         }
@@ -520,7 +525,10 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
     sh.v_bytes &= ~127;
     jobs.clear();
     int at = 0;
+    sh.units = 4;
     for (size_t i = 0; i < np; ++i) {
+        const int nu = (units[i] + g[i] - 1) / g[i];   // the kernel's split: the remainder goes to the last CTAs
+        sh.units = std::max(sh.units, nu <= 4 ? 4 : (nu <= 6 ? 6 : 8));
         const mfem_ctx* o = owner[i];
         const size_t b = d[i].bslot;
         jobs.push_back(ResJob{at, g[i], o->slot.epart ? o->slot.epart + b * 4 * coarse_ld(o->mesh.coarse_n) : nullptr,

@@ -20,7 +20,14 @@
 //
 // What bounds it: the latency of the barriers and of the L2 round trips between
 // them, not bytes -- these problems are the ones whose streamed iteration is
-// three dependent launches that each leave most of the chip idle.
+// three dependent launches that each leave most of the chip idle.  An iteration,
+// streamed and here: 11k tets, one pose, 18.9 -> 11.4 us; 10k tets, 5 poses, 23.4
+// -> 10.8; 50k tets, 3 poses, 26.1 -> 13.9; 200k tets, one pose, 41.0 -> 17.1.
+//
+// The chunks of A_c^{-1} a CTA multiplies stay in tensor memory (seven of its
+// units' 32 KB chunks; the eighth and later ones in shared memory): streaming
+// them from L2 every iteration took 19000 of its 58000 cycles on the 200k figure,
+// and an MMA whose A comes from tensor memory issues in 59 cycles instead of 165.
 //
 // Every wait in global memory or on an mbarrier is bounded by the global timer;
 // one that runs out marks the problem (kFault) and the CTA leaves after its
@@ -41,16 +48,20 @@ namespace {
 
 constexpr int kResStepB = 16 * 16 * 2;              // bytes of B per K step: 16 columns (hi, mid, lo, zeros)
 constexpr int kResChunkB = kResStepB * kTcSteps;    // 4 KB
-constexpr int kResTmemCols = 32;
+constexpr int kResTmemD = 32;                       // tensor-memory columns before the chunks of A: the accumulator
+constexpr int kResTmemChunk = kTcKC / 2;            // columns a chunk takes (two BF16 a word)
+constexpr int kResTmemChunks = 7;                   // chunks tensor memory holds (512 columns)
+static_assert(kResTmemD + kResTmemChunks * kResTmemChunk <= 512, "tensor memory");
 constexpr int kResMaxStages = 8;
 constexpr int kResStatic = 2048;                    // bound of the static shared memory below
-static_assert(kResThreads == 64 * kResUnits, "one thread per row");
+constexpr int kResMaxThreads = kCoarseRows * kResUnits;   // one thread per row
 
 // Scalars of one problem's recurrences; every CTA of the group keeps a copy,
 // formed from the same totals.
 struct ResState {
     double rho, alpha, beta, rr0, rr, tol2;
     int first, iter, maxit, state;
+    double inv_rho, inv_alpha;   // FP32 path: 1 / rho and 1 / alpha, formed while the others update their rows
 };
 
 template <typename T>
@@ -60,9 +71,9 @@ struct ResShared {
     int fail;
     int voff[kResUnits];            // byte offset of a unit's values in the value area, -1: read from global memory
     int slots[kResUnits];
-    double wsum[kResThreads / 32][3];
+    double wsum[kResMaxThreads / 32][3];
     ResState st;
-    float ws[kResThreads / 32][6];
+    float ws[kResMaxThreads / 32][6];
     float qs[kResUnits][9];
 };
 static_assert(sizeof(ResShared<double>) <= kResStatic, "static shared memory");
@@ -85,37 +96,58 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
     for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// w_i = sum over the row's slots, in slot order, NB slots at a time: column ids
-// first, then every neighbour record, then the products.
-template <typename T, int NB, bool SMEM>
-__device__ __forceinline__ void row_product(const int* cp, const T* vp, int w, const T* nb, T& a0, T& a1, T& a2) {
-    for (int k = 0; k < w; k += NB) {
-        int c[NB];
-        T q[NB][3];
-#pragma unroll
-        for (int i = 0; i < NB; ++i) c[i] = k + i < w ? (SMEM ? cp[32 * (k + i)] : __ldg(cp + 32 * (k + i))) : -1;
-#pragma unroll
-        for (int i = 0; i < NB; ++i) {
-            q[i][0] = q[i][1] = q[i][2] = (T)0;
-            if (c[i] >= 0) ld4(nb + 4 * (size_t)c[i], q[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < NB; ++i)
-            if (c[i] >= 0) {
-                const T* vv = vp + 288 * (k + i);
-                T m[9];
-#pragma unroll
-                for (int e = 0; e < 9; ++e) m[e] = SMEM ? vv[32 * e] : __ldg(vv + 32 * e);
-                a0 += m[0] * q[i][0] + m[1] * q[i][1] + m[2] * q[i][2];
-                a1 += m[3] * q[i][0] + m[4] * q[i][1] + m[5] * q[i][2];
-                a2 += m[6] * q[i][0] + m[7] * q[i][1] + m[8] * q[i][2];
-            }
-    }
+// eight 32-bit columns of this thread's TMEM lane
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, uint4 a, uint4 b) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(a.x),
+                 "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+// MMA with A in tensor memory
+__device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
+                                             uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
 }
 
-template <typename T, bool CLUSTER>
-__global__ void __launch_bounds__(kResThreads, 1)
+// The neighbour records of up to NB slots of a row (zero ids: none)
+template <typename T, int NB>
+__device__ __forceinline__ void gather(const T* nb, const int (&c)[NB], T (&q)[NB][3]) {
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        q[i][0] = q[i][1] = q[i][2] = (T)0;
+        if (c[i] >= 0) ld4(nb + 4 * (size_t)c[i], q[i]);
+    }
+}
+template <int NB>
+__device__ __forceinline__ void load_cols(const int* cp, int k, int w, int (&c)[NB]) {
+#pragma unroll
+    for (int i = 0; i < NB; ++i) c[i] = k + i < w ? cp[32 * (k + i)] : -1;
+}
+// w_i += those slots' products, in slot order
+template <typename T, int NB>
+__device__ __forceinline__ void products(const T* vp, const int (&c)[NB], const T (&q)[NB][3], T& a0, T& a1, T& a2) {
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+        if (c[i] >= 0) {
+            const T* vv = vp + 288 * i;
+            a0 += vv[0] * q[i][0] + vv[32] * q[i][1] + vv[64] * q[i][2];
+            a1 += vv[96] * q[i][0] + vv[128] * q[i][1] + vv[160] * q[i][2];
+            a2 += vv[192] * q[i][0] + vv[224] * q[i][1] + vv[256] * q[i][2];
+        }
+}
+
+// U: most units a CTA of this launch owns (registers: 255, 168 or 128 a thread
+// for U = 4, 6, 8)
+template <typename T, bool CLUSTER, int U>
+__global__ void __launch_bounds__(kCoarseRows * U, 1)
     k_pcg_resident(const PcgDesc<T>* __restrict__ D, const ResJob* __restrict__ J, int n_probs, ResShape sh) {
+    constexpr int kThreads = kCoarseRows * U;
+    // neighbour records in flight a thread: a whole row's where the registers allow
+    constexpr int NB = sizeof(T) == 4 ? (U <= 6 ? 16 : 8) : (U <= 4 ? 8 : 4);
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ ResShared<T> S;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -138,11 +170,11 @@ __global__ void __launch_bounds__(kResThreads, 1)
     const int ashift = coarse ? d.agg_shift - 6 : 0;   // units per aggregate (log2)
     const size_t np = npad32(n);
 
-    // this CTA's units: whole tiles of rtile rows (the reduction's granule)
-    const int gran = sh.rtile / kCoarseRows, n_units = (n + kCoarseRows - 1) / kCoarseRows;
-    const int n_tiles = (n + sh.rtile - 1) / sh.rtile;
-    const int t0 = (int)((long long)n_tiles * rank / G), t1 = (int)((long long)n_tiles * (rank + 1) / G);
-    const int u0 = t0 * gran, nu = min(n_units, t1 * gran) - u0;
+    // this CTA's units u0 .. u0 + nu - 1; the last CTAs, which have no coarse unit
+    // when there are fewer of those than CTAs, take the remainder
+    const int n_units = (n + kCoarseRows - 1) / kCoarseRows;
+    const int u_rem = G - n_units % G;
+    const int u0 = (n_units / G) * rank + max(0, rank - u_rem), nu = n_units / G + (rank >= u_rem ? 1 : 0);
     const int ul = t / kCoarseRows, row = (u0 + ul) * kCoarseRows + (t & (kCoarseRows - 1));
     const bool valid = ul < nu && row < n;
 
@@ -151,8 +183,9 @@ __global__ void __launch_bounds__(kResThreads, 1)
     const int nq = coarse ? (nkc + c_per - 1) / c_per : 0, n_cu = coarse ? row_blocks(N) * nq : 0;
     const int ld_e = coarse_ld(N);
     unsigned char* bmem = smem + (size_t)sh.stages * kFuChunkA;
-    unsigned char* vmem = bmem + (size_t)sh.b_chunks * kResChunkB;
     const bool has_cu = rank < n_cu;
+    unsigned char* vmem = has_cu ? bmem + (size_t)sh.b_chunks * kResChunkB : smem;
+    const int v_bytes = has_cu ? sh.v_bytes : sh.smem;
 
     // ---- set-up: barriers, the unit values that fit, the first chunks of A
     if (t == 0) {
@@ -164,7 +197,11 @@ __global__ void __launch_bounds__(kResThreads, 1)
         mbar_init(&S.vals, 1);
         S.fail = 0;
         S.st = ResState{sc->rho, sc->alpha, sc->beta, sc->rr0, sc->rr, sc->tol2, sc->first, sc->iter, sc->maxit,
-                        sc->state};
+                        sc->state, 0.0, 0.0};
+        if (!S.st.first) {
+            S.st.inv_rho = 1.0 / S.st.rho;
+            S.st.inv_alpha = 1.0 / S.st.alpha;
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -176,42 +213,58 @@ __global__ void __launch_bounds__(kResThreads, 1)
         }
         S.slots[t] = s;
     }
-    for (int i = t; i < kResUnits * 9; i += kResThreads) {
+    for (int i = t; i < kResUnits * 9; i += kThreads) {
         const int a = (u0 + i / 9) >> ashift;
         S.qs[i / 9][i % 9] = coarse && i / 9 < nu ? d.aggq[9 * a + i % 9] : 0.f;
     }
     if (has_cu)
-        for (int i = t; i < sh.b_chunks * kResChunkB / 16; i += kResThreads)
+        for (int i = t; i < sh.b_chunks * kResChunkB / 16; i += kThreads)
             reinterpret_cast<uint4*>(bmem)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    // chunks of A an iteration streams, and the loader's place in them (thread 0)
-    int n_a = 0, l_cu = rank, l_c = 0;
-    long long loaded = 0, used = 0;
+    // chunks of A of this CTA's units, in order: the first kResTmemChunks stay in
+    // tensor memory, the others go through the shared-memory ring (and stay there
+    // if it holds them all)
     auto chunks_of = [&](int cu) {
         const int c_lo = (cu % nq) * c_per;
         return min(nkc, c_lo + c_per) - c_lo;
     };
+    auto chunk_ptr = [&](int cu, int c) {
+        return reinterpret_cast<const unsigned char*>(job.Abf) +
+               ((size_t)(cu / nq) * nkc + (cu % nq) * c_per + c) * kFuChunkA;
+    };
+    int n_a = 0;
+    for (int cu = rank; cu < n_cu; cu += G) n_a += chunks_of(cu);
+    const int n_tm = min(n_a, kResTmemChunks), n_ring = n_a - n_tm;
+    const bool keep = n_ring <= sh.stages;
+    const uint32_t tm_need = kResTmemD + n_tm * kResTmemChunk;
+    const uint32_t tm_cols = tm_need <= 32 ? 32 : (tm_need <= 128 ? 128 : (tm_need <= 256 ? 256 : 512));
+    int l_cu = rank, l_c = 0;            // the ring's next chunk (thread 0)
+    long long loaded = 0, used = 0;
+    auto ring_start = [&]() {            // first chunk past the ones in tensor memory
+        l_cu = rank;
+        l_c = n_tm;
+        while (l_cu < n_cu && l_c >= chunks_of(l_cu)) {
+            l_c -= chunks_of(l_cu);
+            l_cu += G;
+        }
+    };
     auto load_next = [&]() {   // one more chunk into its stage (free by now)
         const int s = (int)(loaded % sh.stages);
-        const int rb = l_cu / nq, c = (l_cu % nq) * c_per + l_c;
         mbar_expect_tx(&S.full[s], kFuChunkA);
-        bulk_g2s(smem + (size_t)s * kFuChunkA,
-                 reinterpret_cast<const unsigned char*>(job.Abf) + ((size_t)rb * nkc + c) * kFuChunkA, kFuChunkA,
-                 &S.full[s]);
+        bulk_g2s(smem + (size_t)s * kFuChunkA, chunk_ptr(l_cu, l_c), kFuChunkA, &S.full[s]);
         ++loaded;
         if (++l_c >= chunks_of(l_cu)) {
             l_c = 0;
             l_cu += G;
-            if (l_cu >= n_cu) l_cu = rank;
+            if (l_cu >= n_cu) ring_start();
         }
     };
     if (t == 0) {
-        for (int cu = rank; cu < n_cu; cu += G) n_a += chunks_of(cu);
         int off = 0;
         uint32_t bytes = 0;
         for (int i = 0; i < kResUnits; ++i) {
             const int need = S.slots[i] * (9 * (int)sizeof(T) + 4);
-            const bool fits = i < nu && off + need <= sh.v_bytes;
+            const bool fits = i < nu && off + need <= v_bytes;
             S.voff[i] = fits ? off : -1;
             if (fits) {
                 off += need;
@@ -230,12 +283,13 @@ __global__ void __launch_bounds__(kResThreads, 1)
         } else {
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&S.vals)) : "memory");
         }
-        for (int i = 0; i < n_a && i < sh.stages; ++i) load_next();
+        ring_start();
+        for (int i = 0; i < n_ring && i < sh.stages; ++i) load_next();
     }
     if (has_cu && warp == 0) {
         __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem)),
-                     "r"(kResTmemCols)
+                     "r"(tm_cols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -263,32 +317,62 @@ __global__ void __launch_bounds__(kResThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = has_cu ? S.tmem : 0u;
-    const int voff = ul < kResUnits ? S.voff[ul] : -1;
-    // value and column pointers of the row's first slot
-    const T* vsm = nullptr;
-    const int* csm = nullptr;
-    if (valid && voff >= 0) {
-        const int rel = base - __ldg(d.slice_ptr + 2 * (u0 + ul));   // slots of the unit before the row's slice
-        vsm = reinterpret_cast<const T*>(vmem + voff) + (size_t)rel * 9 + lane;
-        csm = reinterpret_cast<const int*>(vmem + voff + (size_t)S.slots[ul] * 9 * sizeof(T)) + rel + lane;
+    // chunks of A into tensor memory: lane = row, two consecutive columns of A a
+    // word; a warp reaches the 32 lanes of its number mod 4
+    if (has_cu) {
+        const uint32_t lane0 = (uint32_t)((warp & 3) * 32) << 16;
+        const int arow = (warp & 3) * 32 + lane;
+        int i = 0;
+        for (int cu = rank; cu < n_cu; cu += G)
+            for (int c = 0, nch = chunks_of(cu); c < nch && i < n_tm; ++c, ++i) {
+                const unsigned char* src = chunk_ptr(cu, c) + (arow >> 3) * 256 + (arow & 7) * 16;
+#pragma unroll 4
+                for (int k = warp >> 2; k < kTcSteps; k += kThreads / 128) {
+                    const uint4 x = __ldg(reinterpret_cast<const uint4*>(src + k * kFuStepA));
+                    const uint4 y = __ldg(reinterpret_cast<const uint4*>(src + k * kFuStepA + 128));
+                    tmem_st8(tmem + lane0 + kResTmemD + i * kResTmemChunk + 8 * k, x, y);
+                }
+            }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        tc_fence_before();
     }
+    const int voff = ul < kResUnits ? S.voff[ul] : -1;
+    // the row's first slot in the value area (bytes), if its unit is there
+    const bool in_smem = valid && voff >= 0;
+    int v_at = 0, c_at = 0;
+    if (in_smem) {
+        const int rel = base - __ldg(d.slice_ptr + 2 * (u0 + ul));   // slots of the unit before the row's slice
+        v_at = voff + (rel * 9 + lane) * (int)sizeof(T);
+        c_at = voff + S.slots[ul] * 9 * (int)sizeof(T) + (rel + lane) * 4;
+    }
+    const T* vg = d.val + (size_t)base * 9 + lane;
+    const int* cg = d.col + base + lane;
     if (!mbar_wait(&S.vals, 0)) S.fail = 1;
     const bool landed = !__syncthreads_or(S.fail);
 
+    int c0[NB];   // the first slots' column ids
+    load_cols(in_smem ? reinterpret_cast<const int*>(vmem + c_at) : cg, 0, landed ? w : 0, c0);
+
     unsigned bar_n = 0;
     uint32_t done_ph = 0;
-    // every write of the group's CTAs before it is visible to their reads after it
-    auto barrier = [&]() {
+    // every write of the group's CTAs before arrive() is visible to their reads after wait()
+    auto arrive = [&]() {
         if (CLUSTER) {
             __syncwarp();
-            asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
             return;
         }
         __syncthreads();
         ++bar_n;
+        if (t == 0) red_release(job.bar);
+    };
+    auto wait = [&]() {
+        if (CLUSTER) {
+            __syncwarp();
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+            return;
+        }
         if (t == 0) {
-            __threadfence();
-            red_release(job.bar);
             const unsigned target = bar_n * (unsigned)G;
             const uint64_t ts = global_ns();
             while (ld_acquire(job.bar) < target)
@@ -296,7 +380,6 @@ __global__ void __launch_bounds__(kResThreads, 1)
                     S.fail = 1;
                     break;
                 }
-            __threadfence();
         }
         __syncthreads();
     };
@@ -306,10 +389,11 @@ __global__ void __launch_bounds__(kResThreads, 1)
         T u[3] = {zb[0], zb[1], zb[2]};
         if (coarse) {
             // ---- coarse product: this CTA's units
+            int a_at = 0;   // chunks issued this iteration (thread 0)
             for (int cu = rank; cu < n_cu; cu += G) {
                 const int rb = cu / nq, q = cu % nq, c_lo = q * c_per, nch = chunks_of(cu);
                 // B: r_c of the part's columns as three BF16 rows, eight columns (one core-matrix row) a thread
-                for (int g = t; g < nch * (kTcKC / 8); g += kResThreads) {
+                for (int g = t; g < nch * (kTcKC / 8); g += kThreads) {
                     const int k = c_lo * kTcKC + 8 * g;
                     float v[8];
                     if (ashift == 0) {
@@ -361,22 +445,32 @@ __global__ void __launch_bounds__(kResThreads, 1)
                 if (t == 0) {
                     constexpr uint32_t idesc = umma_idesc_bf16(kTcM, 16);
                     const uint32_t a_base = smem_u32(smem), b_base = smem_u32(bmem);
-                    const bool keep = n_a <= sh.stages;   // every chunk stays in its stage
-                    for (int c = 0; c < nch; ++c, ++used) {
-                        const int s = (int)((keep ? used % n_a : used) % sh.stages);
+                    tc_fence_after();
+                    for (int c = 0; c < nch; ++c, ++a_at) {
+                        const uint32_t b0 = b_base + c * kResChunkB;
+                        if (a_at < n_tm) {
+                            const uint32_t ta = tmem + kResTmemD + a_at * kResTmemChunk;
+#pragma unroll
+                            for (int k = 0; k < kTcSteps; ++k)
+                                umma_bf16_ta(tmem, ta + 8 * k, umma_desc(b0 + k * kResStepB, 128, 256), idesc,
+                                             (c > 0 || k > 0) ? 1u : 0u);
+                            continue;
+                        }
+                        const int s = (int)((keep ? a_at - n_tm : used) % sh.stages);
                         if (!mbar_wait(&S.full[s], keep ? 0u : (uint32_t)(used / sh.stages) & 1u)) {
                             S.fail = 1;
                             break;
                         }
                         tc_fence_after();
-                        const uint32_t a0 = a_base + s * kFuChunkA, b0 = b_base + c * kResChunkB;
+                        const uint32_t a0 = a_base + s * kFuChunkA;
+#pragma unroll
                         for (int k = 0; k < kTcSteps; ++k)
                             umma_bf16(tmem, umma_desc(a0 + k * kFuStepA, 128, 256),
                                       umma_desc(b0 + k * kResStepB, 128, 256), idesc, (c > 0 || k > 0) ? 1u : 0u);
                         if (keep) continue;
                         umma_commit(&S.empty[s]);
                         // refill the stage before this one, whose products were issued a chunk ago
-                        if (used > 0 && loaded < used + sh.stages) {
+                        if (loaded < used + sh.stages) {
                             const long long prev = loaded - sh.stages;
                             if (!mbar_wait(&S.empty[prev % sh.stages], (uint32_t)(prev / sh.stages) & 1u)) {
                                 S.fail = 1;
@@ -384,6 +478,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
                             }
                             load_next();
                         }
+                        ++used;
                     }
                     umma_commit(&S.done);
                 }
@@ -402,7 +497,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
                 if (S.fail) break;
             }
             // the last chunk's stage, for the next iteration
-            if (t == 0 && has_cu && n_a > sh.stages && !S.fail)
+            if (t == 0 && !keep && !S.fail)
                 while (loaded < used + sh.stages) {
                     const long long prev = loaded - sh.stages;
                     if (!mbar_wait(&S.empty[prev % sh.stages], (uint32_t)(prev / sh.stages) & 1u)) {
@@ -411,7 +506,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
                     }
                     load_next();
                 }
-            barrier();
+            arrive();
+            wait();
             if (S.fail) break;
             // ---- u = zb + Q_a P_i e_a, the parts of e_a added in part order
             float ev = 0.f;
@@ -437,92 +533,138 @@ __global__ void __launch_bounds__(kResThreads, 1)
             }
         }
         if (valid) st4(d.nb + 4 * (size_t)row, u[0], u[1], u[2]);
-        barrier();
-        if (S.fail) break;
-        // ---- w = K u and the three inner products
-        T a0 = 0, a1 = 0, a2 = 0;
-        if (vsm) row_product<T, sizeof(T) == 4 ? 8 : 4, true>(csm, vsm, w, d.nb, a0, a1, a2);
-        else if (valid)
-            row_product<T, sizeof(T) == 4 ? 4 : 2, false>(d.col + base + lane, d.val + (size_t)base * 9 + lane, w, d.nb,
-                                                          a0, a1, a2);
+        arrive();
         if (!valid) u[0] = u[1] = u[2] = 0;
+        const Partial<T> d0 = dot3_partial(r[0], r[1], r[2], u[0], u[1], u[2]);
+        const Partial<T> d2 = dot3_partial(r[0], r[1], r[2], r[0], r[1], r[2]);
+        wait();
+        if (S.fail) break;
+        // ---- w = K u
+        T a0 = 0, a1 = 0, a2 = 0;
         {
-            const double v1 = warp_sum_partial(dot3_partial(a0, a1, a2, u[0], u[1], u[2]));
-            const double v0 = warp_sum_partial(dot3_partial(r[0], r[1], r[2], u[0], u[1], u[2]));
-            const double v2 = warp_sum_partial(dot3_partial(r[0], r[1], r[2], r[0], r[1], r[2]));
-            if (lane == 0) {
-                S.wsum[warp][0] = v0;
-                S.wsum[warp][1] = v1;
-                S.wsum[warp][2] = v2;
+            T q[NB][3];
+            gather<T, NB>(d.nb, c0, q);
+            if (in_smem) {
+                products<T, NB>(reinterpret_cast<const T*>(vmem + v_at), c0, q, a0, a1, a2);
+                for (int k = NB; k < w; k += NB) {
+                    int c[NB];
+                    load_cols(reinterpret_cast<const int*>(vmem + c_at), k, w, c);
+                    gather<T, NB>(d.nb, c, q);
+                    products<T, NB>(reinterpret_cast<const T*>(vmem + v_at) + 288 * k, c, q, a0, a1, a2);
+                }
+            } else {
+                products<T, NB>(vg, c0, q, a0, a1, a2);
+                for (int k = NB; k < w; k += NB) {
+                    int c[NB];
+                    load_cols(cg, k, w, c);
+                    gather<T, NB>(d.nb, c, q);
+                    products<T, NB>(vg + 288 * (size_t)k, c, q, a0, a1, a2);
+                }
+            }
+        }
+        {
+            const double v = warp_sums3(d0, dot3_wu(a0, a1, a2, u[0], u[1], u[2]), d2);
+            if (lane < 3) S.wsum[warp][lane] = v;
+        }
+        __syncthreads();
+        // partials: FP64 one per warp (32 rows), which the totals add in the
+        // streamed kernel's order; FP32 one per warp in a cluster and one per CTA of a larger group (FP64 sums of float-float
+        // warp sums: their order shows in the last bits of alpha and beta only,
+        // which are rounded to FP32).  An FP64 instruction takes a scheduler 64
+        // cycles, so few warps do few of them, a value each.
+        if (sizeof(T) == 8 || CLUSTER) {
+            if (t < 6 * nu && 32 * (2 * u0 + t / 3) < n) d.part[4 * (size_t)(2 * u0 + t / 3) + t % 3] = S.wsum[t / 3][t % 3];
+        } else if (warp < 3) {
+            double x = lane < 2 * U ? S.wsum[lane & 15][warp] : 0.0;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if (lane == 0) d.part[4 * (size_t)rank + warp] = x;
+        }
+        arrive();
+        wait();
+        if (S.fail) break;
+        double tot[3] = {0.0, 0.0, 0.0};   // valid in thread 0
+        if (sizeof(T) == 8) {
+            const int nw = sh.rtile / 32, n_tiles = (n + sh.rtile - 1) / sh.rtile, n_warps = (n + 31) / 32;
+            for (int x = t; t < sh.rtile && x < n_tiles; x += sh.rtile)
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    double v[8];
+#pragma unroll
+                    for (int y = 0; y < 8; ++y)
+                        v[y] = y < nw && x * nw + y < n_warps ? d.part[4 * (size_t)(x * nw + y) + i] : 0.0;
+                    tot[i] += ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+                }
+            if (warp < nw) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) tot[i] += __shfl_xor_sync(0xffffffffu, tot[i], o);
+                if (lane == 0)
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) S.wsum[warp][i] = tot[i];
+            }
+            __syncthreads();
+            if (warp == 0) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) tot[i] = lane < nw ? S.wsum[lane & 7][i] : 0.0;
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) tot[i] += __shfl_xor_sync(0xffffffffu, tot[i], o);
+            }
+        } else {
+            if (warp < 3) {   // warp i sums value i
+                const int n_part = CLUSTER ? (n + 31) / 32 : G;   // at most 256
+                double x[8], s = 0.0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j)   // every load first
+                    x[j] = lane + 32 * j < n_part ? d.part[4 * (size_t)(lane + 32 * j) + warp] : 0.0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (32 * j < n_part) s += x[j];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (lane == 0) S.wsum[0][warp] = s;
+            }
+            __syncthreads();
+            if (t == 0)
+#pragma unroll
+                for (int i = 0; i < 3; ++i) tot[i] = S.wsum[0][i];
+        }
+        if (t == 0) {
+            ResState& q = S.st;
+            const double gamma = tot[0], delta = tot[1];
+            q.rr = tot[2];
+            if (!(tot[2] > q.tol2 * q.rr0)) {
+                q.state = kConverged;
+            } else if (q.iter >= q.maxit) {
+                q.state = kMaxIter;
+            } else {
+                double beta = 0.0, den = delta;
+                if (!q.first) {
+                    if (sizeof(T) == 8) {
+                        beta = gamma / q.rho;
+                        den = delta - beta * gamma / q.alpha;
+                    } else {
+                        beta = gamma * q.inv_rho;
+                        den = delta - beta * gamma * q.inv_alpha;
+                    }
+                }
+                if (gamma > 0.0 && den > 0.0 && isfinite(gamma) && isfinite(den)) {
+                    q.alpha = gamma / den;
+                    q.beta = beta;
+                    q.rho = gamma;
+                    q.first = 0;
+                    q.iter = q.iter + 1;
+                } else {
+                    q.alpha = 0.0;
+                    q.beta = 0.0;
+                    q.state = kConverged;
+                }
             }
         }
         __syncthreads();
-        {   // a tile's warps in the order of the streamed kernel's block sum
-            const int nt = t1 - t0, nw = sh.rtile / 32;
-            if (t < 3 * nt) {
-                const int tl = t / 3, i = t - 3 * tl;
-                double v[8];
-#pragma unroll
-                for (int x = 0; x < 8; ++x) v[x] = x < nw ? S.wsum[(tl * nw + x) & (kResThreads / 32 - 1)][i] : 0.0;
-                d.part[4 * (size_t)(t0 + tl) + i] =
-                    ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
-            }
-        }
-        barrier();
-        if (S.fail) break;
-        {   // totals: FP64 in the streamed kernel's order (rtile threads), FP32 by every thread
-            const int nthr = sizeof(T) == 8 ? sh.rtile : kResThreads;
-            double acc[3] = {0.0, 0.0, 0.0};
-            if (t < nthr)
-                for (int x = t; x < n_tiles; x += nthr)
-#pragma unroll
-                    for (int i = 0; i < 3; ++i) acc[i] += d.part[4 * (size_t)x + i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                for (int i = 0; i < 3; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
-            if (lane == 0)
-#pragma unroll
-                for (int i = 0; i < 3; ++i) S.wsum[warp][i] = acc[i];
-            __syncthreads();
-            if (warp == 0) {
-                const int nw = nthr / 32;
-#pragma unroll
-                for (int i = 0; i < 3; ++i) acc[i] = lane < nw ? S.wsum[lane & (kResThreads / 32 - 1)][i] : 0.0;
-#pragma unroll
-                for (int o = 8; o > 0; o >>= 1)
-#pragma unroll
-                    for (int i = 0; i < 3; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
-                if (lane == 0) {
-                    ResState& q = S.st;
-                    const double gamma = acc[0], delta = acc[1];
-                    q.rr = acc[2];
-                    if (!(acc[2] > q.tol2 * q.rr0)) {
-                        q.state = kConverged;
-                    } else if (q.iter >= q.maxit) {
-                        q.state = kMaxIter;
-                    } else {
-                        double beta = 0.0, den = delta;
-                        if (!q.first) {
-                            beta = gamma / q.rho;
-                            den = delta - beta * gamma / q.alpha;
-                        }
-                        if (gamma > 0.0 && den > 0.0 && isfinite(gamma) && isfinite(den)) {
-                            q.alpha = gamma / den;
-                            q.beta = beta;
-                            q.rho = gamma;
-                            q.first = 0;
-                            q.iter = q.iter + 1;
-                        } else {
-                            q.alpha = 0.0;
-                            q.beta = 0.0;
-                            q.state = kConverged;
-                        }
-                    }
-                }
-            }
-            __syncthreads();
-        }
         if (S.st.state != kActive) {
             active = false;
             break;
@@ -566,7 +708,14 @@ __global__ void __launch_bounds__(kResThreads, 1)
                 const int x = t / 6, c = t - 6 * x;
                 d.rcp[6 * (size_t)(u0 + x) + c] = S.ws[2 * x][c] + S.ws[2 * x + 1][c];
             }
-            barrier();
+            arrive();
+        }
+        if (sizeof(T) == 4 && t == kThreads - 32) {
+            S.st.inv_rho = 1.0 / S.st.rho;
+            S.st.inv_alpha = 1.0 / S.st.alpha;
+        }
+        if (coarse) {
+            wait();
             if (S.fail) break;
         }
     }
@@ -596,9 +745,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
             sc->state = S.st.state;
         }
         // copies in flight land before the memory is released
-        const bool keep = n_a <= sh.stages;
         if (keep) {
-            for (int i = 0; i < n_a; ++i) mbar_wait(&S.full[i], 0);
+            for (int i = 0; i < n_ring; ++i) mbar_wait(&S.full[i], 0);
         } else {
             for (long long i = used; i < loaded; ++i)
                 mbar_wait(&S.full[i % sh.stages], (uint32_t)(i / sh.stages) & 1u);
@@ -606,19 +754,19 @@ __global__ void __launch_bounds__(kResThreads, 1)
     }
     __syncthreads();
     if (has_cu && warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kResTmemCols)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tm_cols)
                      : "memory");
 }
 
-template <typename T, bool CLUSTER>
-cudaError_t res_attr(int smem) {
-    cudaError_t e = cudaFuncSetAttribute(k_pcg_resident<T, CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+template <typename T, bool CLUSTER, int U>
+cudaError_t res_attr() {
+    cudaError_t e =
+        cudaFuncSetAttribute(k_pcg_resident<T, CLUSTER, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, res_smem_max());
     if (e == cudaSuccess && CLUSTER)
-        e = cudaFuncSetAttribute(k_pcg_resident<T, CLUSTER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        e = cudaFuncSetAttribute(k_pcg_resident<T, CLUSTER, U>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
 
-template <typename T>
 void res_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, const ResShape& sh, cudaStream_t s) {
     cfg = cudaLaunchConfig_t{};
     if (sh.cluster > 0) {
@@ -631,7 +779,7 @@ void res_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, const ResSha
         attr[0].val.cooperative = 1;
     }
     cfg.gridDim = dim3(sh.grid);
-    cfg.blockDim = dim3(kResThreads);
+    cfg.blockDim = dim3(kCoarseRows * sh.units);
     cfg.dynamicSmemBytes = sh.smem;
     cfg.stream = s;
     cfg.attrs = attr;
@@ -640,6 +788,7 @@ void res_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, const ResSha
 
 }  // namespace
 
+int res_tmem_chunks() { return kResTmemChunks; }
 int res_smem_max() { return 227 * 1024 - kResStatic; }
 int res_smem_coarse(int stages, int b_chunks) { return stages * kFuChunkA + b_chunks * kResChunkB; }
 int res_part_chunks(int N) { return coarse_part_chunks(N); }
@@ -652,24 +801,30 @@ cudaError_t res_init(ResLimits& lim) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim.sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = res_attr<float, true>(res_smem_max());
-    if (e == cudaSuccess) e = res_attr<float, false>(res_smem_max());
-    if (e == cudaSuccess) e = res_attr<double, true>(res_smem_max());
-    if (e == cudaSuccess) e = res_attr<double, false>(res_smem_max());
+#define MFEM_RES_ATTR(T, U)                                   \
+    if (e == cudaSuccess) e = res_attr<T, true, U>();         \
+    if (e == cudaSuccess) e = res_attr<T, false, U>();
+    MFEM_RES_ATTR(float, 4)
+    MFEM_RES_ATTR(float, 6)
+    MFEM_RES_ATTR(float, 8)
+    MFEM_RES_ATTR(double, 4)
+    MFEM_RES_ATTR(double, 6)
+    MFEM_RES_ATTR(double, 8)
+#undef MFEM_RES_ATTR
     if (e != cudaSuccess) return e;
     for (int i = 0, c = 1; i < kResClusterSizes; ++i, c *= 2) {   // clusters of 1, 2, 4, 8, 16 CTAs resident at once
         ResShape sh{};
         sh.grid = c;
         sh.cluster = c;
+        sh.units = kResUnits;
         sh.smem = res_smem_max();
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr[1];
-        res_config<double>(cfg, attr, sh, nullptr);
-        int nf = 0, nd = 0;
-        if (cudaOccupancyMaxActiveClusters(&nf, k_pcg_resident<float, true>, &cfg) != cudaSuccess) nf = 0;
-        if (cudaOccupancyMaxActiveClusters(&nd, k_pcg_resident<double, true>, &cfg) != cudaSuccess) nd = 0;
+        res_config(cfg, attr, sh, nullptr);
+        int nc = 0;   // one CTA an SM in every variant (shared memory)
+        if (cudaOccupancyMaxActiveClusters(&nc, k_pcg_resident<double, true, kResUnits>, &cfg) != cudaSuccess) nc = 0;
         cudaGetLastError();
-        lim.clusters[i] = nf < nd ? nf : nd;
+        lim.clusters[i] = nc;
     }
     return cudaSuccess;
 }
@@ -679,9 +834,16 @@ cudaError_t launch_pcg_resident(const PcgDesc<T>* descs, const ResJob* jobs, int
                                 cudaStream_t s) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    res_config<T>(cfg, attr, sh, s);
-    if (sh.cluster > 0) return cudaLaunchKernelEx(&cfg, k_pcg_resident<T, true>, descs, jobs, n_probs, sh);
-    return cudaLaunchKernelEx(&cfg, k_pcg_resident<T, false>, descs, jobs, n_probs, sh);
+    res_config(cfg, attr, sh, s);
+#define MFEM_RES_CASE(UN)                                                                                           \
+    if (sh.units == UN)                                                                                             \
+        return sh.cluster > 0 ? cudaLaunchKernelEx(&cfg, k_pcg_resident<T, true, UN>, descs, jobs, n_probs, sh)     \
+                              : cudaLaunchKernelEx(&cfg, k_pcg_resident<T, false, UN>, descs, jobs, n_probs, sh);
+    MFEM_RES_CASE(4)
+    MFEM_RES_CASE(6)
+    MFEM_RES_CASE(8)
+#undef MFEM_RES_CASE
+    return cudaErrorInvalidValue;
 }
 
 template cudaError_t launch_pcg_resident<float>(const PcgDesc<float>*, const ResJob*, int, const ResShape&, cudaStream_t);

@@ -174,7 +174,6 @@ bool pcg_tile_supported(int tile_rows);
 // PCG of problems that fit the chip (k_pcg_resident.cu): problem i of the
 // descriptor table runs on CTAs cta0 .. cta0 + ncta - 1 of one launch.
 constexpr int kResUnits = 8;                   // units of 64 rows a CTA may own
-constexpr int kResThreads = 64 * kResUnits;    // one thread per row
 constexpr int kResClusterSizes = 5;            // cluster sizes 1, 2, 4, 8, 16
 struct ResJob {
     int cta0, ncta;
@@ -184,7 +183,8 @@ struct ResJob {
 };
 struct ResShape {
     int grid, cluster;   // CTAs; CTAs per cluster (every group's size), 0: cooperative launch
-    int rtile;           // rows per reduction tile: a CTA owns whole tiles
+    int units;           // most units a CTA owns: 4, 6 or 8 (the kernel's variant)
+    int rtile;           // FP64: rows per tile of the streamed kernel's reduction
     int iters;           // most iterations of this launch
     int stages, b_chunks, v_bytes, smem;   // shared memory: A ring, B chunks, matrix values, all
 };
@@ -194,6 +194,7 @@ struct ResLimits {
 };
 cudaError_t res_init(ResLimits& lim);   // kernel attributes and limits of the current device
 int res_smem_max();
+int res_tmem_chunks();   // chunks of A_c^{-1} a CTA keeps in tensor memory
 int res_smem_coarse(int stages, int b_chunks);
 int res_part_chunks(int N);    // chunks of the K range a coarse unit takes (b_chunks)
 int res_coarse_units(int N);   // coarse units of one product

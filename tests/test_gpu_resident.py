@@ -1,0 +1,63 @@
+"""The resident PCG kernel (problems that fit the chip: one launch runs a whole
+solve) against the streamed kernels: a pose alone takes the first, the same pose
+in a batch too large for the chip the second, and both do the same arithmetic in
+the same order, so positions and iteration counts are equal bit for bit.  Sizes:
+one to many 64-row units a CTA, ragged last units, clusters and the cooperative
+launch, both precisions (FP64: every reduction tile), with and without the coarse
+space, aggregates of several units."""
+import numpy as np
+import pytest
+
+from synth import bar_twist_config, figure_config
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # config, batch that does not fit, options
+    ("bar", 160, dict(precision="mixed")),
+    ("bar", 160, dict(precision="fp64", tile_rows=64)),
+    ("bar", 160, dict(precision="fp64", tile_rows=128)),
+    ("bar", 160, dict(precision="mixed", precond="block_jacobi")),
+    ("fig3000", 80, dict(precision="mixed", coarse_agg=256)),
+    ("fig3000", 80, dict(precision="fp64", tile_rows=256)),
+    ("fig10000", 32, dict(precision="mixed", constraint="penalty", k_s=1e5)),
+    ("fig50000", 8, dict(precision="mixed")),
+    ("fig50000", 8, dict(precision="mixed", precond="block_jacobi", coarse_agg=0)),
+    ("fig50000", 8, dict(precision="fp64", tile_rows=128, coarse_agg=128)),
+]
+
+
+def config(name):
+    if name == "bar":
+        return bar_twist_config()
+    return figure_config(int(name[3:]), model="snh" if name != "fig10000" else "corot", seeds=[3, 4])
+
+
+@pytest.mark.parametrize("name,many,opts", CASES)
+def test_resident_equals_streamed(name, many, opts):
+    from paper_2408_04066_gb300 import mfem
+    cfg = config(name)
+    xf = np.asarray(cfg["xfs"])
+    opts = dict(dict(tile_rows=128, spmv_split=1, newton_max=6), **opts)
+    ctx = mfem.Context.from_config(cfg, max_batch=many, **opts)
+    alone = [ctx.solve_batch(xf[i:i + 1]) for i in range(len(xf))]
+    p = ctx.profile()
+    assert p["kernel_launches"] < p["pcg_launches"]          # one launch a solve
+    out, stats = ctx.solve_batch(np.concatenate([xf] * (many // len(xf))))
+    p = ctx.profile()
+    assert p["kernel_launches"] > p["pcg_launches"]          # launches per iteration
+    for b in range(len(out)):
+        x, st = alone[b % len(xf)]
+        assert np.array_equal(out[b], x[0])
+        assert stats[b]["pcg_iters"] == st[0]["pcg_iters"] and stats[b]["newton_iters"] == st[0]["newton_iters"]
+    ctx.close()
+
+
+def test_iteration_cap():
+    """A solve cut off by cg_max stops after exactly that many iterations a Newton step."""
+    from paper_2408_04066_gb300 import mfem
+    cfg = config("fig3000")
+    ctx = mfem.Context.from_config(cfg, spmv_split=1, tile_rows=64, cg_max=3, newton_max=2, newton_tol=0.0, cg_tol=0.0)
+    _, st = ctx.solve_batch(np.asarray(cfg["xfs"])[:1])
+    assert st[0]["newton_iters"] == 2 and st[0]["pcg_iters"] == 6
+    ctx.close()
