@@ -181,81 +181,18 @@ __device__ __forceinline__ int unit_problem(const PcgDesc<T>* __restrict__ D, in
     return lo;
 }
 
-// Full occupancy (2048 threads per SM) matters more than registers in the FP32
-// kernel: it is latency-bound on its dependent col -> neighbour loads.  The
-// FP64 kernel is bound by the FP64 pipe and takes half that occupancy for the
-// registers its double accumulators need (no spills).
-//
-// SPLIT = threads per row.  SPLIT = 1: lane l of a warp takes row l of its
-// 32-row slice and walks all the row's slots.  SPLIT = 2: a warp takes 16 rows
-// of a slice, lanes l and l + 16 the even and odd slots of row l (each warp
-// load still covers whole 32-byte sectors: 16 lanes read 64 consecutive
-// bytes), so each thread's dependent chain is half as long; the two halves
-// are added with one shuffle.  The autotuner picks the tile and SPLIT.
-template <typename T, int TILE, int SPLIT>
-__global__ void __launch_bounds__(TILE * SPLIT, (sizeof(T) == 4 ? 2048 : 1024) / (TILE * SPLIT))
-    k_pcg_spmv(const PcgDesc<T>* __restrict__ D, int n_probs) {
-    // prologue on data no kernel of the iteration writes (the descriptor table
-    // and the matrix structure), overlapping the previous kernel's drain
-    const int u = blockIdx.x;
-    const PcgDesc<T>& d = D[unit_problem(D, n_probs, u)];
-    ProbScal* sc = d.sc;
-    const int tile = u - d.unit_begin;
+// The end of an SpMV block of NT threads: tile partials (v: the warp's sums, value
+// i in lane i) and, in the problem's last block, the totals, the convergence test
+// and the next step's coefficients.
+template <typename T, int NT>
+__device__ __forceinline__ void spmv_commit(const PcgDesc<T>& d, ProbScal* sc, int tile, double v) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // row of this thread and its first slot (parity) within the row
-    const int half = SPLIT == 2 ? (lane >> 4) : 0;
-    const int rs = SPLIT == 2 ? ((warp & 1) << 4) + (lane & 15) : lane;   // row within the slice
-    const int row = tile * TILE + (SPLIT == 2 ? (warp >> 1) * 32 : warp * 32) + rs;
-    const bool valid = row < d.n_rows;
-    int base = 0, w = 0;
-    if (valid) {
-        const int s = row >> 5;
-        base = __ldg(d.slice_ptr + s);
-        w = (__ldg(d.slice_ptr + s + 1) - base) >> 5;
-    }
-    pdl_wait();
-    pdl_trigger();
-    if (sc->state != kActive) return;
-    T a0 = 0, a1 = 0, a2 = 0;
-#pragma unroll 4
-    for (int k = half; k < w; k += SPLIT) {
-        const int g = base + (k << 5);
-        const int c = __ldcs(d.col + g + rs);
-        if (c >= 0) {
-            const T* vv = d.val + (size_t)g * 9 + rs;
-            T q[3];
-            ld4(d.nb + 4 * (size_t)c, q);
-            a0 += __ldcs(vv) * q[0] + __ldcs(vv + 32) * q[1] + __ldcs(vv + 64) * q[2];
-            a1 += __ldcs(vv + 96) * q[0] + __ldcs(vv + 128) * q[1] + __ldcs(vv + 160) * q[2];
-            a2 += __ldcs(vv + 192) * q[0] + __ldcs(vv + 224) * q[1] + __ldcs(vv + 256) * q[2];
-        }
-    }
-    if (SPLIT == 2) {   // the odd slots' half (lanes 16-31) into the even half
-        a0 += __shfl_xor_sync(0xffffffffu, a0, 16);
-        a1 += __shfl_xor_sync(0xffffffffu, a1, 16);
-        a2 += __shfl_xor_sync(0xffffffffu, a2, 16);
-    }
-    // epilogue at uniform control flow; rows past the end and the second half of
-    // a split row add zeros
-    const bool owner = valid && half == 0;
-    if (!owner) a0 = a1 = a2 = 0;
-    T ur[3] = {0, 0, 0};
-    const size_t np = npad32(d.n_rows);
-    if (owner) {
-        ld4(d.nb + 4 * (size_t)row, ur);
-        st4(rec_field(d.rec, np, kRecW, row), a0, a1, a2);
-    }
-    T r[3] = {0, 0, 0};
-    if (owner) ld4(rec_field(d.rec, np, kRecR, row), r);
-    const double v = warp_sums3(dot3_partial(r[0], r[1], r[2], ur[0], ur[1], ur[2]),
-                                dot3_wu(a0, a1, a2, ur[0], ur[1], ur[2]),
-                                dot3_partial(r[0], r[1], r[2], r[0], r[1], r[2]));   // value i in lane i
     // tile partials and, in the problem's last block, the totals: the sums over
     // the block's warps by three threads, a value each.  An FP64 instruction takes
     // a scheduler 64 cycles, and a shuffle tree over the block's warps spends five
     // levels of them on lanes that hold nothing (200k figure, 16 poses, 128-row
     // tiles: 117.8 -> 114.0 us an iteration, 800k figure, 4 poses: 90.5 -> 87.1)
-    constexpr int NW = TILE * SPLIT / 32;
+    constexpr int NW = NT / 32;
     __shared__ double sm[NW * 3];
     __shared__ int s_last;
     if (lane < 3) sm[3 * warp + lane] = v;
@@ -272,7 +209,7 @@ __global__ void __launch_bounds__(TILE * SPLIT, (sizeof(T) == 4 ? 2048 : 1024) /
     if (!s_last) return;
     __threadfence();
     double acc[3] = {0.0, 0.0, 0.0};
-    for (int x = threadIdx.x; x < d.n_tiles; x += TILE * SPLIT)
+    for (int x = threadIdx.x; x < d.n_tiles; x += NT)
 #pragma unroll
         for (int i = 0; i < 3; ++i) acc[i] += *(volatile double*)&d.part[4 * x + i];
     const double tv = warp_sums3(Partial<double>{acc[0]}, Partial<double>{acc[1]}, Partial<double>{acc[2]});
@@ -310,6 +247,163 @@ __global__ void __launch_bounds__(TILE * SPLIT, (sizeof(T) == 4 ? 2048 : 1024) /
             sc->beta_f = (float)sc->beta;
         }
     }
+}
+
+// The SpMV with two threads per row (the options' or the autotuner's choice): a
+// warp takes 16 rows of a slice, lanes l and l + 16 the even and odd slots of row
+// l (each warp load still covers whole 32-byte sectors: 16 lanes read 64
+// consecutive bytes), so each thread's dependent chain is half as long; the two
+// halves are added with one shuffle.
+template <typename T, int TILE>
+__global__ void __launch_bounds__(TILE * 2, (sizeof(T) == 4 ? 1024 : 512) / TILE)
+    k_pcg_spmv_split(const PcgDesc<T>* __restrict__ D, int n_probs) {
+    // prologue on data no kernel of the iteration writes (the descriptor table
+    // and the matrix structure), overlapping the previous kernel's drain
+    const int u = blockIdx.x;
+    const PcgDesc<T>& d = D[unit_problem(D, n_probs, u)];
+    ProbScal* sc = d.sc;
+    const int tile = u - d.unit_begin;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int half = lane >> 4;                          // parity of this thread's slots
+    const int rs = ((warp & 1) << 4) + (lane & 15);      // row within the slice
+    const int row = tile * TILE + (warp >> 1) * 32 + rs;
+    const bool valid = row < d.n_rows;
+    int base = 0, w = 0;
+    if (valid) {
+        const int s = row >> 5;
+        base = __ldg(d.slice_ptr + s);
+        w = (__ldg(d.slice_ptr + s + 1) - base) >> 5;
+    }
+    pdl_wait();
+    pdl_trigger();
+    if (sc->state != kActive) return;
+    T a0 = 0, a1 = 0, a2 = 0;
+#pragma unroll 4
+    for (int k = half; k < w; k += 2) {
+        const int g = base + (k << 5);
+        const int c = __ldcs(d.col + g + rs);
+        if (c >= 0) {
+            const T* vv = d.val + (size_t)g * 9 + rs;
+            T q[3];
+            ld4(d.nb + 4 * (size_t)c, q);
+            a0 += __ldcs(vv) * q[0] + __ldcs(vv + 32) * q[1] + __ldcs(vv + 64) * q[2];
+            a1 += __ldcs(vv + 96) * q[0] + __ldcs(vv + 128) * q[1] + __ldcs(vv + 160) * q[2];
+            a2 += __ldcs(vv + 192) * q[0] + __ldcs(vv + 224) * q[1] + __ldcs(vv + 256) * q[2];
+        }
+    }
+    // the odd slots' half (lanes 16-31) into the even half
+    a0 += __shfl_xor_sync(0xffffffffu, a0, 16);
+    a1 += __shfl_xor_sync(0xffffffffu, a1, 16);
+    a2 += __shfl_xor_sync(0xffffffffu, a2, 16);
+    // epilogue at uniform control flow; rows past the end and the second half of
+    // a split row add zeros
+    const bool owner = valid && half == 0;
+    if (!owner) a0 = a1 = a2 = 0;
+    T ur[3] = {0, 0, 0};
+    const size_t np = npad32(d.n_rows);
+    if (owner) {
+        ld4(d.nb + 4 * (size_t)row, ur);
+        st4(rec_field(d.rec, np, kRecW, row), a0, a1, a2);
+    }
+    T r[3] = {0, 0, 0};
+    if (owner) ld4(rec_field(d.rec, np, kRecR, row), r);
+    const double v = warp_sums3(dot3_partial(r[0], r[1], r[2], ur[0], ur[1], ur[2]),
+                                dot3_wu(a0, a1, a2, ur[0], ur[1], ur[2]),
+                                dot3_partial(r[0], r[1], r[2], r[0], r[1], r[2]));   // value i in lane i
+    spmv_commit<T, TILE * 2>(d, sc, tile, v);
+}
+
+// The SpMV with one thread per row: the row's first kRowCols column ids are
+// loaded before the programmatic-launch wait (no kernel of the iteration writes
+// them), so that the dependent chain after it is one load deep, and the slots are
+// taken NB at a time, every load of the NB first.
+//
+// What bounds it: the latency of the value stream and of the gathers while the
+// second, partial wave of blocks drains (16 poses of the 200k figure are 2.1 waves
+// at full occupancy), then DRAM.  Half the occupancy (64 registers a thread) and
+// two slots in flight measured best; us per launched iteration on the 200k figure
+// (16 SNH poses / 16 corot poses) and the 800k figure (4 poses), 128-row blocks:
+//   one slot at a time, ids loaded in the loop, 2048 threads an SM   81.3 / 114 / 87.5
+//   ids first, 1024 threads, NB 2                                    72.6 / 102 / 76.9
+//   1024, NB 3: 73.3 / 104 / 77.8    1024, NB 1: 76.0 / 107 / 79.3
+//   768, NB 4: 77.0 / 110 / 81.7     512, NB 8: 89.5 / 130 / 91.8
+//   1024, NB 2, the next neighbours prefetched: 74.5 / 106 / 78.5
+// Slices in shared memory by bulk copies were slower (80.6 / 116 / 88.9): the
+// gathers live off the L1 that the copies' buffers take.
+constexpr int kRowCols = 16;
+template <typename T>
+struct RowShape {
+    static constexpr int kOcc = 1024, kNB = 2;   // threads an SM, slots in flight
+};
+template <>
+struct RowShape<double> {   // 8 poses of the 200k figure: 124.1 -> 118.7 us (1024, NB 2: 128.8; 768, NB 1: 120.6)
+    static constexpr int kOcc = 512, kNB = 2;
+};
+template <typename T, int TILE>
+__global__ void __launch_bounds__(TILE, RowShape<T>::kOcc / TILE) k_pcg_spmv_row(const PcgDesc<T>* __restrict__ D, int n_probs) {
+    constexpr int NB = RowShape<T>::kNB;
+    const int u = blockIdx.x;
+    const PcgDesc<T>& d = D[unit_problem(D, n_probs, u)];
+    ProbScal* sc = d.sc;
+    const int tile = u - d.unit_begin;
+    const int lane = threadIdx.x & 31;
+    const int row = tile * TILE + threadIdx.x;
+    const bool valid = row < d.n_rows;
+    int base = 0, w = 0;
+    if (valid) {
+        const int s = row >> 5;
+        base = __ldg(d.slice_ptr + s);
+        w = (__ldg(d.slice_ptr + s + 1) - base) >> 5;
+    }
+    const int* cp = d.col + base + lane;
+    int c[kRowCols];
+#pragma unroll
+    for (int i = 0; i < kRowCols; ++i) c[i] = i < w ? __ldg(cp + 32 * i) : -1;
+    pdl_wait();
+    pdl_trigger();
+    if (sc->state != kActive) return;
+    const T* vp = d.val + (size_t)base * 9 + lane;
+    T a0 = 0, a1 = 0, a2 = 0;
+#pragma unroll
+    for (int k = 0; k < kRowCols; k += NB) {
+        T q[NB][3], m[NB][9];
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+            if (c[k + i] >= 0) {
+                ld4(d.nb + 4 * (size_t)c[k + i], q[i]);
+#pragma unroll
+                for (int e = 0; e < 9; ++e) m[i][e] = __ldcs(vp + 288 * (k + i) + 32 * e);
+            }
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+            if (c[k + i] >= 0) {
+                a0 += m[i][0] * q[i][0] + m[i][1] * q[i][1] + m[i][2] * q[i][2];
+                a1 += m[i][3] * q[i][0] + m[i][4] * q[i][1] + m[i][5] * q[i][2];
+                a2 += m[i][6] * q[i][0] + m[i][7] * q[i][1] + m[i][8] * q[i][2];
+            }
+    }
+    for (int k = kRowCols; k < w; ++k) {   // longer rows
+        const int cc = __ldg(cp + 32 * k);
+        if (cc >= 0) {
+            T q[3];
+            ld4(d.nb + 4 * (size_t)cc, q);
+            const T* vv = vp + 288 * (size_t)k;
+            a0 += __ldcs(vv) * q[0] + __ldcs(vv + 32) * q[1] + __ldcs(vv + 64) * q[2];
+            a1 += __ldcs(vv + 96) * q[0] + __ldcs(vv + 128) * q[1] + __ldcs(vv + 160) * q[2];
+            a2 += __ldcs(vv + 192) * q[0] + __ldcs(vv + 224) * q[1] + __ldcs(vv + 256) * q[2];
+        }
+    }
+    T ur[3] = {0, 0, 0}, r[3] = {0, 0, 0};
+    const size_t np = npad32(d.n_rows);
+    if (valid) {
+        ld4(d.nb + 4 * (size_t)row, ur);
+        ld4(rec_field(d.rec, np, kRecR, row), r);
+        st4(rec_field(d.rec, np, kRecW, row), a0, a1, a2);
+    }
+    const double v = warp_sums3(dot3_partial(r[0], r[1], r[2], ur[0], ur[1], ur[2]),
+                                dot3_wu(a0, a1, a2, ur[0], ur[1], ur[2]),
+                                dot3_partial(r[0], r[1], r[2], r[0], r[1], r[2]));
+    spmv_commit<T, TILE>(d, sc, tile, v);
 }
 
 template <typename T, int TILE>
@@ -612,7 +706,8 @@ cudaError_t launch_pcg_iters_t(const PcgDesc<T>* descs, int n_probs, int n_units
                 if (e != cudaSuccess) return e;
             }
         }
-        e = cudaLaunchKernelEx(&cfg_s, k_pcg_spmv<T, TILE, SPLIT>, descs, n_probs);
+        if constexpr (SPLIT == 1) e = cudaLaunchKernelEx(&cfg_s, k_pcg_spmv_row<T, TILE>, descs, n_probs);
+        else e = cudaLaunchKernelEx(&cfg_s, k_pcg_spmv_split<T, TILE>, descs, n_probs);
         if (e != cudaSuccess) return e;
         e = cudaLaunchKernelEx(&cfg_u, k_pcg_update<T, kRowTileU>, descs, n_probs);
         if (e != cudaSuccess) return e;
