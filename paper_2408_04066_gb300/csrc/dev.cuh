@@ -36,18 +36,31 @@ __host__ __device__ __forceinline__ int ke_offset(int a, int b) {   // a <= b
 // Per-problem PCG vector area, in elements of the PCG type, rows padded to 32
 // (np = npad32(n)): the neighbour record nb[np][4] = (u.xyz, 0) -- the
 // preconditioned residual, the one vector the SpMV gathers from neighbours (16
-// bytes in FP32) -- then six row fields of [np][4] each, field-major (a warp's
-// access to one field of 32 consecutive rows is one contiguous run): the Newton
-// increment dx, the residual r, the search direction p, s = K p, w = K u, and
-// the block-Jacobi part zb of u.  Field f (kRecDX .. kRecZB) of row i is at
-// rec + f * np + 4 i (rec_field).
-constexpr int kVecStride = 28;                 // times npad32(n)
+// bytes in FP32) -- then six row fields of three planes [np] each (component c of
+// 32 consecutive rows is one contiguous run; four-element rows moved a third more
+// bytes): the Newton increment dx, the residual r, the search direction p, s = K p,
+// w = K u, and the block-Jacobi part zb of u.  Component c of field f (kRecDX ..
+// kRecZB) of row i is at rec + (f + c) * np + i (ld3, st3).
+constexpr int kVecStride = 22;                 // times npad32(n)
 constexpr int kOffNB = 0, kOffRec = 4;
-constexpr int kRecDX = 0, kRecR = 4, kRecP = 8, kRecS = 12, kRecW = 16, kRecZB = 20;
+constexpr int kRecDX = 0, kRecR = 3, kRecP = 6, kRecS = 9, kRecW = 12, kRecZB = 15;
+// Block-Jacobi inverses are symmetric, bit for bit (the same cofactor products):
+// six planes, entries 00, 11, 22, 12, 02, 01.
+constexpr int kDinv = 6;
 __host__ __device__ __forceinline__ size_t npad32(int n) { return ((size_t)n + 31) & ~(size_t)31; }
 template <typename T>
-__host__ __device__ __forceinline__ T* rec_field(T* rec, size_t np, int f, size_t row) {
-    return rec + (size_t)f * np + 4 * row;
+__device__ __forceinline__ void ld3(const T* rec, size_t np, int f, size_t row, T (&v)[3]) {
+    const T* p = rec + (size_t)f * np + row;
+    v[0] = p[0];
+    v[1] = p[np];
+    v[2] = p[2 * np];
+}
+template <typename T>
+__device__ __forceinline__ void st3(T* rec, size_t np, int f, size_t row, T a, T b, T c) {
+    T* p = rec + (size_t)f * np + row;
+    p[0] = a;
+    p[np] = b;
+    p[2 * np] = c;
 }
 
 // Problem states (PCG)
@@ -109,9 +122,9 @@ struct PcgDesc {
     const int* slice_ptr;  // [n_slices+1] first slot of each slice
     const int* col;        // [slots] column block or -1
     const T* val;          // [slots/32][9][32]
-    const T* dinv;         // [9][npad32(n)] inverse diagonal blocks, entry-major
+    const T* dinv;         // [kDinv][npad32(n)] inverse diagonal blocks, entry-major
     T* nb;                 // [n][4] neighbour records (u)
-    T* rec;                // the six row fields (dx, r, p, s, w, zb), field-major (rec_field)
+    T* rec;                // the six row fields (dx, r, p, s, w, zb), three planes each (ld3, st3)
     double* part;          // [tiles][4] tile partials
     ProbScal* sc;
     int n_rows, n_tiles, unit_begin;   // the SpMV's tiles (autotuned rows per block)

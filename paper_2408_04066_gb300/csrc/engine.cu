@@ -120,7 +120,7 @@ size_t bytes_per_slot(const mfem_ctx* c) {
     const size_t kt = c->slot.prec == 1 ? 4 : 8;
     const size_t slots = (size_t)c->plan.slice_ptr.back();
     return H * 12 * 8 + 4 * n * 3 * 8 + (kt == 4 ? n * 3 * 8 + H * 9 * 8 : 0) + m * 12 * 8 + m * kKe * kt + slots * 9 * kt +
-           9 * npad32((int)n) * kt +
+           kDinv * npad32((int)n) * kt +
            kVecStride * npad32((int)n) * kt + (size_t)part_tiles_for(c) * 4 * 8 + sizeof(ProbScal) + 4 + 8 + 8 +
            H * 12 * 8 + 128 + (c->opt.init == MFEM_INIT_WARM ? 2 * n * 3 * 8 : 0) + 4 + (line_search(c) ? n * 3 * 8 : 0) +
            (c->mesh.coarse_n > 0 ? ((n + 255) / 256) * 24 * 4 + (coarse_ks(c) + 1) * c->mesh.coarse_n * 4 + 128 +
@@ -161,7 +161,7 @@ mfem_status alloc_slots(mfem_ctx* c, int B) {
     AL(S.ge, B * m * 12 * 8);
     AL(S.Ke, (B * m * kKe + kKePad) * kt);
     AL(S.val, B * slots * 9 * kt);
-    AL(S.dinv, B * 9 * npad32((int)n) * kt);
+    AL(S.dinv, B * kDinv * npad32((int)n) * kt);
     AL(S.vec, B * kVecStride * npad32((int)n) * kt);
     AL(S.part, B * (size_t)S.part_tiles * 4 * 8);
     AL(S.sc, B * sizeof(ProbScal));
@@ -268,7 +268,7 @@ namespace {
 // Algorithmic bytes of one PCG iteration of one problem (each datum crossing
 // HBM once, 3-vectors counted as 3 elements): k_pcg_spmv reads the matrix
 // values and column ids and the row's u and r, and writes w (the neighbours' u
-// are the same vector); k_pcg_update reads u, w, p, s, dx, r and the 9-element
+// are the same vector); k_pcg_update reads u, w, p, s, dx, r and the 6-element
 // D^-1 and writes p, s, dx, r and zb, and u under block Jacobi.  With the
 // two-level preconditioner the update reads the aggregate offset (16) for the
 // restriction and the correction reads zb and the offset and writes u (per
@@ -276,7 +276,7 @@ namespace {
 double pcg_bytes_per_iter(const mfem_ctx* c, bool coarse) {
     const double kt = c->slot.prec == 1 ? 4.0 : 8.0;
     const double nnzb = (double)c->plan.nnz_blocks, n = c->plan.n;
-    double b = nnzb * (9.0 * kt + 4.0) + n * (3.0 * 3.0 * kt) + n * (6.0 * 3.0 * kt + 9.0 * kt + 5.0 * 3.0 * kt);
+    double b = nnzb * (9.0 * kt + 4.0) + n * (3.0 * 3.0 * kt) + n * (6.0 * 3.0 * kt + kDinv * kt + 5.0 * 3.0 * kt);
     b += coarse ? n * (16.0 + 3.0 * kt + 16.0 + 3.0 * kt) : n * 3.0 * kt;
     return b;
 }
@@ -311,7 +311,7 @@ void build_descs(std::vector<Group>& gs, int tile, int prec, std::vector<PcgDesc
             d.slice_ptr = c->mesh.slice_ptr;
             d.col = c->mesh.col;
             d.val = (const T*)c->slot.val + (size_t)b * slots * 9;
-            d.dinv = (const T*)c->slot.dinv + (size_t)b * 9 * npad32(n);
+            d.dinv = (const T*)c->slot.dinv + (size_t)b * kDinv * npad32(n);
             const size_t np = npad32(n);
             T* v = (T*)c->slot.vec + (size_t)b * kVecStride * np;
             d.nb = v + kOffNB * np;

@@ -86,18 +86,6 @@ __global__ void k_coarse_split(const float* __restrict__ rc, int N, int ldr, int
                    rc[(size_t)b * ldr + k]);
 }
 
-__device__ __forceinline__ void ldv(const float* p, float (&v)[3]) {
-    const float4 a = *reinterpret_cast<const float4*>(p);
-    v[0] = a.x;
-    v[1] = a.y;
-    v[2] = a.z;
-}
-__device__ __forceinline__ void ldv(const double* p, double (&v)[3]) {
-    const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
-    v[0] = a.x;
-    v[1] = a.y;
-    v[2] = b.x;
-}
 __device__ __forceinline__ void stv(float* p, const float (&v)[3]) {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], 0.f);
 }
@@ -323,7 +311,7 @@ __global__ void __launch_bounds__(kFuThreads, 1)
         T z[kTcProbs][3];
 #pragma unroll
         for (int p = 0; p < kTcProbs; ++p)
-            if (dp[p]) ldv(rec_field(dp[p]->rec, npad32(n), kRecZB, row), z[p]);
+            if (dp[p]) ld3((const T*)dp[p]->rec, npad32(n), kRecZB, row, z[p]);
 #pragma unroll
         for (int p = 0; p < kTcProbs; ++p) {
             const PcgDesc<T>* d = dp[p];

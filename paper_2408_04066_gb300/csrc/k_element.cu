@@ -25,17 +25,17 @@ constexpr double kFallbackJ = 0.25;    // mixed path: det S below this -> FP64 H
 constexpr int kMaxStagedHandles = 64;   // pose rotations staged in shared memory up to this many handles
 
 // Gather the four vertex positions of tet k of problem b (optionally x + alpha dx).
-// dx, if given, is read with a stride of dx_stride elements per vertex.
+// dx, if given, is three planes, plane elements apart.
 template <typename T>
 __device__ __forceinline__ void gather_x(const double* __restrict__ x, const T* __restrict__ dx,
-                                         double alpha, int4 tv, double (&xa)[4][3], int dx_stride = 3) {
+                                         double alpha, int4 tv, double (&xa)[4][3], size_t plane = 0) {
     const int id[4] = {tv.x, tv.y, tv.z, tv.w};
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             double v = x[3 * (size_t)id[a] + i];
-            if (dx) v = fma(alpha, (double)dx[(size_t)dx_stride * id[a] + i], v);
+            if (dx) v = fma(alpha, (double)dx[i * plane + id[a]], v);
             xa[a][i] = v;
         }
 }
@@ -969,10 +969,9 @@ __global__ void __launch_bounds__(kTetTile) k_energy_trial(ElemArgs A) {
     if (k < m) {
         const double* x = A.slot.x + (size_t)b * n * 3;
         // the dx field: 4 elements per vertex
-        const T* dx = rec_field((const T*)A.slot.vec + (size_t)b * kVecStride * npad32(n) + kOffRec * npad32(n),
-                                npad32(n), kRecDX, 0);
+        const T* dx = (const T*)A.slot.vec + ((size_t)b * kVecStride + kOffRec + kRecDX) * npad32(n);   // three planes
         double xa[4][3], G[4][3], Q[3][3], F[3][3], S[6], sig[6];
-        gather_x<T>(x, dx, A.slot.alpha[b], M.tet[k], xa, 4);
+        gather_x<T>(x, dx, A.slot.alpha[b], M.tet[k], xa, npad32(n));
         load_G(M.Dminv64, m, k, G);
         tet_rotation(A, xf, qs, k, xa, G, Q);
         stretch(xa, G, Q, F, S);
@@ -980,8 +979,8 @@ __global__ void __launch_bounds__(kTetTile) k_energy_trial(ElemArgs A) {
     }
     if (k < n) {
         const double* xv = A.slot.x + ((size_t)b * n + k) * 3;
-        const T* dv = rec_field((const T*)A.slot.vec + (size_t)b * kVecStride * npad32(n) + kOffRec * npad32(n),
-                                npad32(n), kRecDX, k);
+        T dv[3];
+        ld3((const T*)A.slot.vec + ((size_t)b * kVecStride + kOffRec) * npad32(n), npad32(n), kRecDX, k, dv);
         const double al = A.slot.alpha[b];
         const double y[3] = {fma(al, (double)dv[0], xv[0]), fma(al, (double)dv[1], xv[1]),
                              fma(al, (double)dv[2], xv[2])};

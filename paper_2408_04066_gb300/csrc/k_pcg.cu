@@ -120,18 +120,17 @@ __global__ void k_pcg_init(ElemArgs A, double tol2, int maxit, const double* __r
     float r32[3] = {0.f, 0.f, 0.f};
     if (row < n) {
         const double* g = A.slot.g + ((size_t)b * n + row) * 3;
-        const T* di = (const T*)A.slot.dinv + (size_t)b * 9 * npad32(n);
+        const T* di = (const T*)A.slot.dinv + (size_t)b * kDinv * npad32(n);
         T* rec = vecp<T>(A.slot, b, kOffRec, n);
         const size_t np = npad32(n);
         const T r[3] = {(T)(-g[0]), (T)(-g[1]), (T)(-g[2])};
         T z[3];
         apply_dinv(di, np, row, r, z);
-        st4(rec_field(rec, np, kRecDX, row), (T)0, (T)0, (T)0);
-        st4(rec_field(rec, np, kRecR, row), r[0], r[1], r[2]);
-        st4(rec_field(rec, np, kRecP, row), (T)0, (T)0, (T)0);
-        st4(rec_field(rec, np, kRecS, row), (T)0, (T)0, (T)0);
-        st4(rec_field(rec, np, kRecW, row), (T)0, (T)0, (T)0);
-        st4(rec_field(rec, np, kRecZB, row), z[0], z[1], z[2]);
+        st3(rec, np, kRecDX, row, (T)0, (T)0, (T)0);
+        st3(rec, np, kRecR, row, r[0], r[1], r[2]);
+        st3(rec, np, kRecP, row, (T)0, (T)0, (T)0);
+        st3(rec, np, kRecS, row, (T)0, (T)0, (T)0);
+        st3(rec, np, kRecZB, row, z[0], z[1], z[2]);
         if (!coarse) st4(vecp<T>(A.slot, b, kOffNB, n) + 4 * (size_t)row, z[0], z[1], z[2]);
         v[0] = (double)r[0] * (double)r[0] + (double)r[1] * (double)r[1] + (double)r[2] * (double)r[2];
         r32[0] = (float)r[0];
@@ -303,10 +302,10 @@ __global__ void __launch_bounds__(TILE * 2, (sizeof(T) == 4 ? 1024 : 512) / TILE
     const size_t np = npad32(d.n_rows);
     if (owner) {
         ld4(d.nb + 4 * (size_t)row, ur);
-        st4(rec_field(d.rec, np, kRecW, row), a0, a1, a2);
+        st3(d.rec, np, kRecW, row, a0, a1, a2);
     }
     T r[3] = {0, 0, 0};
-    if (owner) ld4(rec_field(d.rec, np, kRecR, row), r);
+    if (owner) ld3(d.rec, np, kRecR, row, r);
     const double v = warp_sums3(dot3_partial(r[0], r[1], r[2], ur[0], ur[1], ur[2]),
                                 dot3_wu(a0, a1, a2, ur[0], ur[1], ur[2]),
                                 dot3_partial(r[0], r[1], r[2], r[0], r[1], r[2]));   // value i in lane i
@@ -397,8 +396,8 @@ __global__ void __launch_bounds__(TILE, RowShape<T>::kOcc / TILE) k_pcg_spmv_row
     const size_t np = npad32(d.n_rows);
     if (valid) {
         ld4(d.nb + 4 * (size_t)row, ur);
-        ld4(rec_field(d.rec, np, kRecR, row), r);
-        st4(rec_field(d.rec, np, kRecW, row), a0, a1, a2);
+        ld3(d.rec, np, kRecR, row, r);
+        st3(d.rec, np, kRecW, row, a0, a1, a2);
     }
     const double v = warp_sums3(dot3_partial(r[0], r[1], r[2], ur[0], ur[1], ur[2]),
                                 dot3_wu(a0, a1, a2, ur[0], ur[1], ur[2]),
@@ -426,11 +425,11 @@ __global__ void __launch_bounds__(TILE) k_pcg_update(const PcgDesc<T>* __restric
         const size_t np = npad32(d.n_rows);
         T uu[3], ww[3], pp[3], ss[3], dx[3], r[3], z[3];
         ld4(d.nb + 4 * (size_t)row, uu);
-        ld4(rec_field(d.rec, np, kRecW, row), ww);
-        ld4(rec_field(d.rec, np, kRecP, row), pp);
-        ld4(rec_field(d.rec, np, kRecS, row), ss);
-        ld4(rec_field(d.rec, np, kRecDX, row), dx);
-        ld4(rec_field(d.rec, np, kRecR, row), r);
+        ld3(d.rec, np, kRecW, row, ww);
+        ld3(d.rec, np, kRecP, row, pp);
+        ld3(d.rec, np, kRecS, row, ss);
+        ld3(d.rec, np, kRecDX, row, dx);
+        ld3(d.rec, np, kRecR, row, r);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             pp[i] = fma(beta, pp[i], uu[i]);
@@ -439,11 +438,11 @@ __global__ void __launch_bounds__(TILE) k_pcg_update(const PcgDesc<T>* __restric
             r[i] = fma(-alpha, ss[i], r[i]);
         }
         apply_dinv(d.dinv, np, row, r, z);
-        st4(rec_field(d.rec, np, kRecP, row), pp[0], pp[1], pp[2]);
-        st4(rec_field(d.rec, np, kRecS, row), ss[0], ss[1], ss[2]);
-        st4(rec_field(d.rec, np, kRecDX, row), dx[0], dx[1], dx[2]);
-        st4(rec_field(d.rec, np, kRecR, row), r[0], r[1], r[2]);
-        st4(rec_field(d.rec, np, kRecZB, row), z[0], z[1], z[2]);
+        st3(d.rec, np, kRecP, row, pp[0], pp[1], pp[2]);
+        st3(d.rec, np, kRecS, row, ss[0], ss[1], ss[2]);
+        st3(d.rec, np, kRecDX, row, dx[0], dx[1], dx[2]);
+        st3(d.rec, np, kRecR, row, r[0], r[1], r[2]);
+        st3(d.rec, np, kRecZB, row, z[0], z[1], z[2]);
         if (!coarse) st4(d.nb + 4 * (size_t)row, z[0], z[1], z[2]);   // u = D^{-1} r
         r32[0] = (float)r[0];
         r32[1] = (float)r[1];
@@ -617,7 +616,7 @@ __global__ void __launch_bounds__(TILE) k_pcg_correct(const PcgDesc<T>* __restri
     if (sc->state != kActive) return;   // block-uniform: before any barrier
     // the row's own load goes out first, so its latency overlaps the staging
     T z[3] = {(T)0, (T)0, (T)0};
-    if (row < d.n_rows) ld4(rec_field(d.rec, npad32(d.n_rows), kRecZB, row), z);
+    if (row < d.n_rows) ld3(d.rec, npad32(d.n_rows), kRecZB, row, z);
     // slice partials of e, one load per thread, then added in slice order
     for (int idx = threadIdx.x; idx < kMaxAgg * 6 * n_ks && idx < TILE; idx += TILE) {
         const int ks = idx / (kMaxAgg * 6), r = idx - ks * kMaxAgg * 6, a = a0 + r / 6;

@@ -295,19 +295,19 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
     }
 
     // ---- the row's state
-    T r[3] = {0, 0, 0}, pp[3] = {0, 0, 0}, ss[3] = {0, 0, 0}, dx[3] = {0, 0, 0}, zb[3] = {0, 0, 0}, di[9];
+    T r[3] = {0, 0, 0}, pp[3] = {0, 0, 0}, ss[3] = {0, 0, 0}, dx[3] = {0, 0, 0}, zb[3] = {0, 0, 0}, di[kDinv];
     float4 off = make_float4(0.f, 0.f, 0.f, 0.f);
     int base = 0, w = 0;
 #pragma unroll
-    for (int e = 0; e < 9; ++e) di[e] = 0;
+    for (int e = 0; e < kDinv; ++e) di[e] = 0;
     if (valid) {
-        ld4(rec_field(d.rec, np, kRecR, row), r);
-        ld4(rec_field(d.rec, np, kRecP, row), pp);
-        ld4(rec_field(d.rec, np, kRecS, row), ss);
-        ld4(rec_field(d.rec, np, kRecDX, row), dx);
-        ld4(rec_field(d.rec, np, kRecZB, row), zb);
+        ld3(d.rec, np, kRecR, row, r);
+        ld3(d.rec, np, kRecP, row, pp);
+        ld3(d.rec, np, kRecS, row, ss);
+        ld3(d.rec, np, kRecDX, row, dx);
+        ld3(d.rec, np, kRecZB, row, zb);
 #pragma unroll
-        for (int e = 0; e < 9; ++e) di[e] = d.dinv[e * np + row];
+        for (int e = 0; e < kDinv; ++e) di[e] = d.dinv[e * np + row];
         if (coarse) off = d.crel[row];
         const int s = row >> 5;
         base = __ldg(d.slice_ptr + s);
@@ -679,8 +679,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
             dx[i] = fma(alpha, pp[i], dx[i]);
             r[i] = fma(-alpha, ss[i], r[i]);
         }
-#pragma unroll
-        for (int i = 0; i < 3; ++i) zb[i] = di[3 * i] * r[0] + di[3 * i + 1] * r[1] + di[3 * i + 2] * r[2];
+        sym_product(di, r, zb);
         if (coarse) {
             float y[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             if (off.w != 0.f) {
@@ -722,12 +721,12 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
 
     // ---- write back: the increment; the other vectors only if the solve goes on
     if (valid) {
-        st4(rec_field(d.rec, np, kRecDX, row), dx[0], dx[1], dx[2]);
+        st3(d.rec, np, kRecDX, row, dx[0], dx[1], dx[2]);
         if (active) {
-            st4(rec_field(d.rec, np, kRecR, row), r[0], r[1], r[2]);
-            st4(rec_field(d.rec, np, kRecP, row), pp[0], pp[1], pp[2]);
-            st4(rec_field(d.rec, np, kRecS, row), ss[0], ss[1], ss[2]);
-            st4(rec_field(d.rec, np, kRecZB, row), zb[0], zb[1], zb[2]);
+            st3(d.rec, np, kRecR, row, r[0], r[1], r[2]);
+            st3(d.rec, np, kRecP, row, pp[0], pp[1], pp[2]);
+            st3(d.rec, np, kRecS, row, ss[0], ss[1], ss[2]);
+            st3(d.rec, np, kRecZB, row, zb[0], zb[1], zb[2]);
         }
     }
     if (t == 0) {

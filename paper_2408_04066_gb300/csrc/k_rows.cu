@@ -112,8 +112,9 @@ __device__ __forceinline__ void add_block(KT (&acc)[9], int code, const KT (&v)[
 // inverse.  Consecutive threads take consecutive upper slots, so the own
 // writes are nearly coalesced; the mirror writes are scattered.  The gradient
 // gather runs in k_gradient.
-// Block Jacobi: the inverse of a 3x3 diagonal block by its cofactors, entry e
-// written at di[e * np] (one run per entry).  The FP64 path forms it in FP64.
+// Block Jacobi: the inverse of a symmetric 3x3 diagonal block by its cofactors,
+// its six entries (00, 11, 22, 12, 02, 01) written at di[e * np] (one run per
+// entry).  The FP64 path forms it in FP64.
 // The mixed path forms it in FP32 from the block scaled by a power of two
 // (the largest entry into [0.5, 1): no overflow or underflow of the
 // determinant, and the scaling is exact).  It is only the preconditioner, and
@@ -123,14 +124,11 @@ __device__ __forceinline__ void block_jacobi(const double (&a)[9], double* di, s
     const double det = a[0] * c00 + a[1] * c01 + a[2] * c02;
     const double id = det != 0.0 ? 1.0 / det : 0.0;
     di[0 * np] = c00 * id;
-    di[1 * np] = (a[2] * a[7] - a[1] * a[8]) * id;
-    di[2 * np] = (a[1] * a[5] - a[2] * a[4]) * id;
-    di[3 * np] = c01 * id;
-    di[4 * np] = (a[0] * a[8] - a[2] * a[6]) * id;
-    di[5 * np] = (a[2] * a[3] - a[0] * a[5]) * id;
-    di[6 * np] = c02 * id;
-    di[7 * np] = (a[1] * a[6] - a[0] * a[7]) * id;
-    di[8 * np] = (a[0] * a[4] - a[1] * a[3]) * id;
+    di[1 * np] = (a[0] * a[8] - a[2] * a[6]) * id;
+    di[2 * np] = (a[0] * a[4] - a[1] * a[3]) * id;
+    di[3 * np] = (a[2] * a[3] - a[0] * a[5]) * id;
+    di[4 * np] = (a[1] * a[5] - a[2] * a[4]) * id;
+    di[5 * np] = (a[2] * a[7] - a[1] * a[8]) * id;
 }
 __device__ __forceinline__ void block_jacobi(const float (&acc)[9], float* di, size_t np) {
     float mx = 0.f;
@@ -147,14 +145,11 @@ __device__ __forceinline__ void block_jacobi(const float (&acc)[9], float* di, s
     // inv(acc) = sc inv(a)
     const float id = det != 0.f ? sc / det : 0.f;
     di[0 * np] = c00 * id;
-    di[1 * np] = (a[2] * a[7] - a[1] * a[8]) * id;
-    di[2 * np] = (a[1] * a[5] - a[2] * a[4]) * id;
-    di[3 * np] = c01 * id;
-    di[4 * np] = (a[0] * a[8] - a[2] * a[6]) * id;
-    di[5 * np] = (a[2] * a[3] - a[0] * a[5]) * id;
-    di[6 * np] = c02 * id;
-    di[7 * np] = (a[1] * a[6] - a[0] * a[7]) * id;
-    di[8 * np] = (a[0] * a[4] - a[1] * a[3]) * id;
+    di[1 * np] = (a[0] * a[8] - a[2] * a[6]) * id;
+    di[2 * np] = (a[0] * a[4] - a[1] * a[3]) * id;
+    di[3 * np] = (a[2] * a[3] - a[0] * a[5]) * id;
+    di[4 * np] = (a[1] * a[5] - a[2] * a[4]) * id;
+    di[5 * np] = (a[2] * a[7] - a[1] * a[8]) * id;
 }
 
 template <typename KT>
@@ -216,7 +211,7 @@ __global__ void __launch_bounds__(kRowTile) k_assemble_slots(ElemArgs A) {
 #pragma unroll
             for (int j = 0; j < 3; ++j) mout[32 * (3 * i + j)] = acc[3 * j + i];
     }
-    if (diag) block_jacobi(acc, (KT*)A.slot.dinv + (size_t)b * 9 * npad32(M.n) + row, npad32(M.n));
+    if (diag) block_jacobi(acc, (KT*)A.slot.dinv + (size_t)b * kDinv * npad32(M.n) + row, npad32(M.n));
 }
 
 // Gradient only (a convergence test that needs no matrix): |g_free|^2 per problem.
@@ -241,7 +236,8 @@ __global__ void __launch_bounds__(kRowTile) k_slope(ElemArgs A) {
     double v[1] = {0.0};
     if (row < n) {
         const double* g = A.slot.g + ((size_t)b * n + row) * 3;
-        const T* dx = rec_field(vecp<T>(A.slot, b, kOffRec, n), npad32(n), kRecDX, row);
+        T dx[3];
+        ld3((const T*)vecp<T>(A.slot, b, kOffRec, n), npad32(n), kRecDX, row, dx);
         v[0] = g[0] * (double)dx[0] + g[1] * (double)dx[1] + g[2] * (double)dx[2];
     }
     double tot[1];
@@ -259,7 +255,7 @@ __global__ void k_update(ElemArgs A) {
     if (i >= 3 * n) return;
     const T* rec = vecp<T>(A.slot, b, kOffRec, n);
     double* x = A.slot.x + (size_t)b * n * 3;
-    x[i] = fma(A.slot.alpha[b], (double)rec_field(rec, npad32(n), kRecDX, i / 3)[i % 3], x[i]);
+    x[i] = fma(A.slot.alpha[b], (double)rec[(kRecDX + i % 3) * npad32(n) + i / 3], x[i]);
 }
 
 __global__ void k_unpermute(ElemArgs A, double* __restrict__ out) {

@@ -64,7 +64,7 @@ struct SlotDev {
     double* ge = nullptr;    // [B][m][12] element forces
     void* Ke = nullptr;      // [B][m][kKe] + kKePad element blocks (float or double)
     void* val = nullptr;     // [B][slots*9]
-    void* dinv = nullptr;    // [B][9][npad32(n)] block-Jacobi inverses, entry-major
+    void* dinv = nullptr;    // [B][kDinv][npad32(n)] block-Jacobi inverses, entry-major
     void* vec = nullptr;     // [B][kVecStride][npad32(n)]: the neighbour record nb and the six row fields
     double* part = nullptr;  // [B][tiles][4]
     int part_tiles = 0;

@@ -123,16 +123,22 @@ __device__ __forceinline__ void coeffs(const ProbScal* sc, double& a, double& b)
     b = sc->beta;
 }
 
-// z_bj = D^{-1} r for one row: D^{-1} row-major 3x3, its entry e of every row
-// stored contiguously (entry e of row `row` at di[e * np + row], np = npad32(n)),
-// so a warp's load of one entry is one contiguous 32-row run
+// z = M r, M symmetric with entries 00, 11, 22, 12, 02, 01
 template <typename T>
-__device__ __forceinline__ void apply_dinv(const T* __restrict__ di, size_t np, int row, const T (&r)[3], T (&z)[3]) {
-    T m[9];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) m[e] = di[e * np + row];
+__device__ __forceinline__ void sym_product(const T (&s)[kDinv], const T (&r)[3], T (&z)[3]) {
+    const T m[9] = {s[0], s[5], s[4], s[5], s[1], s[3], s[4], s[3], s[2]};
 #pragma unroll
     for (int i = 0; i < 3; ++i) z[i] = m[3 * i] * r[0] + m[3 * i + 1] * r[1] + m[3 * i + 2] * r[2];
+}
+// z_bj = D^{-1} r for one row: entry e of D^{-1} of every row stored contiguously
+// (at di[e * np + row], np = npad32(n)), so a warp's load of one entry is one
+// contiguous 32-row run
+template <typename T>
+__device__ __forceinline__ void apply_dinv(const T* __restrict__ di, size_t np, int row, const T (&r)[3], T (&z)[3]) {
+    T m[kDinv];
+#pragma unroll
+    for (int e = 0; e < kDinv; ++e) m[e] = di[e * np + row];
+    sym_product(m, r, z);
 }
 
 }  // namespace mfem
