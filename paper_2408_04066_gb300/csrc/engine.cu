@@ -642,13 +642,15 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
             c->prof.launches++;
         } else if (count) {
             c->prof.end(pe, c->stream);
-            int cl = nj;   // coarse kernels: per job the product (fused with the correction on the tensor cores) ...
-            bool cuda_core = false;
+            // coarse kernels: one for the tensor-core products and corrections of up
+            // to kCoarseJobs meshes, one product per CUDA-core job, the per-aggregate
+            // sums of larger aggregates, and the correction after CUDA-core products
+            int n_tc = 0, n_cc = 0, rc = 0;
             for (const auto& j : jobs) {
-                cl += j.agg_units > 1;   // ... the per-aggregate sums of larger aggregates ...
-                cuda_core |= j.Abf == nullptr;
+                (j.Abf ? n_tc : n_cc)++;
+                rc |= j.agg_units > 1;
             }
-            cl += cuda_core ? 1 : 0;   // ... and the correction after CUDA-core products
+            const int cl = (n_tc + kCoarseJobs - 1) / kCoarseJobs + n_cc + rc + (n_cc ? 1 : 0);
             c->prof.launches += (2 + cl) * n_it;
             c->prof.pcg_launches += 2 * n_it;
             c->prof.coarse_launches += cl * n_it;

@@ -44,18 +44,24 @@ namespace mfem {
 
 namespace {
 
-constexpr int kFuStages = 4;                      // shared-memory ring of A + B chunks
+// Shared-memory ring of A + B chunks: four stages, one CTA an SM; two stages and
+// two CTAs an SM where a launch of several meshes has more CTAs than the device
+// has SMs, so that none waits for a second wave (12 + 12 streams of the 200k and
+// 50k figures 80.9 -> 78.6 us an iteration, the 10k/50k/200k requests 18.2 -> 17.7
+// ms; one mesh alone is slower with two: 72.0 -> 74.8 us, 16 poses of the 200k figure).
+constexpr int kFuStages = 4, kFuStagesMulti = 2;
 constexpr int kFuThreads = 320;                   // 10 warps: one per 32 vertex rows of 5 x 64
 constexpr int kTcProbs = kCoarseGroupSlots;       // request slots per CTA group
 constexpr int kTcN = kCoarseBRows;                // MMA N: three BF16 parts per slot
 constexpr int kFuStepB = kTcN * 16 * 2;           // bytes of B per K step (1.5 KB)
 constexpr int kFuChunkB = kFuStepB * kTcSteps;    // 12 KB
 constexpr int kFuStage = kFuChunkA + kFuChunkB;   // 44 KB
-constexpr int kFuSmem = kFuStages * kFuStage + 128;
+constexpr int fu_smem(int stages) { return stages * kFuStage + 128; }
 constexpr int kTcTmemCols = 64;                   // >= kTcN, a power of two >= 32
 
 static_assert(6 * kFuAggsBlk <= kTcM, "a row block's coarse rows fit the MMA's M");
 static_assert(kFuChunkB == kCoarseBChunk * 2, "B chunk layout shared with the restriction");
+constexpr int kSms = 152;                         // SMs of a GB300
 static_assert(kTcM * kTcN * 4 <= kFuStage, "the partial product fits one stage for the cluster sum");
 static_assert(kFuChunkA % 16 == 0 && kFuChunkB % 16 == 0 && kFuStage % 1024 == 0, "bulk copies: 16-byte units");
 static_assert(kFuThreads >= 128, "warps 0-3 read the 128 TMEM lanes");
@@ -111,22 +117,34 @@ __device__ __forceinline__ float ld_cluster_f32(const float* local, uint32_t ran
     return v;
 }
 
-// Cluster (rb, pg): row block rb (aggregates kFuAggsBlk rb ..), request slots
+// The jobs (meshes) of one launch: job j's clusters are c0[j] .. c0[j + 1] - 1.
+// One launch for all of them: a small mesh's product takes as long as a large
+// one's (its chain of latencies) on a few SMs, so several run side by side.
+struct TcJobs {
+    struct Job {
+        const __nv_bfloat16* Abf;
+        const uint16_t* Bs;
+        unsigned* err;
+        int N, d0, nd;
+    } job[kCoarseJobs];
+    int c0[kCoarseJobs + 1];
+    int n;
+};
+
+// Cluster (rb, pg) of a job: row block rb (aggregates kFuAggsBlk rb ..), request slots
 // 16 pg .. 16 pg + 15 of the context; CTA q = cluster rank takes chunks
 // [q c_per, (q + 1) c_per) of the K range and corrects aggregates
 // kFuAggsBlk rb + kFuAggsCta q ...  The problems are found in the descriptor
 // table d0 .. d0+nd-1 by slot; a slot without a two-level problem inside PCG
 // contributes nothing (its B columns give outputs never read).
 // e_out (mfem_coarse_apply): write e[slot][row] instead of the correction.
-template <typename T>
-__global__ void __launch_bounds__(kFuThreads, 1)
-    k_coarse_fused(const __nv_bfloat16* __restrict__ Abf, int N, int nkc, const uint16_t* __restrict__ Bs,
-                   const PcgDesc<T>* __restrict__ D, int d0, int nd, unsigned* __restrict__ err,
-                   float* __restrict__ e_out) {
+template <typename T, int ST>
+__global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
+    k_coarse_fused(const __grid_constant__ TcJobs J, const PcgDesc<T>* __restrict__ D, float* __restrict__ e_out) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kFuStages * kFuStage);   // chunk landed
-    uint64_t* empty = full + kFuStages;                                           // its MMAs done
-    uint64_t* done = empty + kFuStages;                                           // every MMA done
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + ST * kFuStage);   // chunk landed
+    uint64_t* empty = full + ST;                                           // its MMAs done
+    uint64_t* done = empty + ST;                                           // every MMA done
     uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
     float* red = reinterpret_cast<float*>(smem);   // after the K loop: the partial product [kTcN][kTcM]
     __shared__ const PcgDesc<T>* dp[kTcProbs];
@@ -135,10 +153,19 @@ __global__ void __launch_bounds__(kFuThreads, 1)
     __shared__ int any, s_ok;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const uint32_t q = cluster_rank();
-    const int rb = blockIdx.x / kFuSplit, pg = blockIdx.y;
+    const int cid = blockIdx.x / kFuSplit;   // cluster
+    int ji = 0;
+#pragma unroll
+    for (int i = 1; i < kCoarseJobs; ++i) ji += i < J.n && cid >= J.c0[i];
+    const __nv_bfloat16* __restrict__ Abf = J.job[ji].Abf;
+    const uint16_t* __restrict__ Bs = J.job[ji].Bs;
+    unsigned* __restrict__ err = J.job[ji].err;
+    const int N = J.job[ji].N, d0 = J.job[ji].d0, nd = J.job[ji].nd;
+    const int nkc = coarse_chunks(N);
+    const int rb = (cid - J.c0[ji]) % row_blocks(N), pg = (cid - J.c0[ji]) / row_blocks(N);
     const int c_per = coarse_part_chunks(N);
     const int c_lo = min(nkc, (int)q * c_per), nch = min(nkc, c_lo + c_per) - c_lo;   // this CTA's chunks
-    const int nst = nch < kFuStages ? nch : kFuStages;
+    const int nst = nch < ST ? nch : ST;
     const unsigned char* gA =
         reinterpret_cast<const unsigned char*>(Abf) + ((size_t)rb * nkc + c_lo) * kFuChunkA;
     const unsigned char* gB =
@@ -160,7 +187,7 @@ __global__ void __launch_bounds__(kFuThreads, 1)
     if (t == 0) {
         any = 0;
         s_ok = 1;
-        for (int c = 0; c < 2 * kFuStages + 1; ++c) mbar_init(&full[c], 1);
+        for (int c = 0; c < 2 * ST + 1; ++c) mbar_init(&full[c], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         for (int c = 0; c < nst; ++c) {
@@ -213,8 +240,8 @@ __global__ void __launch_bounds__(kFuThreads, 1)
         bool ok = true;
         int issued = nst;   // chunks whose copies were issued
         for (int c = 0; c < nch && ok; ++c) {
-            const int s = c % kFuStages;
-            ok = mbar_wait(&full[s], (uint32_t)(c / kFuStages) & 1u);
+            const int s = c % ST;
+            ok = mbar_wait(&full[s], (uint32_t)(c / ST) & 1u);
             if (!ok) break;
             tc_fence_after();
             const uint32_t a0 = base + s * kFuStage, b0 = a0 + kFuChunkA;
@@ -223,11 +250,11 @@ __global__ void __launch_bounds__(kFuThreads, 1)
                           (c > 0 || k > 0) ? 1u : 0u);
             umma_commit(&empty[s]);
             // refill the stage of the previous chunk (its MMAs were issued one
-            // chunk ago) with the chunk kFuStages after it
-            const int cp = c - 1, cn = cp + kFuStages;
+            // chunk ago) with the chunk ST after it
+            const int cp = c - 1, cn = cp + ST;
             if (cp >= 0 && cn < nch) {
-                const int sp = cp % kFuStages;
-                ok = mbar_wait(&empty[sp], (uint32_t)(cp / kFuStages) & 1u);
+                const int sp = cp % ST;
+                ok = mbar_wait(&empty[sp], (uint32_t)(cp / ST) & 1u);
                 if (!ok) break;
                 mbar_expect_tx(&full[sp], kFuStage);
                 bulk_g2s(smem + sp * kFuStage, gA + (size_t)cn * kFuChunkA, kFuChunkA, &full[sp]);
@@ -242,7 +269,7 @@ __global__ void __launch_bounds__(kFuThreads, 1)
             atomicOr(err, 1u);
             // the copies in flight: the last use of each stage that was issued, bounded
             for (int c = issued - nst; c < issued; ++c)
-                if (c >= 0) mbar_wait(&full[c % kFuStages], (uint32_t)(c / kFuStages) & 1u);
+                if (c >= 0) mbar_wait(&full[c % ST], (uint32_t)(c / ST) & 1u);
         }
     }
     const bool fin = mbar_wait(done, 0);
@@ -351,16 +378,32 @@ cudaError_t coarse_split(const float* rc, int N, int ldr, int B, void* Bs, cudaS
     return cudaGetLastError();
 }
 
+template <typename T, int ST>
+static cudaError_t fu_attr() {
+    return cudaFuncSetAttribute(k_coarse_fused<T, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, fu_smem(ST));
+}
 cudaError_t coarse_tc_init() {
-    cudaError_t e = cudaFuncSetAttribute(k_coarse_fused<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFuSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_coarse_fused<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFuSmem);
+    cudaError_t e = fu_attr<float, kFuStages>();
+    if (e == cudaSuccess) e = fu_attr<double, kFuStages>();
+    if (e == cudaSuccess) e = fu_attr<float, kFuStagesMulti>();
+    if (e == cudaSuccess) e = fu_attr<double, kFuStagesMulti>();
     return e;
 }
 
 template <typename T>
-cudaError_t launch_coarse_fused(const cudaLaunchConfig_t& base, const CoarseJob& j, const PcgDesc<T>* descs,
-                                float* e_out) {
+cudaError_t launch_coarse_fused(const cudaLaunchConfig_t& base, const CoarseJob* jobs, int n_jobs,
+                                const PcgDesc<T>* descs, float* e_out) {
+    TcJobs J{};
+    int nc = 0;
+    for (int i = 0; i < n_jobs; ++i) {   // at most kCoarseJobs
+        const CoarseJob& j = jobs[i];
+        J.job[i] = TcJobs::Job{static_cast<const __nv_bfloat16*>(j.Abf), static_cast<const uint16_t*>(j.Bs), j.err,
+                               j.N, j.d0, j.nd};
+        J.c0[i] = nc;
+        nc += row_blocks(j.N) * ((j.slots + kCoarseGroupSlots - 1) / kCoarseGroupSlots);
+    }
+    J.n = n_jobs;
+    J.c0[n_jobs] = nc;
     cudaLaunchConfig_t cfg = base;
     cudaLaunchAttribute attr[2];
     int na = 0;
@@ -372,16 +415,19 @@ cudaError_t launch_coarse_fused(const cudaLaunchConfig_t& base, const CoarseJob&
     ++na;
     cfg.attrs = attr;
     cfg.numAttrs = na;
-    cfg.gridDim = dim3(kFuSplit * row_blocks(j.N), (j.slots + kCoarseGroupSlots - 1) / kCoarseGroupSlots);
+    cfg.gridDim = dim3(kFuSplit * nc);
     cfg.blockDim = dim3(kFuThreads);
-    cfg.dynamicSmemBytes = kFuSmem;
-    return cudaLaunchKernelEx(&cfg, k_coarse_fused<T>, static_cast<const __nv_bfloat16*>(j.Abf), j.N,
-                              coarse_chunks(j.N), static_cast<const uint16_t*>(j.Bs), descs, j.d0, j.nd, j.err, e_out);
+    if (n_jobs > 1 && kFuSplit * nc > kSms) {
+        cfg.dynamicSmemBytes = fu_smem(kFuStagesMulti);
+        return cudaLaunchKernelEx(&cfg, k_coarse_fused<T, kFuStagesMulti>, J, descs, e_out);
+    }
+    cfg.dynamicSmemBytes = fu_smem(kFuStages);
+    return cudaLaunchKernelEx(&cfg, k_coarse_fused<T, kFuStages>, J, descs, e_out);
 }
 
-template cudaError_t launch_coarse_fused<float>(const cudaLaunchConfig_t&, const CoarseJob&, const PcgDesc<float>*,
-                                                float*);
-template cudaError_t launch_coarse_fused<double>(const cudaLaunchConfig_t&, const CoarseJob&, const PcgDesc<double>*,
-                                                 float*);
+template cudaError_t launch_coarse_fused<float>(const cudaLaunchConfig_t&, const CoarseJob*, int,
+                                                const PcgDesc<float>*, float*);
+template cudaError_t launch_coarse_fused<double>(const cudaLaunchConfig_t&, const CoarseJob*, int,
+                                                 const PcgDesc<double>*, float*);
 
 }  // namespace mfem

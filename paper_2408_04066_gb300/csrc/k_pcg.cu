@@ -463,11 +463,11 @@ __global__ void __launch_bounds__(TILE) k_pcg_update(const PcgDesc<T>* __restric
 // in a fixed order.  Slice products go to ec[slice][row]; k_pcg_correct adds
 // the slices in order.
 // r_c of aggregates larger than one 64-row unit: the units' partials added in
-// unit order, for the problems d0 .. d0+nd-1 (grid.y) of one mesh.
+// unit order, for every problem of the table (grid.y) that has such aggregates.
 template <typename T>
-__global__ void k_coarse_rc(const PcgDesc<T>* __restrict__ D, int d0, int nd) {
-    const PcgDesc<T>& q = D[d0 + blockIdx.y];
-    const bool coarse = q.coarse != 0;
+__global__ void k_coarse_rc(const PcgDesc<T>* __restrict__ D) {
+    const PcgDesc<T>& q = D[blockIdx.y];
+    const bool coarse = q.coarse != 0 && q.agg_shift > 6;
     ProbScal* sc = q.sc;
     pdl_wait();
     pdl_trigger();
@@ -673,19 +673,27 @@ cudaError_t launch_pcg_iters_t(const PcgDesc<T>* descs, int n_probs, int n_units
         cudaError_t e;
         if (n_jobs > 0) {   // two-level: finish u of the current residual first
             bool any_cuda_core = false;
+            int rc_n = 0;   // the largest coarse space with aggregates of several units: their sums first
+            for (int j = 0; j < n_jobs; ++j)
+                if (jobs[j].agg_units > 1) rc_n = max(rc_n, jobs[j].N);
+            if (rc_n > 0) {
+                cudaLaunchConfig_t rc = cfg;
+                rc.gridDim = dim3((rc_n + 255) / 256, n_probs);
+                rc.blockDim = dim3(256);
+                e = cudaLaunchKernelEx(&rc, k_coarse_rc<T>, descs);
+                if (e != cudaSuccess) return e;
+            }
+            // tensor cores, BF16 A_c^{-1}: product and correction of every mesh in one launch
+            CoarseJob tc[kCoarseJobs];
+            int n_tc = 0;
             for (int j = 0; j < n_jobs; ++j) {
-                if (jobs[j].agg_units > 1) {   // per-aggregate sums of the unit partials
-                    cudaLaunchConfig_t rc = cfg;
-                    rc.gridDim = dim3((jobs[j].N + 255) / 256, jobs[j].nd);
-                    rc.blockDim = dim3(256);
-                    e = cudaLaunchKernelEx(&rc, k_coarse_rc<T>, descs, jobs[j].d0, jobs[j].nd);
+                if (jobs[j].Abf) tc[n_tc++] = jobs[j];
+                if (n_tc > 0 && (n_tc == kCoarseJobs || j == n_jobs - 1)) {
+                    e = launch_coarse_fused<T>(cfg, tc, n_tc, descs, nullptr);
                     if (e != cudaSuccess) return e;
+                    n_tc = 0;
                 }
-                if (jobs[j].Abf) {   // tensor cores, BF16 A_c^{-1}: product and correction in one kernel
-                    e = launch_coarse_fused<T>(cfg, jobs[j], descs, nullptr);
-                    if (e != cudaSuccess) return e;
-                    continue;
-                }
+                if (jobs[j].Abf) continue;
                 any_cuda_core = true;
                 cudaLaunchConfig_t gc = cfg;
                 const int np = jobs[j].nd <= 8 ? 8 : 16;
@@ -745,7 +753,7 @@ cudaError_t launch_coarse_only(const PcgDesc<float>* descs, int n_probs, const C
                                cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.stream = s;
-    if (job->Abf) return launch_coarse_fused<float>(cfg, *job, descs, e_out);
+    if (job->Abf) return launch_coarse_fused<float>(cfg, job, 1, descs, e_out);
     const int np = job->nd <= 8 ? 8 : 16;
     cfg.gridDim = dim3((job->N + 32 * kCoarseRowPasses - 1) / (32 * kCoarseRowPasses),
                        (job->N + kCoarseKC - 1) / kCoarseKC, (job->nd + np - 1) / np);

@@ -217,15 +217,17 @@ cudaError_t launch_coarse_only(const PcgDesc<float>* descs, int n_probs, const C
 // the packed BF16 rows of an N x N inverse and of the B operand for `slots`
 // request slots, the packing from the FP32 inverse, the split of FP32 coarse
 // residuals (rows of ldr floats) into the B operand, the one-time kernel
-// attribute set-up (before any capture), and the launch for one job (e_out
-// null: correction of the problems' u; else the product alone into e_out).
+// attribute set-up (before any capture), and the launch for up to kCoarseJobs
+// jobs (e_out null: correction of the problems' u; else the product alone into
+// e_out).
+constexpr int kCoarseJobs = 8;
 size_t coarse_tc_bytes(int N);
 size_t coarse_b_bytes(int N, int slots);
 cudaError_t coarse_tc_pack(const float* Ainv, int N, void* Abf, cudaStream_t s);
 cudaError_t coarse_split(const float* rc, int N, int ldr, int B, void* Bs, cudaStream_t s);
 cudaError_t coarse_tc_init();
 template <typename T>
-cudaError_t launch_coarse_fused(const cudaLaunchConfig_t& base, const CoarseJob& j, const PcgDesc<T>* descs,
-                                float* e_out);
+cudaError_t launch_coarse_fused(const cudaLaunchConfig_t& base, const CoarseJob* jobs, int n_jobs,
+                                const PcgDesc<T>* descs, float* e_out);
 
 }  // namespace mfem
