@@ -96,9 +96,9 @@ mfem_status upload(mfem_ctx* c, U** dst, const U* src, size_t count) {
 
 void free_slots(mfem_ctx* c) {
     SlotDev& S = c->slot;
-    void* ptrs[] = {S.xf, S.xf_prev, S.xpred, S.dcorr, S.tol2, S.coarse_on, S.rcp, S.ec, S.rcs, S.aggq, S.bsplit, S.epart, S.rbar,
+    void* ptrs[] = {S.xf, S.xf_prev, S.xpred, S.dcorr, S.rcp, S.ec, S.rcs, S.aggq, S.bsplit, S.epart, S.rbar,
                     S.x, S.xff, S.qff, S.xprev, S.xp,
-                    S.g, S.ge, S.Ke, S.val, S.dinv, S.vec, S.part, S.sc, S.active, S.alpha, S.outbuf};
+                    S.g, S.ge, S.Ke, S.val, S.dinv, S.vec, S.part, S.sc, S.active, S.outbuf};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     int prec = S.prec;
@@ -109,6 +109,9 @@ void free_slots(mfem_ctx* c) {
 
 // slices of the coarse product (ec partials per problem)
 size_t coarse_ks(const mfem_ctx* c) { return ((size_t)c->mesh.coarse_n + kCoarseKC - 1) / kCoarseKC; }
+
+// bytes of the control block of B problems (see alloc_slots)
+size_t ctl_bytes(size_t B) { return B * (2 * sizeof(int) + 2 * sizeof(double)); }
 
 int part_tiles_for(const mfem_ctx* c) {
     int a = (c->plan.n + 31) / 32, b = (c->plan.m + kTetTile - 1) / kTetTile;
@@ -165,10 +168,10 @@ mfem_status alloc_slots(mfem_ctx* c, int B) {
     AL(S.vec, B * kVecStride * npad32((int)n) * kt);
     AL(S.part, B * (size_t)S.part_tiles * 4 * 8);
     AL(S.sc, B * sizeof(ProbScal));
-    AL(S.active, B * sizeof(int));
-    AL(S.alpha, B * sizeof(double));
-    AL(S.tol2, B * sizeof(double));
-    AL(S.coarse_on, B * sizeof(int));
+    AL(S.active, ctl_bytes(B));   // the control block: active and coarse_on [B] ints, alpha and tol2 [B] doubles
+    S.coarse_on = S.active + B;
+    S.alpha = reinterpret_cast<double*>(S.active + 2 * (size_t)B);
+    S.tol2 = S.alpha + B;
     AL(S.rbar, B * (size_t)128);
     if (c->mesh.coarse_n > 0) {
         S.rcp_stride = (((size_t)n + 255) / 256) * (256 / kCoarseRows) * 6;
@@ -194,13 +197,12 @@ mfem_status alloc_slots(mfem_ctx* c, int B) {
     c->pcg_hist.assign((size_t)B * kPcgHistSteps, 0);
     // pinned host staging
     if (c->sc_host) cudaFreeHost(c->sc_host);
-    if (c->active_host) cudaFreeHost(c->active_host);
-    if (c->alpha_host) cudaFreeHost(c->alpha_host);
-    if (c->alpha_ring) cudaFreeHost(c->alpha_ring);
+    if (c->ctl_ring) cudaFreeHost(c->ctl_ring);
     CK(cudaMallocHost((void**)&c->sc_host, B * sizeof(ProbScal)));
-    CK(cudaMallocHost((void**)&c->active_host, (size_t)kStageRing * B * sizeof(int)));
-    CK(cudaMallocHost((void**)&c->alpha_host, B * sizeof(double)));
-    CK(cudaMallocHost((void**)&c->alpha_ring, (size_t)kStageRing * B * sizeof(double)));
+    CK(cudaMallocHost((void**)&c->ctl_ring, kStageRing * ctl_bytes(B)));
+    c->alpha_host.assign(B, 0.0);
+    c->tol2_host.assign(B, 0.0);
+    c->coarse_host.assign(B, 0);
     c->ring_pos = 0;
     size_t dcap = 2 * B * (std::max(sizeof(PcgDesc<float>), sizeof(PcgDesc<double>)) + sizeof(ResJob));
     if (dcap > c->descs_cap) {
@@ -359,37 +361,23 @@ mfem_status next_stage(mfem_ctx* c, int& pos) {
     return MFEM_OK;
 }
 
-mfem_status upload_active(mfem_ctx* c, int B, const std::vector<int>& flags) {
+// The problems a kernel acts on -> device; with `rest`, the whole control block
+// (step lengths, PCG targets and coarse flags as the host holds them) in the same
+// copy.
+mfem_status upload_active(mfem_ctx* c, int B, const std::vector<int>& flags, bool rest = false) {
     int pos = 0;
     mfem_status st = next_stage(c, pos);
     if (st != MFEM_OK) return st;
-    int* h = c->active_host + (size_t)pos * c->slot.cap;
-    for (int b = 0; b < B; ++b) h[b] = flags[b];
-    CK(cudaMemcpyAsync(c->slot.active, h, B * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    return MFEM_OK;
-}
-
-// B doubles -> device through a staging region that is not rewritten before
-// the copy has run
-mfem_status upload_doubles(mfem_ctx* c, int B, const double* v, double* dst) {
-    int pos = 0;
-    mfem_status st = next_stage(c, pos);
-    if (st != MFEM_OK) return st;
-    double* h = c->alpha_ring + (size_t)pos * c->slot.cap;
-    for (int b = 0; b < B; ++b) h[b] = v[b];
-    CK(cudaMemcpyAsync(dst, h, B * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    return MFEM_OK;
-}
-
-mfem_status upload_alpha(mfem_ctx* c, int B) { return upload_doubles(c, B, c->alpha_host, c->slot.alpha); }
-
-mfem_status upload_ints(mfem_ctx* c, int B, const int* v, int* dst) {
-    int pos = 0;
-    mfem_status st = next_stage(c, pos);
-    if (st != MFEM_OK) return st;
-    int* h = c->active_host + (size_t)pos * c->slot.cap;
-    for (int b = 0; b < B; ++b) h[b] = v[b];
-    CK(cudaMemcpyAsync(dst, h, B * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    const size_t cap = c->slot.cap;
+    char* h = c->ctl_ring + (size_t)pos * ctl_bytes(cap);
+    int* flag = reinterpret_cast<int*>(h);
+    for (size_t b = 0; b < (rest ? cap : (size_t)B); ++b) flag[b] = (int)b < B ? flags[b] : 0;
+    if (rest) {
+        std::memcpy(flag + cap, c->coarse_host.data(), cap * sizeof(int));
+        std::memcpy(flag + 2 * cap, c->alpha_host.data(), cap * sizeof(double));
+        std::memcpy(flag + 4 * cap, c->tol2_host.data(), cap * sizeof(double));
+    }
+    CK(cudaMemcpyAsync(c->slot.active, h, rest ? ctl_bytes(cap) : B * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     return MFEM_OK;
 }
 
@@ -540,7 +528,7 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
 
 template <typename T>
 mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, int split, int max_iters, bool count,
-                    bool one_chunk = false, bool slopes = false, bool per_request = false) {
+                    bool one_chunk = false, bool slopes = false, bool per_request = false, bool* ahead = nullptr) {
     mfem_ctx* c = c0;
     std::vector<PcgDesc<T>> d;
     std::vector<CoarseJob> jobs;
@@ -607,10 +595,10 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
         chunk = std::min(kPcgChunkMax, std::max(per_request ? kPcgChunkMin : 8, (best + 7) / 8 * 8));
         // resident: every problem of a batch call runs to its own end (none waits
         // for another inside the launch); served requests keep the round's length
-        if (resident && !per_request) chunk = cap;
+        if (resident && !per_request) chunk = cap + 1;   // (the cap itself is seen one product later)
     }
     for (int done = 0; done < cap; done += chunk) {
-        const int n_it = std::min(chunk, cap - done);
+        const int n_it = resident ? chunk : std::min(chunk, cap - done);
         if (one_chunk && done > 0) break;
         if (one_chunk)
             for (auto& g : gs)
@@ -677,6 +665,15 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
                 gc->prof.end(pl, c->stream);
                 gc->prof.launches++;
             }
+        // a batch's resident solves end inside the launch, whatever their results:
+        // the step is taken and the next element pass enqueued before they are read
+        // (one host round trip a Newton step instead of two)
+        if (resident && !per_request && ahead) {
+            *ahead = true;
+            c->ahead_jobs = nj;
+            c->ahead_bytes = coarse_bytes;
+            return MFEM_OK;
+        }
         bool any = false;
         int ran = 0;
         for (auto& g : gs)
@@ -812,9 +809,7 @@ mfem_status backtrack(std::vector<Group>& gs, Group& g, std::vector<int> testing
     cudaStream_t s = gc->stream;
     bool any = any_of(testing);
     for (int k = k_first; any && k <= kLsMax; ++k) {
-        mfem_status st = upload_active(gc, g.B, testing);
-        if (st != MFEM_OK) return st;
-        st = upload_alpha(gc, g.B);
+        mfem_status st = upload_active(gc, g.B, testing, true);
         if (st != MFEM_OK) return st;
         int pl = gc->prof.begin(3, s);
         launch_energy_trial(elem_args(gc), g.B, s);
@@ -869,9 +864,7 @@ mfem_status check_speculative(std::vector<Group>& gs, Group& g, std::vector<int>
     if (!any) return MFEM_OK;
     mfem_status st = backtrack(gs, g, rejected, e0, slope, 1);
     if (st != MFEM_OK) return st;
-    st = upload_active(gc, g.B, rejected);
-    if (st != MFEM_OK) return st;
-    st = upload_alpha(gc, g.B);
+    st = upload_active(gc, g.B, rejected, true);
     if (st != MFEM_OK) return st;
     launch_update(elem_args(gc), g.B, gc->stream);
     gc->prof.launches++;
@@ -879,6 +872,15 @@ mfem_status check_speculative(std::vector<Group>& gs, Group& g, std::vector<int>
 }
 
 }  // namespace
+
+// Accounts of problem b's PCG solve (scalars in sc_host) of Newton step `it`.
+static void finish_pcg(mfem_ctx* gc, int b, ProbHost& p, int it) {
+    const int iter = gc->sc_host[b].iter;
+    p.pcg_iters += iter;
+    gc->pcg_hist[(size_t)b * kPcgHistSteps + std::min(it, kPcgHistSteps - 1)] = std::max(1, iter);
+    gc->prof.pcg_iters += iter;
+    gc->prof.pcg_bytes += iter * pcg_bytes_per_iter(gc, p.coarse);
+}
 
 mfem_status advance(std::vector<Group>& gs, bool per_request) {
     mfem_ctx* c = gs[0].ctx;
@@ -916,23 +918,17 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
         }
         st = upload_active(gc, g.B, f);
         if (st != MFEM_OK) return st;
-        std::vector<double> gref(g.B, -1.0);
         const size_t xbytes = sizeof(double) * 3 * (size_t)gc->plan.n * g.B;
         bool parked = false;
         if (need_ref) {   // reference gradient at the rigid guess
             for (int b = 0; b < g.B; ++b) parked |= start[b] == 2;
             if (parked) CK(cudaMemcpyAsync(gc->slot.outbuf, gc->slot.x, xbytes, cudaMemcpyDeviceToDevice, s));
             ElemArgs a = elem_args(gc);
+            a.ref = 1;   // |g|^2 -> gref2, read back with the first element pass
             launch_pose_init(a, g.B, 0, s);
             launch_element(a, g.B, s, false);   // forces only: the reference needs no Hessian
             launch_gradient(a, g.B, s);
             gc->prof.launches += 3;
-            st = read_scalars(gc, g.B);
-            if (st != MFEM_OK) return st;
-            CK(cudaStreamSynchronize(s));
-            synced(gs);
-            for (int b = 0; b < g.B; ++b)
-                if (f[b]) gref[b] = std::sqrt(gc->sc_host[b].gnorm2);
             if (parked) CK(cudaMemcpyAsync(gc->slot.x, gc->slot.outbuf, xbytes, cudaMemcpyDeviceToDevice, s));
         }
         for (int code = 0; code < 3; ++code) {   // apply the starts (pins on their targets)
@@ -951,7 +947,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 p.active = 1;
                 p.pred = pred[b];
                 p.corr = corr[b];
-                p.g0 = gref[b];
+                p.ref_pend = need_ref;
             }
     }
     // ---- a1-a4: element pass, assembly and gradient for problems that need it
@@ -999,9 +995,28 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
     if (any_elem) {
         CK(cudaStreamSynchronize(s));
         synced(gs);
+        int ran = 0;   // iterations of the resident solves read back now
         for (auto& g : gs) {
             mfem_ctx* gc = g.ctx;
             std::vector<int> start(g.B, 0), redo;
+            for (int b = 0; b < g.B; ++b) {
+                ProbHost& p = g.ph[b];
+                if (!p.active || p.in_pcg) continue;
+                if (p.ref_pend) {
+                    p.g0 = std::sqrt(gc->sc_host[b].gref2);
+                    p.ref_pend = 0;
+                }
+                // a resident solve whose step was taken before its result was read
+                if (p.pend) {
+                    p.pend = 0;
+                    if (gc->sc_host[b].state == kFault)
+                        return ctx_fail(c, MFEM_ECUDA, "PCG: a bounded wait in the resident kernel ran out");
+                    finish_pcg(gc, b, p, p.it - 1);
+                    ran = std::max(ran, gc->sc_host[b].iter);
+                    if (p.spec) p.spec_slope = gc->sc_host[b].slope;
+                    if (p.spec && !(-p.spec_slope > kLsNoise * std::fabs(p.spec_e0))) p.spec = 0;
+                }
+            }
             mfem_status sst = check_speculative(gs, g, redo);
             if (sst != MFEM_OK) return sst;
             for (int b = 0; b < g.B; ++b) {
@@ -1046,8 +1061,6 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 st = autotune_tile(c, one);
                 if (st != MFEM_OK) return st;
             }
-            mfem_status st = upload_active(gc, g.B, start);
-            if (st != MFEM_OK) return st;
             // PCG target of this Newton step: cg_tol; where the Newton model is
             // trusted -- a quadratic energy (ARAP or corot with rig rotations:
             // Newton is iterative refinement of one linear solve) or a warm start
@@ -1066,7 +1079,6 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
             // costs cold SNH poses 1.3%, which therefore keep the fixed target.
             const bool quadratic = gc->model != MFEM_SNH && gc->opt.rotation == MFEM_ROT_RIG;
             const bool trusted = quadratic || gc->opt.init == MFEM_INIT_WARM;
-            std::vector<double> t2(g.B, 0.0);
             for (int b = 0; b < g.B; ++b) {
                 ProbHost& p = g.ph[b];
                 double eta = p.pred ? std::min(gc->opt.cg_tol, kPredTol) : gc->opt.cg_tol;
@@ -1083,8 +1095,8 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                     last = need > eta;
                     eta = std::min(0.5, std::max(eta, need));
                 }
-                t2[b] = eta * eta;
                 if (start[b]) {
+                    gc->tol2_host[b] = eta * eta;
                     p.expect_conv = last;
                     if (!p.pred) {
                         p.gprev = p.gn;
@@ -1092,8 +1104,6 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                     }
                 }
             }
-            st = upload_doubles(gc, g.B, t2.data(), gc->slot.tol2);
-            if (st != MFEM_OK) return st;
             // the two-level preconditioner on every step, the co-rotational
             // predictor and a first step from the rigid guess included (measured
             // on the 200k figure, batch of 16: the predictor's PCG 85 -> 43
@@ -1104,8 +1114,9 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 ProbHost& p = g.ph[b];
                 p.coarse = gc->mesh.coarse_n > 0;
                 co[b] = p.coarse;
+                gc->coarse_host[b] = p.coarse;
             }
-            st = upload_ints(gc, g.B, co.data(), gc->slot.coarse_on);
+            mfem_status st = upload_active(gc, g.B, start, true);
             if (st != MFEM_OK) return st;
             if (any_of(co)) {   // the coarse modes' rotations for these iterates (active = start)
                 launch_agg_rotations(elem_args(gc), g.B, s);
@@ -1121,12 +1132,17 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                     g.ph[b].pcg_seen = 0;
                 }
         }
+        // counted as the streamed kernels' launch pairs
+        c->prof.pcg_launches += 2 * ran;
+        c->prof.coarse_launches += c->ahead_jobs * ran;
+        c->prof.pcg_bytes += c->ahead_bytes * ran;
     }
     // ---- a5: one chunk of PCG iterations over every problem inside PCG
     bool any_pcg = false;
     for (auto& g : gs)
         for (int b = 0; b < g.B; ++b) any_pcg |= g.ph[b].active && g.ph[b].in_pcg;
     if (!any_pcg) return MFEM_OK;
+    bool ahead[2] = {false, false};   // per precision: the solves run to their ends unread (see run_pcg)
     for (int prec = 0; prec < 2; ++prec) {
         bool any = false;
         for (auto& g : gs)
@@ -1134,9 +1150,9 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 for (int b = 0; b < g.B; ++b) any |= g.ph[b].active && g.ph[b].in_pcg;
         if (!any) continue;
         mfem_status st = prec == 1 ? run_pcg<float>(c, gs, 1, c->tile_rows, c->spmv_split, 0, true, true, true,
-                                                    per_request)
+                                                    per_request, &ahead[prec])
                                    : run_pcg<double>(c, gs, 0, c->tile_rows, c->spmv_split, 0, true, true, true,
-                                                     per_request);
+                                                     per_request, &ahead[prec]);
         if (st != MFEM_OK) return st;
     }
     CK(cudaGetLastError());
@@ -1148,14 +1164,12 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
         fin[gi].assign(g.B, 0);
         for (int b = 0; b < g.B; ++b) {
             ProbHost& p = g.ph[b];
-            if (p.active && p.in_pcg && g.ctx->sc_host[b].state != kActive) {
+            const bool unread = ahead[g.ctx->slot.prec];
+            if (p.active && p.in_pcg && (unread || g.ctx->sc_host[b].state != kActive)) {
                 fin[gi][b] = 1;
                 any_fin = true;
-                p.pcg_iters += g.ctx->sc_host[b].iter;
-                g.ctx->pcg_hist[(size_t)b * kPcgHistSteps + std::min(p.it, kPcgHistSteps - 1)] =
-                    std::max(1, g.ctx->sc_host[b].iter);
-                g.ctx->prof.pcg_iters += g.ctx->sc_host[b].iter;
-                g.ctx->prof.pcg_bytes += g.ctx->sc_host[b].iter * pcg_bytes_per_iter(g.ctx, p.coarse);
+                p.pend = unread;
+                if (!unread) finish_pcg(g.ctx, b, p, p.it);
                 g.ctx->alpha_host[b] = 1.0;
             }
         }
@@ -1185,7 +1199,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
             if (!ls[gi][b]) continue;
             ProbHost& p = g.ph[b];
             const double e0 = p.energy, slope = gc->sc_host[b].slope;
-            if (!(-slope > kLsNoise * std::fabs(e0))) continue;
+            if (!p.pend && !(-slope > kLsNoise * std::fabs(e0))) continue;   // unread: tested with the result
             p.spec = 1;
             p.spec_e0 = e0;
             p.spec_slope = slope;
@@ -1198,9 +1212,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
         Group& g = gs[gi];
         if (!any_of(fin[gi])) continue;
         mfem_ctx* gc = g.ctx;
-        mfem_status st = upload_active(gc, g.B, fin[gi]);
-        if (st != MFEM_OK) return st;
-        st = upload_alpha(gc, g.B);
+        mfem_status st = upload_active(gc, g.B, fin[gi], true);
         if (st != MFEM_OK) return st;
         launch_update(elem_args(gc), g.B, s);
         gc->prof.launches++;
@@ -1384,7 +1396,7 @@ void mfem_destroy(mfem_ctx* c) {
                     M.crel, M.agg_handle, M.Ainv, M.Abf, M.coarse_err, c->descs_dev, c->diag_dev, c->fext_dev};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    void* hp[] = {c->sc_host, c->active_host, c->alpha_host, c->alpha_ring, c->descs_host,
+    void* hp[] = {c->sc_host, c->ctl_ring, c->descs_host,
                   c->diag_host, c->cerr_host};
     for (void* p : hp)
         if (p) cudaFreeHost(p);

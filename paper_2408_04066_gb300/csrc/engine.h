@@ -40,6 +40,8 @@ struct ProbHost {
     double spec_e0 = 0.0, spec_slope = 0.0;
     int pcg_launched = 0;   // PCG iterations launched in the current solve
     int pcg_seen = 0;       // its iteration count at the last readback
+    int pend = 0;           // its result is still to be read (resident solve, step already taken)
+    int ref_pend = 0;       // the reference gradient is still to be read
 };
 
 // Profile accumulator with a pool of CUDA events on the context stream.
@@ -83,9 +85,9 @@ struct mfem_ctx {
     // region is never rewritten before its copy has run; the ring restarts after
     // every stream synchronisation.
     mfem::ProbScal* sc_host = nullptr;
-    int* active_host = nullptr;      // [kStageRing][cap]
-    double* alpha_host = nullptr;    // current step lengths [cap]
-    double* alpha_ring = nullptr;    // [kStageRing][cap]
+    char* ctl_ring = nullptr;        // [kStageRing] control blocks
+    std::vector<double> alpha_host, tol2_host;   // current step lengths and squared PCG targets [cap]
+    std::vector<int> coarse_host;    // two-level preconditioner in the current PCG solve [cap]
     int ring_pos = 0;
     void* descs_host = nullptr;
     unsigned* diag_dev = nullptr;
@@ -108,6 +110,8 @@ struct mfem_ctx {
     mfem::Profiler prof;
     // PCG chunks captured as CUDA graphs, keyed by the launch parameters
     std::map<std::string, cudaGraphExec_t> graphs;
+    int ahead_jobs = 0;          // coarse jobs and bytes an iteration of the resident solve not read yet
+    double ahead_bytes = 0.0;
     bool graphs_off = false;   // capture failed once (e.g. a stream that cannot capture)
     mfem::ResLimits res_lim;   // what the device holds of the resident PCG kernel (sms = 0: not used)
     mfem_profile last_profile{};

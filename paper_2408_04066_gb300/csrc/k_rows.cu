@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kRowTile) k_gradient(ElemArgs A) {
     double tot[1];
     double* part = A.slot.part + (size_t)b * A.slot.part_tiles * 4;
     if (tile_commit<1>(gn, part, blockIdx.x, gridDim.x, &A.slot.sc[b].tk_g, 0, tot) && threadIdx.x == 0)
-        A.slot.sc[b].gnorm2 = tot[0];
+        (A.ref ? A.slot.sc[b].gref2 : A.slot.sc[b].gnorm2) = tot[0];
 }
 
 template <typename T>

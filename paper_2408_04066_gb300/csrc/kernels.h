@@ -95,6 +95,7 @@ struct ElemArgs {
     int64_t fext_stride = 0;       // doubles between problems' force fields (0: one shared field)
     int rot_polar = 0;             // 1: R_k = rotation factor of F_k (co-rotational FEM), else the rig's
     int f32_forces = 0;            // mixed path: element forces formed in FP32 from the FP64 stress
+    int ref = 0;                   // gradient pass of the reference: |g|^2 goes to gref2
     int ff_elem = 0;               // mixed path: F, S, stress and energy in float-float arithmetic (xff)
 };
 // The mixed path forms element forces in FP32 when the Newton stop test is at
