@@ -9,8 +9,8 @@
 //   * A cluster of kFuSplit CTAs owns a row block of kFuAggsBlk aggregates
 //     (their 6 kFuAggsBlk rows of A_c^{-1}, padded to the MMA's M = 128); CTA q
 //     of the cluster streams the q-th part of the K range: per chunk of kTcKC
-//     columns one 32 KB block of A (packed at set-up in the MMA's no-swizzle
-//     K-major core-matrix layout) and the matching 12 KB chunk of the B
+//     columns one 32 KB block of A (packed at set-up in the MMA's 128-byte-swizzled
+//     K-major layout) and the matching 12 KB chunk of the B
 //     operand, by 1-D bulk copies (the TMA engine) into a ring of kFuStages
 //     shared-memory stages; one thread issues the MMAs (M = 128, N = 48,
 //     K = 16), FP32 accumulation in tensor memory.
@@ -66,13 +66,6 @@ static_assert(kTcM * kTcN * 4 <= kFuStage, "the partial product fits one stage f
 static_assert(kFuChunkA % 16 == 0 && kFuChunkB % 16 == 0 && kFuStage % 1024 == 0, "bulk copies: 16-byte units");
 static_assert(kFuThreads >= 128, "warps 0-3 read the 128 TMEM lanes");
 
-// Element (row, k) of a row block's chunk (bf16 elements): K step s, K-core j2,
-// 8-row group g, row r in the group.
-__host__ __device__ __forceinline__ size_t a_offset(int row, int kk) {
-    const int s = kk >> 4, j2 = (kk >> 3) & 1, c = kk & 7, g = row >> 3, r = row & 7;
-    return (size_t)s * (kTcM * 16) + (size_t)(g * 2 + j2) * 64 + r * 8 + c;
-}
-
 // Set-up: FP32 A_c^{-1} (rows of ld floats) -> per row block and chunk, BF16.
 __global__ void k_coarse_pack_bf16(const float* __restrict__ Ainv, int N, int ld, int nkc,
                                    __nv_bfloat16* __restrict__ out) {
@@ -81,7 +74,7 @@ __global__ void k_coarse_pack_bf16(const float* __restrict__ Ainv, int N, int ld
     const int ch = blockIdx.z;
     const int row = rb * 6 * kFuAggsBlk + r, k = ch * kTcKC + kk;
     const float v = (r < 6 * kFuAggsBlk && row < N && k < N) ? Ainv[(size_t)row * ld + k] : 0.f;
-    out[((size_t)rb * nkc + ch) * (kFuChunkA / 2) + a_offset(r, kk)] = __float2bfloat16_rn(v);
+    out[((size_t)rb * nkc + ch) * (kFuChunkA / 2) + a_piece(r, kk >> 3) / 2 + (kk & 7)] = __float2bfloat16_rn(v);
 }
 
 // mfem_coarse_apply: r_c of B problems (rows of ldr floats) -> their B operand.
@@ -246,7 +239,7 @@ __global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
             tc_fence_after();
             const uint32_t a0 = base + s * kFuStage, b0 = a0 + kFuChunkA;
             for (int k = 0; k < kTcSteps; ++k)
-                umma_bf16(tmem, umma_desc(a0 + k * kFuStepA, 128, 256), umma_desc(b0 + k * kFuStepB, 128, 256), idesc,
+                umma_bf16(tmem, umma_desc_sw128(a0 + a_step(k)), umma_desc(b0 + k * kFuStepB, 128, 256), idesc,
                           (c > 0 || k > 0) ? 1u : 0u);
             umma_commit(&empty[s]);
             // refill the stage of the previous chunk (its MMAs were issued one

@@ -325,11 +325,11 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         int i = 0;
         for (int cu = rank; cu < n_cu; cu += G)
             for (int c = 0, nch = chunks_of(cu); c < nch && i < n_tm; ++c, ++i) {
-                const unsigned char* src = chunk_ptr(cu, c) + (arow >> 3) * 256 + (arow & 7) * 16;
+                const unsigned char* src = chunk_ptr(cu, c);
 #pragma unroll 4
                 for (int k = warp >> 2; k < kTcSteps; k += kThreads / 128) {
-                    const uint4 x = __ldg(reinterpret_cast<const uint4*>(src + k * kFuStepA));
-                    const uint4 y = __ldg(reinterpret_cast<const uint4*>(src + k * kFuStepA + 128));
+                    const uint4 x = __ldg(reinterpret_cast<const uint4*>(src + a_piece(arow, 2 * k)));
+                    const uint4 y = __ldg(reinterpret_cast<const uint4*>(src + a_piece(arow, 2 * k + 1)));
                     tmem_st8(tmem + lane0 + kResTmemD + i * kResTmemChunk + 8 * k, x, y);
                 }
             }
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                         const uint32_t a0 = a_base + s * kFuChunkA;
 #pragma unroll
                         for (int k = 0; k < kTcSteps; ++k)
-                            umma_bf16(tmem, umma_desc(a0 + k * kFuStepA, 128, 256),
+                            umma_bf16(tmem, umma_desc_sw128(a0 + a_step(k)),
                                       umma_desc(b0 + k * kResStepB, 128, 256), idesc, (c > 0 || k > 0) ? 1u : 0u);
                         if (keep) continue;
                         umma_commit(&S.empty[s]);

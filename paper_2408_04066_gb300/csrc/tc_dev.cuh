@@ -90,6 +90,22 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lead, uint
     return d;
 }
 
+// Descriptor of a 128-byte-swizzled K-major operand (rows of 128 bytes, 1024-byte
+// aligned 8-row atoms 1024 bytes apart; within a row the 16-byte pieces are permuted
+// by piece ^ (row mod 8)): A_c^{-1}.  A K step of 16 columns is 32 bytes further.
+// An MMA (M = 128, N = 16 or 48) whose A is not swizzled waits for its A operand:
+// 165 cycles an instruction.
+__device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t addr) {
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+// Byte offset of K step k (16 columns) of a chunk's A
+__host__ __device__ __forceinline__ uint32_t a_step(int k) { return (uint32_t)(k >> 2) * (kTcM * 128) + (k & 3) * 32; }
+// Byte offset of 16-byte piece j (columns 8 j .. 8 j + 7) of row `row` of a chunk's A
+__host__ __device__ __forceinline__ uint32_t a_piece(int row, int j) {
+    return (uint32_t)(j >> 3) * (kTcM * 128) + row * 128 + (((j & 7) ^ (row & 7)) << 4);
+}
+
 // Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
 // K-major, N and M as given.
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
