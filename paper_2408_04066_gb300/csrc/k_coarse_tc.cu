@@ -144,6 +144,7 @@ __global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
     __shared__ float es[6 * kFuAggsCta][kTcProbs + 1];
     __shared__ float qs[kFuAggsCta][kTcProbs][9];
     __shared__ int any, s_ok;
+    constexpr bool kEarly = ST != kFuStagesMulti;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const uint32_t q = cluster_rank();
     const int cid = blockIdx.x / kFuSplit;   // cluster
@@ -164,19 +165,9 @@ __global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
     const unsigned char* gB =
         reinterpret_cast<const unsigned char*>(Bs) + ((size_t)pg * nkc + c_lo) * kFuChunkB;
     const int a_cta = kFuAggsBlk * rb + kFuAggsCta * (int)q;   // first aggregate this CTA corrects
-    // prologue on data fixed during the solve, overlapping the previous kernel:
-    // the slots' descriptors and aggregate rotations, and the first chunks of
-    // A_c^{-1} (their barriers also expect the B chunk, copied after the wait)
-    if (t < kTcProbs) {
-        const int slot = pg * kTcProbs + t;
-        const PcgDesc<T>* mine = nullptr;
-#pragma unroll 8
-        for (int i = 0; i < nd; ++i) {   // independent loads: no early exit
-            const bool hit = D[d0 + i].bslot == slot && D[d0 + i].coarse;
-            if (hit && !mine) mine = &D[d0 + i];
-        }
-        dp[t] = mine;
-    }
+    // set-up: barriers, the first chunks of A_c^{-1} (their barriers also expect
+    // the B chunk, copied after the wait), tensor memory for the 128 x 48 FP32
+    // accumulator
     if (t == 0) {
         any = 0;
         s_ok = 1;
@@ -188,44 +179,46 @@ __global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
             bulk_g2s(smem + c * kFuStage, gA + (size_t)c * kFuChunkA, kFuChunkA, &full[c]);
         }
     }
-    __syncthreads();
-    for (int i = t; i < kFuAggsCta * kTcProbs * 9; i += kFuThreads) {
-        const int ai = i / (kTcProbs * 9), p = (i / 9) % kTcProbs, e = i % 9;
-        const PcgDesc<T>* d = dp[p];
-        const int a = a_cta + ai;
-        qs[ai][p][e] = (d && d->aggq && a < N / 6) ? d->aggq[9 * a + e] : 0.f;
-    }
-    pdl_wait();
-    pdl_trigger();
-    if (t == 0)   // B chunks of the first stages: written by the previous kernel
-        for (int c = 0; c < nst; ++c)
-            bulk_g2s(smem + c * kFuStage + kFuChunkA, gB + (size_t)c * kFuChunkB, kFuChunkB, &full[c]);
-    __syncthreads();
-    if (t < kTcProbs) {
-        const PcgDesc<T>* d = dp[t];
-        if (d && d->sc->state != kActive) d = nullptr;
-        dp[t] = d;
-        if (d) atomicOr(&any, 1);
-    }
-    __syncthreads();
-    // the same for every CTA of the cluster (same slots, states final after the wait)
-    if (!any) {   // nothing to compute; let the copies land before the memory is released
-        if (t == 0)
-            for (int c = 0; c < nst; ++c)
-                if (!mbar_wait(&full[c], 0)) atomicOr(err, 4u);
-        return;
-    }
-    if (warp == 0) {   // tensor memory for the 128 x 48 FP32 accumulator
+    if (t < kTcProbs) dp[t] = nullptr;
+    if (warp == kFuThreads / 32 - 1) {
         __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                      "r"(kTcTmemCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    __syncthreads();
+    pdl_wait();
+    pdl_trigger();
+    if (t == 0)   // B chunks of the first stages: written by the previous kernel
+        for (int c = 0; c < nst; ++c)
+            bulk_g2s(smem + c * kFuStage + kFuChunkA, gB + (size_t)c * kFuChunkB, kFuChunkB, &full[c]);
+    // the group's problems by slot, meanwhile: a thread per descriptor
+    if (warp == 1)
+        for (int i = lane; i < nd; i += 32) {
+            const PcgDesc<T>* d = &D[d0 + i];
+            const int p = d->bslot - pg * kTcProbs;
+            if (d->coarse && d->sc->state == kActive && p >= 0 && p < kTcProbs) {
+                dp[p] = d;
+                any = 1;
+            }
+        }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
+    // the same for every CTA of the cluster (same slots, states final after the wait)
+    if (!any) {   // nothing to compute; let the copies land before the memory is released
+        if (t == 0)
+            for (int c = 0; c < nst; ++c)
+                if (!mbar_wait(&full[c], 0)) atomicOr(err, 4u);
+        if (warp == 0) {
+            __syncwarp();
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols)
+                         : "memory");
+        }
+        return;
+    }
 
     if (t == 0) {   // one thread issues every MMA and keeps the ring full
         constexpr uint32_t idesc = umma_idesc_bf16(kTcM, kTcN);
@@ -265,6 +258,31 @@ __global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
                 if (c >= 0) mbar_wait(&full[c % ST], (uint32_t)(c / ST) & 1u);
         }
     }
+    // the other warps meanwhile: the aggregates' rotations, and zb and the rest
+    // offset of the thread's first vertex row (every load that the correction
+    // needs but the product; the two-CTA variant has no registers for them)
+    const PcgDesc<T>* d0p = nullptr;
+    for (int p = 0; p < kTcProbs && !d0p; ++p) d0p = dp[p];
+    const int shift = d0p->agg_shift, n = d0p->n_rows, n_agg = N / 6;
+    const int row0 = a_cta << shift;
+    const int row1 = e_out ? row0 : min(n, min(n_agg, a_cta + kFuAggsCta) << shift);
+    const float4* crel = d0p->crel;
+    const size_t np = npad32(n);
+    float4 off0 = make_float4(0.f, 0.f, 0.f, 0.f);
+    T z0[kTcProbs][3];
+    if (kEarly && row0 + t < row1) {
+        off0 = crel[row0 + t];
+#pragma unroll
+        for (int p = 0; p < kTcProbs; ++p)
+            if (dp[p]) ld3((const T*)dp[p]->rec, np, kRecZB, row0 + t, z0[p]);
+    }
+    if (t >= 32)
+        for (int i = t - 32; i < kFuAggsCta * kTcProbs * 9; i += kFuThreads - 32) {
+            const int ai = i / (kTcProbs * 9), p = (i / 9) % kTcProbs, e = i % 9;
+            const PcgDesc<T>* d = dp[p];
+            const int a = a_cta + ai;
+            qs[ai][p][e] = (d && d->aggq && a < N / 6) ? d->aggq[9 * a + e] : 0.f;
+        }
     const bool fin = mbar_wait(done, 0);
     tc_fence_after();
     const int all_done = __syncthreads_and(fin ? 1 : 0);
@@ -319,23 +337,19 @@ __global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
         return;
     }
     // correction of the aggregates' vertex rows for every problem of the group
-    const PcgDesc<T>* d0p = nullptr;
-    for (int p = 0; p < kTcProbs && !d0p; ++p) d0p = dp[p];
-    const int shift = d0p->agg_shift, n = d0p->n_rows, n_agg = N / 6;
-    const int row0 = a_cta << shift;
-    const int row1 = min(n, min(n_agg, a_cta + kFuAggsCta) << shift);
-    const float4* crel = d0p->crel;
     for (int row = row0 + t; row < row1; row += kFuThreads) {
-        const float4 off = crel[row];
+        const bool early = kEarly && row == row0 + t;
+        const float4 off = early ? off0 : crel[row];
         const int ai = (row >> shift) - a_cta;
-        T z[kTcProbs][3];
+        if (!early)
 #pragma unroll
-        for (int p = 0; p < kTcProbs; ++p)
-            if (dp[p]) ld3((const T*)dp[p]->rec, npad32(n), kRecZB, row, z[p]);
+            for (int p = 0; p < kTcProbs; ++p)
+                if (dp[p]) ld3((const T*)dp[p]->rec, np, kRecZB, row, z0[p]);
 #pragma unroll
         for (int p = 0; p < kTcProbs; ++p) {
             const PcgDesc<T>* d = dp[p];
             if (!d) continue;
+            T z[3] = {z0[p][0], z0[p][1], z0[p][2]};
             if (off.w != 0.f) {
                 const float e0 = es[6 * ai][p], e1 = es[6 * ai + 1][p], e2 = es[6 * ai + 2][p];
                 const float e3 = es[6 * ai + 3][p], e4 = es[6 * ai + 4][p], e5 = es[6 * ai + 5][p];
@@ -344,9 +358,9 @@ __global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
                 const float l2 = e2 + (e3 * off.y - e4 * off.x);
                 const float* Q = qs[ai][p];
 #pragma unroll
-                for (int i = 0; i < 3; ++i) z[p][i] += (T)(Q[3 * i] * l0 + Q[3 * i + 1] * l1 + Q[3 * i + 2] * l2);
+                for (int i = 0; i < 3; ++i) z[i] += (T)(Q[3 * i] * l0 + Q[3 * i + 1] * l1 + Q[3 * i + 2] * l2);
             }
-            stv(d->nb + 4 * (size_t)row, z[p]);
+            stv(d->nb + 4 * (size_t)row, z);
         }
     }
 }
