@@ -72,6 +72,7 @@ struct ProbScal {
     double rho, alpha, beta, rr0, rr, tol2;   // rho: the last (r, u); alpha, beta: the next step's
     double gnorm2, energy, slope, energy_trial;
     double gref2, pad0;   // |g_free|^2 at the rigid guess
+    double inv_rho, inv_alpha;   // FP32 path: 1 / rho and 1 / alpha, formed beside the update
     float alpha_f, beta_f;   // FP32 copies of alpha and beta for the FP32 kernels
     int iter, state, maxit, active;
     unsigned tk_a, tk_b, tk_g, tk_e, tk_s, tk_init, tk_c;

@@ -183,14 +183,18 @@ __device__ __forceinline__ int unit_problem(const PcgDesc<T>* __restrict__ D, in
 // The end of an SpMV block of NT threads: tile partials (v: the warp's sums, value
 // i in lane i) and, in the problem's last block, the totals, the convergence test
 // and the next step's coefficients.
+//
+// The last block's part is a serial tail of every iteration: an FP64 instruction
+// takes a scheduler 64 cycles, a division some 20 of them, an L2 round trip ~1200.
+// So the sums over warps are formed by three threads, a value each, instead of
+// shuffle trees over empty lanes (200k figure, 16 poses: 117.8 -> 114.0 us an
+// iteration); FP32 takes its totals with a warp per value, the scalars are
+// loaded before they are needed, and two of its three divisions are the update's
+// (inv_rho, inv_alpha).  FP64 keeps the order of its sums and its divisions, which
+// its results show.
 template <typename T, int NT>
 __device__ __forceinline__ void spmv_commit(const PcgDesc<T>& d, ProbScal* sc, int tile, double v) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // tile partials and, in the problem's last block, the totals: the sums over
-    // the block's warps by three threads, a value each.  An FP64 instruction takes
-    // a scheduler 64 cycles, and a shuffle tree over the block's warps spends five
-    // levels of them on lanes that hold nothing (200k figure, 16 poses, 128-row
-    // tiles: 117.8 -> 114.0 us an iteration, 800k figure, 4 poses: 90.5 -> 87.1)
     constexpr int NW = NT / 32;
     __shared__ double sm[NW * 3];
     __shared__ int s_last;
@@ -207,43 +211,65 @@ __device__ __forceinline__ void spmv_commit(const PcgDesc<T>& d, ProbScal* sc, i
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (int x = threadIdx.x; x < d.n_tiles; x += NT)
+    ProbScal q;   // thread 0: what the coefficients need
+    if (threadIdx.x == 0) {
+        q.tol2 = sc->tol2;
+        q.rr0 = sc->rr0;
+        q.iter = sc->iter;
+        q.maxit = sc->maxit;
+        q.first = sc->first;
+        q.rho = sc->rho;
+        q.alpha = sc->alpha;
+        q.inv_rho = sc->inv_rho;
+        q.inv_alpha = sc->inv_alpha;
+    }
+    if (sizeof(T) == 4 && NW >= 4) {
+        if (warp < 3) {   // warp i: value i
+            double s = 0.0;
+#pragma unroll 4
+            for (int x = lane; x < d.n_tiles; x += 32) s += *(volatile double*)&d.part[4 * x + warp];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) acc[i] += *(volatile double*)&d.part[4 * x + i];
-    const double tv = warp_sums3(Partial<double>{acc[0]}, Partial<double>{acc[1]}, Partial<double>{acc[2]});
-    if (lane < 3) sm[3 * warp + lane] = tv;
-    __syncthreads();
-    if (threadIdx.x < 3) sm[threadIdx.x] = warps_sum<NW>(sm + threadIdx.x);   // thread i reads and writes column i
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) sm[warp] = s;
+        }
+    } else {
+        double acc[3] = {0.0, 0.0, 0.0};
+        for (int x = threadIdx.x; x < d.n_tiles; x += NT)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) acc[i] += *(volatile double*)&d.part[4 * x + i];
+        const double tv = warp_sums3(Partial<double>{acc[0]}, Partial<double>{acc[1]}, Partial<double>{acc[2]});
+        if (lane < 3) sm[3 * warp + lane] = tv;
+        __syncthreads();
+        if (threadIdx.x < 3) sm[threadIdx.x] = warps_sum<NW>(sm + threadIdx.x);   // thread i reads and writes column i
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        const double tot[3] = {sm[0], sm[1], sm[2]};
+        const double gamma = sm[0], delta = sm[1], rr = sm[2];
         sc->tk_a = 0u;
-        const double gamma = tot[0], delta = tot[1];
-        sc->rr = tot[2];
-        if (!(tot[2] > sc->tol2 * sc->rr0)) {   // |r| at target: dx is the solve's result
+        sc->rr = rr;
+        if (!(rr > q.tol2 * q.rr0)) {   // |r| at target: dx is the solve's result
             sc->state = kConverged;
-        } else if (sc->iter >= sc->maxit) {
+        } else if (q.iter >= q.maxit) {
             sc->state = kMaxIter;
         } else {
-            double beta = 0.0, den = delta;
-            if (!sc->first) {
-                beta = gamma / sc->rho;
-                den = delta - beta * gamma / sc->alpha;
+            double beta = 0.0, den = delta, alpha = 0.0;
+            if (!q.first) {
+                beta = sizeof(T) == 4 ? gamma * q.inv_rho : gamma / q.rho;
+                den = sizeof(T) == 4 ? delta - beta * gamma * q.inv_alpha : delta - beta * gamma / q.alpha;
             }
             if (gamma > 0.0 && den > 0.0 && isfinite(gamma) && isfinite(den)) {
-                sc->alpha = gamma / den;
-                sc->beta = beta;
+                alpha = gamma / den;
                 sc->rho = gamma;
                 sc->first = 0;
-                sc->iter = sc->iter + 1;
+                sc->iter = q.iter + 1;
             } else {   // breakdown (u orthogonal to r, or K / M lost definiteness along u): keep dx
-                sc->alpha = 0.0;
-                sc->beta = 0.0;
+                beta = 0.0;
                 sc->state = kConverged;
             }
-            sc->alpha_f = (float)sc->alpha;
-            sc->beta_f = (float)sc->beta;
+            sc->alpha = alpha;
+            sc->beta = beta;
+            sc->alpha_f = (float)alpha;
+            sc->beta_f = (float)beta;
         }
     }
 }
@@ -420,6 +446,10 @@ __global__ void __launch_bounds__(TILE) k_pcg_update(const PcgDesc<T>* __restric
     if (sc->state != kActive) return;   // block-uniform
     T alpha, beta;
     coeffs(sc, alpha, beta);
+    if (sizeof(T) == 4 && tile == 0 && threadIdx.x == TILE - 1) {   // for the next coefficients (spmv_commit)
+        sc->inv_rho = 1.0 / sc->rho;
+        sc->inv_alpha = 1.0 / sc->alpha;
+    }
     float r32[3] = {0.f, 0.f, 0.f};
     if (row < d.n_rows) {
         const size_t np = npad32(d.n_rows);

@@ -736,6 +736,10 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
             sc->rho = S.st.rho;
             sc->alpha = S.st.alpha;
             sc->beta = S.st.beta;
+            if (sizeof(T) == 4) {
+                sc->inv_rho = S.st.inv_rho;
+                sc->inv_alpha = S.st.inv_alpha;
+            }
             sc->alpha_f = (float)S.st.alpha;
             sc->beta_f = (float)S.st.beta;
             sc->rr = S.st.rr;
