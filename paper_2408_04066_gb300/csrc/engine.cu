@@ -18,7 +18,11 @@ thread_local std::string g_thread_err = "no error";
 constexpr double kLsC = 1.0e-4;      // Armijo constant
 constexpr int kLsMax = 20;           // halvings
 constexpr double kLsNoise = 1.0e-10; // predicted decrease below this * |E|: take the step
-constexpr int kPcgTiles[3] = {64, 128, 256};   // PCG rows per block the autotuner times
+// SpMV rows per block the autotuner times.  64 (still an option) is slower with one
+// thread per row: us per launched iteration at 64 / 128 / 256 rows, 16 poses of the
+// 200k figure 71.5 / 69.5 / 69.1, 4 poses of the 800k figure 78.6 / 74.1 / 72.3.
+constexpr int kPcgTiles[2] = {128, 256};
+constexpr int kTileDefault = 256;               // until a streamed solve has been timed
 constexpr int kPcgChunk = 16;                   // PCG iterations enqueued between convergence checks (no history)
 constexpr int kPcgChunkMin = 16, kPcgChunkMax = 64;   // bounds of a predicted chunk (multiples of 8)
 constexpr int kResStages = 4;                   // 32 KB chunks of A_c^{-1} the resident kernel's ring holds
@@ -245,8 +249,8 @@ void end_profile(mfem_ctx* c) {
     P.coarse_launches = c->prof.coarse_launches;
     P.coarse_tc = c->mesh.coarse_n > 0 && c->mesh.coarse_tc ? 1 : 0;
     P.pcg_iters = c->prof.pcg_iters;
-    P.tile_rows = c->tile_rows;
-    P.spmv_split = c->spmv_split;
+    P.tile_rows = c->tile_rows ? c->tile_rows : kTileDefault;
+    P.spmv_split = c->spmv_split ? c->spmv_split : 1;
     P.grid_blocks = c->grid_blocks;
     for (int i = 0; i < c->prof.used; ++i) {
         float ms = 0.f;
@@ -524,6 +528,24 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
         at += g[i];
     }
     return true;
+}
+
+int tile_of(const mfem_ctx* c) { return c->tile_rows ? c->tile_rows : kTileDefault; }
+int split_of(const mfem_ctx* c) { return c->spmv_split ? c->spmv_split : 1; }
+
+// Whether the problems inside PCG run in the resident kernel.
+bool fits_chip(mfem_ctx* c, std::vector<Group>& gs, int tile) {
+    auto fits = [&](auto zero, int prec) {
+        using T = decltype(zero);
+        std::vector<PcgDesc<T>> d;
+        std::vector<mfem_ctx*> owner;
+        int u = 0, uu = 0;
+        build_descs<T>(gs, tile, prec, d, u, uu, nullptr, &owner);
+        ResShape sh;
+        std::vector<ResJob> jobs;
+        return d.empty() || plan_resident<T>(c, d, owner, tile, sh, jobs);
+    };
+    return fits(0.f, 1) && fits(0.0, 0);
 }
 
 template <typename T>
@@ -1053,12 +1075,21 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 start[b] = 1;
             }
             if (!any_of(start)) continue;
-            if (c->tile_rows == 0 || c->spmv_split == 0) {   // first PCG of this context: time the shapes
+            // first streamed PCG of this context: time the shapes (a resident one has
+            // none) on the problems that start now, the others' state untouched
+            if (c->tile_rows == 0 || c->spmv_split == 0) {
+                const std::vector<ProbHost> keep(g.ph, g.ph + g.B);
+                for (int b = 0; b < g.B; ++b) {
+                    g.ph[b].in_pcg = start[b];
+                    g.ph[b].coarse = gc->mesh.coarse_n > 0;
+                }
                 std::vector<Group> one{Group{gc, g.B, g.ph}};
-                for (int b = 0; b < g.B; ++b) g.ph[b].in_pcg = start[b];
-                mfem_status st = upload_active(gc, g.B, start);
-                if (st != MFEM_OK) return st;
-                st = autotune_tile(c, one);
+                mfem_status st = MFEM_OK;
+                if (per_request || !fits_chip(c, one, tile_of(c))) {
+                    st = upload_active(gc, g.B, start);
+                    if (st == MFEM_OK) st = autotune_tile(c, one);
+                }
+                std::copy(keep.begin(), keep.end(), g.ph);
                 if (st != MFEM_OK) return st;
             }
             // PCG target of this Newton step: cg_tol; where the Newton model is
@@ -1122,7 +1153,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 launch_agg_rotations(elem_args(gc), g.B, s);
                 gc->prof.launches++;
             }
-            launch_pcg_init(elem_args(gc), g.B, c->tile_rows, 0.0, gc->opt.cg_max, gc->slot.tol2,
+            launch_pcg_init(elem_args(gc), g.B, tile_of(c), 0.0, gc->opt.cg_max, gc->slot.tol2,
                             gc->slot.coarse_on, s);
             gc->prof.launches++;
             for (int b = 0; b < g.B; ++b)
@@ -1149,9 +1180,9 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
             if (g.ctx->slot.prec == prec)
                 for (int b = 0; b < g.B; ++b) any |= g.ph[b].active && g.ph[b].in_pcg;
         if (!any) continue;
-        mfem_status st = prec == 1 ? run_pcg<float>(c, gs, 1, c->tile_rows, c->spmv_split, 0, true, true, true,
+        mfem_status st = prec == 1 ? run_pcg<float>(c, gs, 1, tile_of(c), split_of(c), 0, true, true, true,
                                                     per_request, &ahead[prec])
-                                   : run_pcg<double>(c, gs, 0, c->tile_rows, c->spmv_split, 0, true, true, true,
+                                   : run_pcg<double>(c, gs, 0, tile_of(c), split_of(c), 0, true, true, true,
                                                      per_request, &ahead[prec]);
         if (st != MFEM_OK) return st;
     }
