@@ -178,9 +178,11 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], bool warp_done = fals
 #pragma unroll
         for (int i = 0; i < NV; ++i) v[i] = lane < nwarps ? sm[lane][i] : 0.0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
+        for (int o = 16; o > 0; o >>= 1) {
+            if (o >= nwarps) continue;   // lanes past the last warp hold zeros
 #pragma unroll
             for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+        }
     }
     __syncthreads();
 }

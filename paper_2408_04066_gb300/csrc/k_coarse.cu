@@ -208,10 +208,24 @@ __global__ void __launch_bounds__(32) k_agg_rotations(ElemArgs A) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) m[3 * p + q] = fma(xi[p], ri[q], m[3 * p + q]);
     }
+    // the nine warp sums by halving: at each level of the tree a lane keeps the half
+    // of the values that its bit names and adds its partner's (16 FP64 additions a
+    // warp instead of 45 -- each takes a scheduler 64 cycles -- in the tree's order)
+    double v[16];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
+    for (int e = 0; e < 16; ++e) v[e] = e < 9 ? m[e] : 0.0;
 #pragma unroll
-        for (int e = 0; e < 9; ++e) m[e] += __shfl_xor_sync(0xffffffffu, m[e], o);
+    for (int o = 16, c = 8; o > 1; o >>= 1, c >>= 1)
+#pragma unroll
+        for (int e = 0; e < c; ++e) {
+            const bool up = lane & o;
+            const double give = up ? v[e] : v[e + c], own = up ? v[e + c] : v[e];
+            v[e] = own + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    // value e is with the lanes whose bits 4..1 are e's bits 3..0
+#pragma unroll
+    for (int e = 0; e < 9; ++e) m[e] = __shfl_sync(0xffffffffu, v[0], e << 1);
     if (lane == 0) {
         const float Mm[3][3] = {{(float)m[0], (float)m[1], (float)m[2]},
                                 {(float)m[3], (float)m[4], (float)m[5]},

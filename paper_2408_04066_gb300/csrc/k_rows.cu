@@ -26,8 +26,26 @@ __device__ __forceinline__ double row_gradient(const ElemArgs& A, int b, int row
     // gradient of row: sum of element forces in fixed incidence order
     const double* ge = A.slot.ge + (size_t)b * M.m * 12;
     double g0 = 0, g1 = 0, g2 = 0;
-    for (int ii = M.vinc_ptr[row]; ii < M.vinc_ptr[row + 1]; ++ii) {
-        const int code = M.vinc[ii];
+    int ii = M.vinc_ptr[row];
+    const int i1 = M.vinc_ptr[row + 1];
+    for (; ii + 3 < i1; ii += 4) {   // four tets at a time, every load first, added in order
+        int code[4];
+        double f[4][3];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) code[q] = __ldg(M.vinc + ii + q);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) f[q][i] = __ldg(ge + (size_t)(code[q] >> 2) * 12 + 3 * (code[q] & 3) + i);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            g0 += f[q][0];
+            g1 += f[q][1];
+            g2 += f[q][2];
+        }
+    }
+    for (; ii < i1; ++ii) {
+        const int code = __ldg(M.vinc + ii);
         const double* f = ge + (size_t)(code >> 2) * 12 + 3 * (code & 3);
         g0 += f[0];
         g1 += f[1];
