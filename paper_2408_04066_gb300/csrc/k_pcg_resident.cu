@@ -719,6 +719,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         }
     }
 
+    __syncthreads();   // the reciprocals of the last coefficients
     // ---- write back: the increment; the other vectors only if the solve goes on
     if (valid) {
         st3(d.rec, np, kRecDX, row, dx[0], dx[1], dx[2]);
@@ -727,7 +728,13 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
             st3(d.rec, np, kRecP, row, pp[0], pp[1], pp[2]);
             st3(d.rec, np, kRecS, row, ss[0], ss[1], ss[2]);
             st3(d.rec, np, kRecZB, row, zb[0], zb[1], zb[2]);
+            // a served solve may go on in the streamed kernels: what their update leaves
+            if (!coarse) st4(d.nb + 4 * (size_t)row, zb[0], zb[1], zb[2]);
         }
+    }
+    if (active && d.bunit && t < 6 * nu) {   // ... the residual's B operand among it
+        const int k = 6 * u0 + t;
+        if (k < N) coarse_b_store(d.bunit, d.bslot % kCoarseGroupSlots, k, d.rcp[k]);
     }
     if (t == 0) {
         if (S.fail) {

@@ -61,3 +61,32 @@ def test_iteration_cap():
     _, st = ctx.solve_batch(np.asarray(cfg["xfs"])[:1])
     assert st[0]["newton_iters"] == 2 and st[0]["pcg_iters"] == 6
     ctx.close()
+
+
+@pytest.mark.parametrize("precond", ["two_level", "block_jacobi"])
+def test_served_requests_that_join_a_resident_solve(precond):
+    """A request alone in the server runs in the resident kernel a chunk at a time; requests
+    that arrive while it runs make the table too large, and its solve goes on in the streamed
+    kernels.  Every result still equals the same pose solved alone, bit for bit."""
+    import time
+
+    from paper_2408_04066_gb300 import mfem
+    cfg = figure_config(50000, model="corot", seeds=range(16))
+    xf = np.asarray(cfg["xfs"])
+    opts = dict(tile_rows=256, spmv_split=1, precond=precond, max_batch=16)
+    ctx = mfem.Context.from_config(cfg, **opts)
+    alone = [ctx.solve_batch(x[None])[0][0] for x in xf]
+    ctx.close()
+    srv = mfem.Server(max_slots=16)
+    mid = srv.add(mfem.Context.from_config(cfg, **opts))
+    srv.wait(srv.submit(mid, xf[0]))                          # first launches, slot pools
+    for pause_us in (300, 600, 1000, 1500, 2000, 3000):
+        tickets = [srv.submit(mid, xf[0])]
+        t = time.perf_counter()
+        while (time.perf_counter() - t) * 1e6 < pause_us:
+            pass
+        tickets += [srv.submit(mid, x) for x in xf[1:]]
+        for b, ticket in enumerate(tickets):
+            out, _, _ = srv.wait(ticket)
+            assert np.array_equal(out, alone[b]), (pause_us, b)
+    srv.close()
