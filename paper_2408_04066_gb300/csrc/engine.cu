@@ -491,7 +491,7 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
             if ((int)np > lim.clusters[k] && cl / 2 >= most) continue;
             std::vector<int> gc(np, cl);
             sh.stages = ring(gc);
-            sh.v_bytes = sh.smem - res_smem_coarse(sh.stages, sh.b_chunks);
+            sh.v_bytes = sh.smem - res_smem_coarse(sh.stages, sh.b_chunks) - res_smem_exchange(sizeof(T) == 8);
             bool fits = (int)np <= kResWaves * lim.clusters[k];
             for (size_t i = 0; i < np; ++i) fits = fits && bytes[i] <= (size_t)cl * sh.v_bytes;
             if (!fits) break;

@@ -13,8 +13,9 @@
 //   work)  |  u = zb + P e  |  w = K u, dots  |  alpha, beta; p, s, dx, r, zb,
 //   restriction  |
 //
-// A group of at most 16 CTAs is a thread-block cluster and uses the cluster
-// barrier; a larger one is part of a cooperative launch (every CTA resident) and
+// A group of at most 16 CTAs is a thread-block cluster: it uses the cluster
+// barrier, and u, r_c and the inner-product partials go through distributed shared
+// memory instead of L2.  A larger one is part of a cooperative launch (every CTA resident) and
 // counts arrivals in global memory.  Groups do not wait for one another: each
 // problem ends when it converges.
 //
@@ -96,6 +97,37 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
     for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Exchange area of a cluster's CTA, at the same offset in each: the other CTAs
+// write its copies of the inner-product partials and of r_c, and read its u.
+constexpr int kExPart = 0;                                          // [256][3] doubles, by warp of 32 rows
+constexpr int kExRc = kExPart + 256 * 3 * 8;                        // [16 kResUnits][6] floats
+constexpr int kExU = kExRc + 16 * kResUnits * 6 * 4;                // [rows of the CTA][4]
+template <typename T>
+constexpr int kExBytes = kExU + kResMaxThreads * 4 * (int)sizeof(T);
+static_assert(kExBytes<float> % 1024 == 0 && kExBytes<double> % 1024 == 0, "the A ring after it is aligned");
+
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void ld_cluster(uint32_t a, float (&q)[3]) {
+    asm volatile("{\n\t.reg .f32 w;\n\tld.shared::cluster.v4.f32 {%0, %1, %2, w}, [%3];\n\t}\n"
+                 : "=f"(q[0]), "=f"(q[1]), "=f"(q[2])
+                 : "r"(a)
+                 : "memory");
+}
+__device__ __forceinline__ void ld_cluster(uint32_t a, double (&q)[3]) {
+    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(q[0]), "=d"(q[1]) : "r"(a) : "memory");
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(q[2]) : "r"(a + 16) : "memory");
+}
+
 // eight 32-bit columns of this thread's TMEM lane
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, uint4 a, uint4 b) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(a.x),
@@ -113,13 +145,16 @@ __device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, u
         : "memory");
 }
 
-// The neighbour records of up to NB slots of a row (zero ids: none)
-template <typename T, int NB>
+// The neighbour records of up to NB slots of a row (-1: none): column ids into nb,
+// or, in a cluster, shared-memory addresses of the owning CTA's u
+template <typename T, int NB, bool CLUSTER>
 __device__ __forceinline__ void gather(const T* nb, const int (&c)[NB], T (&q)[NB][3]) {
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
         q[i][0] = q[i][1] = q[i][2] = (T)0;
-        if (c[i] >= 0) ld4(nb + 4 * (size_t)c[i], q[i]);
+        if (c[i] < 0) continue;
+        if (CLUSTER) ld_cluster((uint32_t)c[i], q[i]);
+        else ld4(nb + 4 * (size_t)c[i], q[i]);
     }
 }
 template <int NB>
@@ -182,10 +217,12 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
     const int nkc = coarse ? coarse_chunks(N) : 0, c_per = coarse ? coarse_part_chunks(N) : 1;
     const int nq = coarse ? (nkc + c_per - 1) / c_per : 0, n_cu = coarse ? row_blocks(N) * nq : 0;
     const int ld_e = coarse_ld(N);
-    unsigned char* bmem = smem + (size_t)sh.stages * kFuChunkA;
+    constexpr int kEx = CLUSTER ? kExBytes<T> : 0;
+    unsigned char* ring = smem + kEx;
+    unsigned char* bmem = ring + (size_t)sh.stages * kFuChunkA;
     const bool has_cu = rank < n_cu;
-    unsigned char* vmem = has_cu ? bmem + (size_t)sh.b_chunks * kResChunkB : smem;
-    const int v_bytes = has_cu ? sh.v_bytes : sh.smem;
+    unsigned char* vmem = has_cu ? bmem + (size_t)sh.b_chunks * kResChunkB : ring;
+    const int v_bytes = has_cu ? sh.v_bytes : sh.smem - kEx;
 
     // ---- set-up: barriers, the unit values that fit, the first chunks of A
     if (t == 0) {
@@ -251,7 +288,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
     auto load_next = [&]() {   // one more chunk into its stage (free by now)
         const int s = (int)(loaded % sh.stages);
         mbar_expect_tx(&S.full[s], kFuChunkA);
-        bulk_g2s(smem + (size_t)s * kFuChunkA, chunk_ptr(l_cu, l_c), kFuChunkA, &S.full[s]);
+        bulk_g2s(ring + (size_t)s * kFuChunkA, chunk_ptr(l_cu, l_c), kFuChunkA, &S.full[s]);
         ++loaded;
         if (++l_c >= chunks_of(l_cu)) {
             l_c = 0;
@@ -350,8 +387,49 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
     if (!mbar_wait(&S.vals, 0)) S.fail = 1;
     const bool landed = !__syncthreads_or(S.fail);
 
+    double* xpart = reinterpret_cast<double*>(smem + kExPart);   // cluster: every warp's inner products
+    float* xrc = reinterpret_cast<float*>(smem + kExRc);         // cluster: r_c by unit
+    T* xu = reinterpret_cast<T*>(smem + kExU);                   // cluster: u of this CTA's rows
+    // cluster: shared-memory address of a row's u in its CTA
+    const int q_units = n_units / G;
+    auto u_address = [&](int c) {
+        const int unit = c >> 6;
+        const int rk = unit < q_units * u_rem ? unit / max(1, q_units) : u_rem + (unit - q_units * u_rem) / (q_units + 1);
+        const int local = (unit - q_units * rk - max(0, rk - u_rem)) * kCoarseRows + (c & (kCoarseRows - 1));
+        return (int)mapa(smem_u32(xu) + local * 4 * (int)sizeof(T), rk);
+    };
+    if (CLUSTER) {
+        if (landed && in_smem)   // column ids -> addresses, once
+            for (int k = 0; k < w; ++k) {
+                int* cp = reinterpret_cast<int*>(vmem + c_at) + 32 * k;
+                if (*cp >= 0) *cp = u_address(*cp);
+            }
+        // the other CTAs' copies start from this launch's residual
+        if (coarse && has_cu)
+            for (int i = t; i < 6 * n_units; i += kThreads) xrc[i] = d.rcp[i];
+        __syncthreads();
+    }
     int c0[NB];   // the first slots' column ids
     load_cols(in_smem ? reinterpret_cast<const int*>(vmem + c_at) : cg, 0, landed ? w : 0, c0);
+    if (CLUSTER && !in_smem)
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+            if (c0[i] >= 0) c0[i] = u_address(c0[i]);
+    // a failed wait is told to every CTA of the cluster before its next barrier, so
+    // that all leave together and none reads the memory of one that has left
+    auto tell_fail = [&]() {
+        if (CLUSTER && t == 0 && S.fail)
+            for (int rk = 0; rk < G; ++rk)
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(smem_u32(&S.fail), rk)), "r"(1) : "memory");
+    };
+    if (CLUSTER) {   // every CTA of the cluster runs before the first remote access
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        tell_fail();
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    const bool go = CLUSTER ? !S.fail : landed;
 
     unsigned bar_n = 0;
     uint32_t done_ph = 0;
@@ -385,7 +463,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
     };
 
     bool active = true;
-    for (int it = 0; landed && it < sh.iters; ++it) {
+    for (int it = 0; go && it < sh.iters; ++it) {
         T u[3] = {zb[0], zb[1], zb[2]};
         if (coarse) {
             // ---- coarse product: this CTA's units
@@ -396,22 +474,23 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                 for (int g = t; g < nch * (kTcKC / 8); g += kThreads) {
                     const int k = c_lo * kTcKC + 8 * g;
                     float v[8];
+                    const float* rc = CLUSTER ? xrc : d.rcp;
                     if (ashift == 0) {
                         if (k + 7 < N) {
-                            const float4 x = *reinterpret_cast<const float4*>(d.rcp + k);
-                            const float4 y = *reinterpret_cast<const float4*>(d.rcp + k + 4);
+                            const float4 x = *reinterpret_cast<const float4*>(rc + k);
+                            const float4 y = *reinterpret_cast<const float4*>(rc + k + 4);
                             v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
                             v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
                         } else {
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) v[e] = k + e < N ? d.rcp[k + e] : 0.f;
+                            for (int e = 0; e < 8; ++e) v[e] = k + e < N ? rc[k + e] : 0.f;
                         }
                     } else {
                         for (int e = 0; e < 8; ++e) {
                             float s = 0.f;
                             if (k + e < N) {
                                 const int a = (k + e) / 6, comp = (k + e) - 6 * a, e1 = min(n_units, (a + 1) << ashift);
-                                for (int x = a << ashift; x < e1; ++x) s += d.rcp[6 * (size_t)x + comp];
+                                for (int x = a << ashift; x < e1; ++x) s += rc[6 * (size_t)x + comp];
                             }
                             v[e] = s;
                         }
@@ -444,7 +523,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                 __syncthreads();
                 if (t == 0) {
                     constexpr uint32_t idesc = umma_idesc_bf16(kTcM, 16);
-                    const uint32_t a_base = smem_u32(smem), b_base = smem_u32(bmem);
+                    const uint32_t a_base = smem_u32(ring), b_base = smem_u32(bmem);
                     tc_fence_after();
                     for (int c = 0; c < nch; ++c, ++a_at) {
                         const uint32_t b0 = b_base + c * kResChunkB;
@@ -506,6 +585,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                     }
                     load_next();
                 }
+            tell_fail();
             arrive();
             wait();
             if (S.fail) break;
@@ -532,7 +612,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                 for (int i = 0; i < 3; ++i) u[i] += (T)(Q[3 * i] * l0 + Q[3 * i + 1] * l1 + Q[3 * i + 2] * l2);
             }
         }
-        if (valid) st4(d.nb + 4 * (size_t)row, u[0], u[1], u[2]);
+        if (valid) st4(CLUSTER ? xu + 4 * t : d.nb + 4 * (size_t)row, u[0], u[1], u[2]);
         arrive();
         if (!valid) u[0] = u[1] = u[2] = 0;
         const Partial<T> d0 = dot3_partial(r[0], r[1], r[2], u[0], u[1], u[2]);
@@ -543,13 +623,13 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         T a0 = 0, a1 = 0, a2 = 0;
         {
             T q[NB][3];
-            gather<T, NB>(d.nb, c0, q);
+            gather<T, NB, CLUSTER>(d.nb, c0, q);
             if (in_smem) {
                 products<T, NB>(reinterpret_cast<const T*>(vmem + v_at), c0, q, a0, a1, a2);
                 for (int k = NB; k < w; k += NB) {
                     int c[NB];
                     load_cols(reinterpret_cast<const int*>(vmem + c_at), k, w, c);
-                    gather<T, NB>(d.nb, c, q);
+                    gather<T, NB, CLUSTER>(d.nb, c, q);
                     products<T, NB>(reinterpret_cast<const T*>(vmem + v_at) + 288 * k, c, q, a0, a1, a2);
                 }
             } else {
@@ -557,7 +637,11 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                 for (int k = NB; k < w; k += NB) {
                     int c[NB];
                     load_cols(cg, k, w, c);
-                    gather<T, NB>(d.nb, c, q);
+                    if (CLUSTER)
+#pragma unroll
+                        for (int i = 0; i < NB; ++i)
+                            if (c[i] >= 0) c[i] = u_address(c[i]);
+                    gather<T, NB, CLUSTER>(d.nb, c, q);
                     products<T, NB>(vg + 288 * (size_t)k, c, q, a0, a1, a2);
                 }
             }
@@ -572,7 +656,12 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         // warp sums: their order shows in the last bits of alpha and beta only,
         // which are rounded to FP32).  An FP64 instruction takes a scheduler 64
         // cycles, so few warps do few of them, a value each.
-        if (sizeof(T) == 8 || CLUSTER) {
+        if (CLUSTER) {   // to every CTA of the cluster
+            for (int i = t; i < 6 * nu * G; i += kThreads) {
+                const int k = i % (6 * nu), w0 = 2 * u0 + k / 3;
+                if (32 * w0 < n) st_cluster(mapa(smem_u32(xpart + 3 * w0 + k % 3), i / (6 * nu)), S.wsum[k / 3][k % 3]);
+            }
+        } else if (sizeof(T) == 8) {
             if (t < 6 * nu && 32 * (2 * u0 + t / 3) < n) d.part[4 * (size_t)(2 * u0 + t / 3) + t % 3] = S.wsum[t / 3][t % 3];
         } else if (warp < 3) {
             double x = lane < 2 * U ? S.wsum[lane & 15][warp] : 0.0;
@@ -592,7 +681,9 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                     double v[8];
 #pragma unroll
                     for (int y = 0; y < 8; ++y)
-                        v[y] = y < nw && x * nw + y < n_warps ? d.part[4 * (size_t)(x * nw + y) + i] : 0.0;
+                        v[y] = y >= nw || x * nw + y >= n_warps ? 0.0
+                               : CLUSTER                        ? xpart[3 * (x * nw + y) + i]
+                                                                : d.part[4 * (size_t)(x * nw + y) + i];
                     tot[i] += ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
                 }
             if (warp < nw) {
@@ -619,7 +710,9 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                 double x[8], s = 0.0;
 #pragma unroll
                 for (int j = 0; j < 8; ++j)   // every load first
-                    x[j] = lane + 32 * j < n_part ? d.part[4 * (size_t)(lane + 32 * j) + warp] : 0.0;
+                    x[j] = lane + 32 * j >= n_part ? 0.0
+                           : CLUSTER                ? xpart[3 * (lane + 32 * j) + warp]
+                                                    : d.part[4 * (size_t)(lane + 32 * j) + warp];
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
                     if (32 * j < n_part) s += x[j];
@@ -705,7 +798,10 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
             __syncthreads();
             if (t < 6 * nu) {
                 const int x = t / 6, c = t - 6 * x;
-                d.rcp[6 * (size_t)(u0 + x) + c] = S.ws[2 * x][c] + S.ws[2 * x + 1][c];
+                const float v = S.ws[2 * x][c] + S.ws[2 * x + 1][c];
+                d.rcp[6 * (size_t)(u0 + x) + c] = v;
+                if (CLUSTER)   // to the CTAs that multiply it
+                    for (int rk = 0; rk < min(G, n_cu); ++rk) st_cluster(mapa(smem_u32(xrc + 6 * (u0 + x) + c), rk), v);
             }
             arrive();
         }
@@ -799,6 +895,7 @@ void res_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, const ResSha
 }  // namespace
 
 int res_tmem_chunks() { return kResTmemChunks; }
+int res_smem_exchange(bool fp64) { return fp64 ? kExBytes<double> : kExBytes<float>; }
 int res_smem_max() { return 227 * 1024 - kResStatic; }
 int res_smem_coarse(int stages, int b_chunks) { return stages * kFuChunkA + b_chunks * kResChunkB; }
 int res_part_chunks(int N) { return coarse_part_chunks(N); }

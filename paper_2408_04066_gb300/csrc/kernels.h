@@ -195,6 +195,7 @@ struct ResLimits {
 };
 cudaError_t res_init(ResLimits& lim);   // kernel attributes and limits of the current device
 int res_smem_max();
+int res_smem_exchange(bool fp64);   // of a cluster's CTA
 int res_tmem_chunks();   // chunks of A_c^{-1} a CTA keeps in tensor memory
 int res_smem_coarse(int stages, int b_chunks);
 int res_part_chunks(int N);    // chunks of the K range a coarse unit takes (b_chunks)
