@@ -133,8 +133,9 @@ typedef struct {
                             linear solve from any start); a state set by
                             mfem_set_state is used as it is */
     int32_t max_batch;   /* poses per mfem_solve_batch call allocated for (16) */
-    int32_t tile_rows;   /* SpMV rows per block: 64, 128 or 256; 0 = autotune (timed
-                            on the first assembled system) */
+    int32_t tile_rows;   /* SpMV rows per block: 64, 128 or 256; 0 = autotune (128 or
+                            256, timed on the first system solved by the streamed
+                            kernels) */
     int32_t diagnostics; /* 1: fill inverted/skew/angle fields of mfem_stats (0) */
     int32_t rotation;    /* MFEM_ROT_RIG (default): R_k is the rotation of the tet's
                             cluster handle (§3, Eq. 3; §3.1) -- the paper's method.
@@ -197,11 +198,13 @@ typedef struct {
 /* Device-side profile of the last solve call, timed with CUDA events on the
  * context's stream.  The dominant work is the PCG iteration: an SpMV+dot
  * kernel and an update kernel per iteration, plus on two-level iterations one
- * kernel per mesh for the coarse product and correction (tensor cores), or the
+ * kernel for every mesh's coarse product and correction (tensor cores), or the
  * product and a correction kernel (CUDA cores), enqueued in chunks. */
 typedef struct {
     int32_t kernel_launches;  /* all library kernels launched in the call */
-    int32_t pcg_launches;     /* SpMV and update launches (two per iteration) */
+    int32_t pcg_launches;     /* SpMV and update launches (two per iteration; problems that fit
+                                 the chip run their iterations inside one launch, which count
+                                 here as two each too) */
     double pcg_ms;            /* summed time of the PCG iteration chunks (all their kernels) */
     double pcg_bytes;         /* algorithmic bytes moved by those chunks */
     int64_t pcg_iters;        /* PCG iterations summed over poses */
@@ -294,11 +297,9 @@ mfem_status mfem_get_elem(mfem_ctx* ctx, double* s, double* lam);
 
 /* mfem_get_elem for callers that cannot allocate device memory after set-up.
  * The paper has no counterpart; this is a deployment variant.  mfem_get_elem
- * allocates and frees a device staging buffer on every call, and cudaFree
- * waits for the whole device; a per-frame animation loop or a host
- * application's plugin that owns a fixed device budget may allocate only while
- * it sets up, so it cannot call that.  This entry point runs the same kernel
- * but stages through a fixed file-scope device array of 15 doubles per tet for
+ * stages its outputs in the context's element-block storage; this entry point
+ * runs the same kernel but touches none of the context's buffers: it stages
+ * through a fixed file-scope device array of 15 doubles per tet for
  * at most MFEM_ELEM_STATIC_MAX_TETS tets (7.5 MiB), held by every GPU that
  * loads the library until the process exits; it calls no cudaMalloc, cudaFree
  * or allocating library routine.  Arguments and outputs are those of
