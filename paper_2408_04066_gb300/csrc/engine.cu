@@ -272,7 +272,7 @@ void end_profile(mfem_ctx* c) {
 namespace {
 
 // Algorithmic bytes of one PCG iteration of one problem (each datum crossing
-// HBM once, 3-vectors counted as 3 elements): k_pcg_spmv reads the matrix
+// HBM once, 3-vectors counted as 3 elements): the SpMV reads the matrix
 // values and column ids and the row's u and r, and writes w (the neighbours' u
 // are the same vector); k_pcg_update reads u, w, p, s, dx, r and the 6-element
 // D^-1 and writes p, s, dx, r and zb, and u under block Jacobi.  With the
@@ -483,7 +483,7 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
     if (most <= 16) {
         // the largest cluster size that leaves no CTA without rows and runs every
         // problem at once: a smaller one halves the SMs that read a problem's matrix
-        // (11k tets, 47 units: 16 us an iteration on 8 CTAs, 11 on 16)
+        // (11k tets, 47 units, through L2: 16 us an iteration on 8 CTAs, 11 on 16)
         int least = 0;
         for (size_t i = 0; i < np; ++i) least = i ? std::min(least, units[i]) : units[i];
         for (int k = kResClusterSizes - 1, cl = 16; k >= 0 && sh.cluster == 0; --k, cl /= 2) {

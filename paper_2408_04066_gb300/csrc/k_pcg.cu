@@ -96,9 +96,9 @@ __device__ __forceinline__ void restrict_units(const float (&r)[3], bool valid, 
 //
 // Kernels of one iteration, over every problem of the descriptor table (a
 // block is one (problem, tile) unit and returns at once for an inactive problem):
-//   [coarse product e = Ahat r_c per mesh]
-//   k_pcg_correct: u = zb + P e                      (two-level problems only)
-//   k_pcg_spmv:    w = K u (neighbour u gathered), partials of (r,u), (w,u),
+//   k_coarse_fused: e = Ahat r_c, u = zb + P e       (two-level problems only;
+//                  with FP32 coarse products k_coarse_gemm and k_pcg_correct)
+//   k_pcg_spmv_row (or _split): w = K u (neighbour u gathered), partials of (r,u), (w,u),
 //                  (r,r); the last tile of a problem tests convergence
 //                  (|r| <= tol |r0| or the iteration cap) and sets alpha, beta
 //   k_pcg_update:  p, s, dx, r as above; zb = D^{-1} r; u = zb (block Jacobi) or
@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(256) k_coarse_gemm(const float* __restrict__ A
 
 // u_i = zb_i + Q_a P_i e_a (e_a = the six coarse values of row i's aggregate,
 // e_t + e_w x (X_i - c_a) turned by the aggregate's rotation), written
-// to the neighbour record the next k_pcg_spmv gathers.  The block first gathers
+// to the neighbour record the next SpMV gathers.  The block first gathers
 // the slice partials of e of its aggregates (added in slice order) and their
 // rotations into shared memory.  Problems without the coarse correction return
 // at once (their u was written by the update).

@@ -6,8 +6,8 @@
 // kResUnits units of 64 rows, a thread owns one row and keeps its r, p, s, dx,
 // zb and D^{-1} in registers, and the CTA's slices of the matrix sit in shared
 // memory as far as they fit (the rest is read from L2).  Only u, the coarse
-// residual, the coarse partial products and the inner-product partials go
-// through global memory (L2), separated by four group barriers an iteration:
+// residual, the coarse partial products and the inner-product partials are
+// exchanged, between four group barriers an iteration:
 //
 //   coarse product (tcgen05, the K-range parts of k_coarse_fused as units of
 //   work)  |  u = zb + P e  |  w = K u, dots  |  alpha, beta; p, s, dx, r, zb,
@@ -22,16 +22,17 @@
 // What bounds it: the latency of the barriers and of the L2 round trips between
 // them, not bytes -- these problems are the ones whose streamed iteration is
 // three dependent launches that each leave most of the chip idle.  An iteration,
-// streamed and here: 11k tets, one pose, 18.9 -> 11.4 us; 10k tets, 5 poses, 23.4
-// -> 10.8; 50k tets, 3 poses, 26.1 -> 13.9; 200k tets, one pose, 41.0 -> 17.1.
+// streamed and here: 11k tets, one pose, 18.9 -> 9.7 us; 10k tets, 5 poses, 23.4
+// -> 9.5; 50k tets, 3 poses, 26.1 -> 13.5; 200k tets, one pose, 41.0 -> 16.3 (streamed:
+// before the later changes of those kernels).
 //
 // The chunks of A_c^{-1} a CTA multiplies stay in tensor memory (seven of its
 // units' 32 KB chunks; the eighth and later ones in shared memory): streaming
 // them from L2 every iteration took 19000 of its 58000 cycles on the 200k figure,
 // and an MMA whose A comes from tensor memory issues in 59 cycles instead of 165.
 //
-// Every wait in global memory or on an mbarrier is bounded by the global timer;
-// one that runs out marks the problem (kFault) and the CTA leaves after its
+// Every wait is bounded, in global memory by a number of polls, on an mbarrier by
+// the global timer; one that runs out marks the problem (kFault) and the CTA leaves after its
 // copies in flight have landed and its tensor memory is freed.  A CTA that has
 // left no longer counts in the cluster barrier.
 #include <cuda_bf16.h>
@@ -54,6 +55,7 @@ constexpr int kResTmemChunk = kTcKC / 2;            // columns a chunk takes (tw
 constexpr int kResTmemChunks = 7;                   // chunks tensor memory holds (512 columns)
 static_assert(kResTmemD + kResTmemChunks * kResTmemChunk <= 512, "tensor memory");
 constexpr int kResMaxStages = 8;
+constexpr int kResPolls = 1 << 18;                  // polls of a group barrier before it gives up (over 0.1 s of running time)
 constexpr int kResStatic = 2048;                    // bound of the static shared memory below
 constexpr int kResMaxThreads = kCoarseRows * kResUnits;   // one thread per row
 
@@ -465,9 +467,8 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         }
         if (t == 0) {
             const unsigned target = bar_n * (unsigned)G;
-            const uint64_t ts = global_ns();
-            while (ld_acquire(job.bar) < target)
-                if (global_ns() - ts > kTcWaitNs) {
+            for (int i = 0; ld_acquire(job.bar) < target; ++i)
+                if (i >= kResPolls) {
                     S.fail = 1;
                     break;
                 }
