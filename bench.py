@@ -170,9 +170,9 @@ def hbm_peak():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-PCG_SOURCES = ("k_pcg.cu", "k_coarse_tc.cu", "dev.cuh")
-PCG_KERNELS = ("PCG iteration (k_pcg_spmv + k_pcg_update; on two-level steps also the coarse product "
-               "k_coarse_tc and k_pcg_correct)")
+PCG_SOURCES = ("k_pcg.cu", "k_coarse_tc.cu", "pcg_dev.cuh", "tc_dev.cuh", "dev.cuh")
+PCG_KERNELS = ("PCG iteration (k_pcg_spmv_row + k_pcg_update; on two-level steps also the coarse product "
+               "and correction, k_coarse_fused)")
 
 
 def kernel_source_hash():
@@ -196,7 +196,7 @@ def pcg_traffic(tr, pose_iters, coarse_launches, pairs):
             + tr["coarse_dram_bytes_per_launch"] * coarse_launches) / pairs
 
 
-TRAFFIC_NOTE = ("ncu dram__bytes_read+write of one two-level iteration (k_coarse_tc, k_pcg_correct, k_pcg_spmv, "
+TRAFFIC_NOTE = ("ncu dram__bytes_read+write of one two-level iteration (k_coarse_fused, k_pcg_spmv_row, "
                 "k_pcg_update) on the profiling case (8 poses of this mesh): the row kernels' bytes per "
                 "pose-iteration and the coarse product's per launch, scaled by this run's pose-iterations and "
                 "coarse launches per launch pair")
@@ -460,7 +460,7 @@ def run_mfem(args, dist):
     poses = dist.sum(nb * args.steps)
     value = poses / (total_ms_max / 1e3)
 
-    # roofline of the dominant work: the PCG iteration, one k_pcg_spmv and one
+    # roofline of the dominant work: the PCG iteration, one k_pcg_spmv_row and one
     # k_pcg_update launch per iteration, timed per 16-iteration chunk with CUDA
     # events on the stream the library launches on
     pcg_ms = sum(p["pcg_ms"] for p in prof)
