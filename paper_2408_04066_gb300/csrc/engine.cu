@@ -729,19 +729,20 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
     return MFEM_OK;
 }
 
-// Pick the SpMV's shape -- rows per block (64, 128, 256) and threads per row
+// Pick the SpMV's shape -- rows per block (kPcgTiles) and threads per row
 // (1, 2) -- by timing a fixed number of PCG iterations of each candidate on the
 // first assembled system (results are discarded; PCG is re-initialised
 // afterwards).  A shape fixed by the options is not searched.
-// MFEM_AUTOTUNE_CACHE names a file of earlier picks ("key tile split" lines).
+// MFEM_AUTOTUNE_CACHE names a file of earlier picks ("key tile split" lines; any
+// supported tile).
 mfem_status autotune_tile(mfem_ctx* c, std::vector<Group>& gs) {
     const char* cache = std::getenv("MFEM_AUTOTUNE_CACHE");
     char key[128];
     snprintf(key, sizeof key, "%d %d %lld %d %d", c->plan.n, c->plan.m, (long long)c->plan.nnz_blocks,
              c->slot.prec, gs[0].B);
     std::vector<int> tiles, splits;
-    for (int t : kPcgTiles)
-        if (!c->opt.tile_rows || t == c->opt.tile_rows) tiles.push_back(t);
+    if (c->opt.tile_rows) tiles.push_back(c->opt.tile_rows);
+    else tiles.assign(std::begin(kPcgTiles), std::end(kPcgTiles));
     for (int sp = 1; sp <= 2; ++sp)
         if (!c->opt.spmv_split || sp == c->opt.spmv_split) splits.push_back(sp);
     if (cache) {
@@ -751,7 +752,7 @@ mfem_status autotune_tile(mfem_ctx* c, std::vector<Group>& gs) {
                 int tile = 0, sp = 1;
                 size_t kl = strlen(key);
                 if (strncmp(line, key, kl) == 0 && sscanf(line + kl, " %d %d", &tile, &sp) >= 1 &&
-                    std::find(tiles.begin(), tiles.end(), tile) != tiles.end() &&
+                    (c->opt.tile_rows ? tile == c->opt.tile_rows : pcg_tile_supported(tile)) &&
                     std::find(splits.begin(), splits.end(), sp) != splits.end()) {
                     c->tile_rows = tile;
                     c->spmv_split = sp;

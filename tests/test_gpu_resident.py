@@ -63,6 +63,26 @@ def test_iteration_cap():
     ctx.close()
 
 
+@pytest.mark.parametrize("saved", [False, True])
+def test_64_row_blocks_without_a_search_of_them(saved, tmp_path, monkeypatch):
+    """The shape search leaves 64-row blocks out, but the option and an earlier pick saved
+    in the cache file still give them."""
+    from paper_2408_04066_gb300 import mfem
+    cfg = config("bar")
+    xf = np.concatenate([np.asarray(cfg["xfs"])] * 160)[:160]
+    f = tmp_path / "picks"
+    if saved:
+        monkeypatch.setenv("MFEM_AUTOTUNE_CACHE", str(f))
+        ctx = mfem.Context.from_config(cfg, max_batch=160)
+        ctx.solve_batch(xf)
+        ctx.close()
+        f.write_text(" ".join(f.read_text().split()[:-2] + ["64", "1"]) + "\n")
+    ctx = mfem.Context.from_config(cfg, max_batch=160, tile_rows=0 if saved else 64)
+    _, stats = ctx.solve_batch(xf)
+    assert ctx.profile()["tile_rows"] == 64 and all(s["converged"] for s in stats)
+    ctx.close()
+
+
 @pytest.mark.parametrize("precond", ["two_level", "block_jacobi"])
 def test_served_requests_that_join_a_resident_solve(precond):
     """A request alone in the server runs in the resident kernel a chunk at a time; requests
