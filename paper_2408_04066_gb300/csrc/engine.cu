@@ -22,6 +22,7 @@ constexpr double kLsNoise = 1.0e-10; // predicted decrease below this * |E|: tak
 // thread per row: us per launched iteration at 64 / 128 / 256 rows, 16 poses of the
 // 200k figure 71.5 / 69.5 / 69.1, 4 poses of the 800k figure 78.6 / 74.1 / 72.3.
 constexpr int kPcgTiles[2] = {128, 256};
+constexpr int kResIters = 1 << 13;   // most iterations of a batch's resident launch but one: ~0.15 s
 constexpr int kTileDefault = 256;               // until a streamed solve has been timed
 constexpr int kPcgChunk = 16;                   // PCG iterations enqueued between convergence checks (no history)
 constexpr int kPcgChunkMin = 16, kPcgChunkMax = 64;   // bounds of a predicted chunk (multiples of 8)
@@ -617,7 +618,8 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
         chunk = std::min(kPcgChunkMax, std::max(per_request ? kPcgChunkMin : 8, (best + 7) / 8 * 8));
         // resident: every problem of a batch call runs to its own end (none waits
         // for another inside the launch); served requests keep the round's length
-        if (resident && !per_request) chunk = cap + 1;   // (the cap itself is seen one product later)
+        // (the cap itself is seen one product later; past kResIters a launch ends and is read)
+        if (resident && !per_request) chunk = std::min(cap, kResIters) + 1;
     }
     for (int done = 0; done < cap; done += chunk) {
         const int n_it = resident ? chunk : std::min(chunk, cap - done);
@@ -690,7 +692,7 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
         // a batch's resident solves end inside the launch, whatever their results:
         // the step is taken and the next element pass enqueued before they are read
         // (one host round trip a Newton step instead of two)
-        if (resident && !per_request && ahead) {
+        if (resident && !per_request && ahead && n_it > cap) {
             *ahead = true;
             c->ahead_jobs = nj;
             c->ahead_bytes = coarse_bytes;

@@ -63,6 +63,20 @@ def test_iteration_cap():
     ctx.close()
 
 
+@pytest.mark.parametrize("cap", [8192, 8193, 2**31 - 1])
+def test_large_iteration_caps(cap):
+    """Caps at and past the most iterations of one launch give the default cap's solve."""
+    from paper_2408_04066_gb300 import mfem
+    cfg = config("bar")
+    res = []
+    for opts in (dict(), dict(cg_max=cap)):
+        ctx = mfem.Context.from_config(cfg, spmv_split=1, tile_rows=128, **opts)
+        x, st = ctx.solve_batch(np.asarray(cfg["xfs"])[:1])
+        res.append((x, st[0]["pcg_iters"], st[0]["newton_iters"], st[0]["converged"]))
+        ctx.close()
+    assert np.array_equal(res[0][0], res[1][0]) and res[0][1:] == res[1][1:] and res[0][3]
+
+
 @pytest.mark.parametrize("saved", [False, True])
 def test_64_row_blocks_without_a_search_of_them(saved, tmp_path, monkeypatch):
     """The shape search leaves 64-row blocks out, but the option and an earlier pick saved
