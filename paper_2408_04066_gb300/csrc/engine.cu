@@ -732,21 +732,24 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
 }
 
 // Pick the SpMV's shape -- rows per block (kPcgTiles) and threads per row
-// (1, 2) -- by timing a fixed number of PCG iterations of each candidate on the
-// first assembled system (results are discarded; PCG is re-initialised
-// afterwards).  A shape fixed by the options is not searched.
+// (1, 2) -- for calls that `lead` leads, by timing a fixed number of PCG iterations of
+// each candidate on the first assembled system of group g (results are discarded; PCG
+// is re-initialised afterwards).  g may belong to another context than `lead`: only
+// g's own buffers are written.  A shape fixed by the lead's options is not searched.
 // MFEM_AUTOTUNE_CACHE names a file of earlier picks ("key tile split" lines; any
 // supported tile).
-mfem_status autotune_tile(mfem_ctx* c, std::vector<Group>& gs) {
+mfem_status autotune_tile(mfem_ctx* lead, const Group& g) {
+    mfem_ctx* c = g.ctx;
+    std::vector<Group> gs{g};
     const char* cache = std::getenv("MFEM_AUTOTUNE_CACHE");
     char key[128];
     snprintf(key, sizeof key, "%d %d %lld %d %d", c->plan.n, c->plan.m, (long long)c->plan.nnz_blocks,
-             c->slot.prec, gs[0].B);
+             c->slot.prec, g.B);
     std::vector<int> tiles, splits;
-    if (c->opt.tile_rows) tiles.push_back(c->opt.tile_rows);
+    if (lead->opt.tile_rows) tiles.push_back(lead->opt.tile_rows);
     else tiles.assign(std::begin(kPcgTiles), std::end(kPcgTiles));
     for (int sp = 1; sp <= 2; ++sp)
-        if (!c->opt.spmv_split || sp == c->opt.spmv_split) splits.push_back(sp);
+        if (!lead->opt.spmv_split || sp == lead->opt.spmv_split) splits.push_back(sp);
     if (cache) {
         if (FILE* f = fopen(cache, "r")) {
             char line[256];
@@ -754,14 +757,14 @@ mfem_status autotune_tile(mfem_ctx* c, std::vector<Group>& gs) {
                 int tile = 0, sp = 1;
                 size_t kl = strlen(key);
                 if (strncmp(line, key, kl) == 0 && sscanf(line + kl, " %d %d", &tile, &sp) >= 1 &&
-                    (c->opt.tile_rows ? tile == c->opt.tile_rows : pcg_tile_supported(tile)) &&
+                    (lead->opt.tile_rows ? tile == lead->opt.tile_rows : pcg_tile_supported(tile)) &&
                     std::find(splits.begin(), splits.end(), sp) != splits.end()) {
-                    c->tile_rows = tile;
-                    c->spmv_split = sp;
+                    lead->tile_rows = tile;
+                    lead->spmv_split = sp;
                 }
             }
             fclose(f);
-            if (c->tile_rows && c->spmv_split) return MFEM_OK;
+            if (lead->tile_rows && lead->spmv_split) return MFEM_OK;
         }
     }
     cudaEvent_t e0, e1;
@@ -769,13 +772,12 @@ mfem_status autotune_tile(mfem_ctx* c, std::vector<Group>& gs) {
     CK(cudaEventCreate(&e1));
     float best = 1e30f;
     int best_tile = tiles.back(), best_split = splits.front();
-    for (auto& g : gs)
-        for (int b = 0; b < g.B; ++b) g.ph[b].coarse = 0;   // timed with block Jacobi
+    for (int b = 0; b < g.B; ++b) g.ph[b].coarse = 0;   // timed with block Jacobi
     ElemArgs a = elem_args(c);
     for (int tile : tiles)
         for (int sp : splits)
             for (int rep = 0; rep < 2; ++rep) {
-                launch_pcg_init(a, gs[0].B, tile, 0.0, 1 << 30, nullptr, nullptr, c->stream);
+                launch_pcg_init(a, g.B, tile, 0.0, 1 << 30, nullptr, nullptr, c->stream);
                 CK(cudaEventRecord(e0, c->stream));
                 mfem_status st = c->slot.prec == 1 ? run_pcg<float>(c, gs, 1, tile, sp, 20, false)
                                                    : run_pcg<double>(c, gs, 0, tile, sp, 20, false);
@@ -793,8 +795,8 @@ mfem_status autotune_tile(mfem_ctx* c, std::vector<Group>& gs) {
             }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    c->tile_rows = best_tile;
-    c->spmv_split = best_split;
+    lead->tile_rows = best_tile;
+    lead->spmv_split = best_split;
     if (cache) {
         if (FILE* f = fopen(cache, "a")) {
             fprintf(f, "%s %d %d\n", key, best_tile, best_split);
@@ -1090,7 +1092,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 mfem_status st = MFEM_OK;
                 if (per_request || !fits_chip(c, one, tile_of(c))) {
                     st = upload_active(gc, g.B, start);
-                    if (st == MFEM_OK) st = autotune_tile(c, one);
+                    if (st == MFEM_OK) st = autotune_tile(c, one[0]);
                 }
                 std::copy(keep.begin(), keep.end(), g.ph);
                 if (st != MFEM_OK) return st;

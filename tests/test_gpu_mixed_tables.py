@@ -1,0 +1,41 @@
+"""Several meshes in one call of which the first fits the chip and another does not:
+the SpMV's shape is then searched on a group that is not the call's first, with more
+poses than the first context has slots for."""
+import numpy as np
+import pytest
+
+from synth import figure_config
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("lead,other", [("mixed", "mixed"), ("mixed", "fp64"), ("fp64", "mixed")])
+def test_shape_search_on_a_later_group(lead, other):
+    from paper_2408_04066_gb300 import mfem
+    cfgs = [dict(figure_config(3000, seeds=[5]), model="snh"),
+            dict(figure_config(60000, seeds=range(12)), model="corot")]
+    opts = dict(spmv_split=1)
+    # one slot in the first context, twelve poses in the second: 12 x 25 blocks of 512 rows, past 152 SMs
+    ctxs = [mfem.Context.from_config(c, precision=p, max_batch=len(c["xfs"]), **opts)
+            for c, p in zip(cfgs, (lead, other))]
+    outs, stats = mfem.solve_multi(ctxs, [c["xfs"] for c in cfgs])
+    assert ctxs[0].profile()["tile_rows"] in (128, 256)
+    tile = ctxs[0].profile()["tile_rows"]
+    again, stats2 = mfem.solve_multi(ctxs, [c["xfs"] for c in cfgs])
+    for i, (cfg, p) in enumerate(zip(cfgs, (lead, other))):
+        alone = mfem.Context.from_config(cfg, precision=p, max_batch=1, tile_rows=tile, **opts)
+        for b in range(len(cfg["xfs"])):
+            x, st = alone.solve_batch(cfg["xfs"][b:b + 1])
+            assert st[0]["converged"] and stats[i][b]["converged"]
+            for k in ("newton_iters", "pcg_iters"):
+                assert stats2[i][b][k] == st[0][k], (i, b, k)
+            assert np.array_equal(again[i][b], x[0]), (i, b)
+            # the call that made the search: a group's first reductions may have been taken with
+            # the default rows per block, which FP64 sums show in their last bits
+            if p == "mixed":
+                assert np.array_equal(outs[i][b], x[0]), (i, b)
+            else:
+                assert np.abs(outs[i][b] - x[0]).max() <= 1e-5 * np.ptp(cfg["X"], axis=0).max()
+        alone.close()
+    for c in ctxs:
+        c.close()
