@@ -403,18 +403,21 @@ mfem_status read_scalars(mfem_ctx* c, int B) {
 // exactly that many iterations, no checks -- used by the autotuner).
 // One chunk of PCG iterations: replayed from a CUDA graph captured the first
 // time these launch parameters occur (the descriptor table lives at a fixed
-// device address; only its contents change), else launched directly.
+// device address; only its contents change), else launched directly.  The key holds
+// every parameter that a capture keeps, the jobs' buffers among them: those of another
+// context of the call are allocated anew when its slots grow or it is made again.
 template <typename T>
 mfem_status launch_chunk(mfem_ctx* c, const PcgDesc<T>* dst, int nd, int units, int units_u, int tile, int split,
                          int n_it, const std::vector<CoarseJob>& jobs) {
     const int nj = (int)jobs.size();
     if (c->opt.launch == MFEM_LAUNCH_GRAPH && !c->graphs_off) {
-        char buf[96];
+        char buf[192];
         snprintf(buf, sizeof buf, "%d %p %d %d %d %d %d %d", (int)sizeof(T), (const void*)dst, nd, units, units_u, tile,
                  split, n_it);
         std::string key(buf);
         for (const auto& j : jobs) {
-            snprintf(buf, sizeof buf, " %p %d %d %d %d %d", j.key, j.Abf ? 1 : 0, j.N, j.d0, j.nd, j.agg_units);
+            snprintf(buf, sizeof buf, " %p %p %p %p %d %d %d %d %d", (const void*)j.Ainv, j.Abf, j.Bs, (const void*)j.err,
+                     j.N, j.d0, j.nd, j.agg_units, j.slots);
             key += buf;
         }
         auto it = c->graphs.find(key);

@@ -39,3 +39,22 @@ def test_shape_search_on_a_later_group(lead, other):
         alone.close()
     for c in ctxs:
         c.close()
+
+
+def test_second_context_grows_between_calls():
+    """The captured launches of a call hold the buffers of all its contexts: when the second
+    one's slots are allocated anew, the next call of the same sizes uses the new ones."""
+    from paper_2408_04066_gb300 import mfem
+    cfgs = [dict(figure_config(20000, seeds=range(4)), model="corot"),
+            dict(figure_config(60000, seeds=range(6)), model="corot")]
+    ctxs = [mfem.Context.from_config(c, max_batch=len(c["xfs"]), tile_rows=128, spmv_split=1) for c in cfgs]
+    xfs = [c["xfs"] for c in cfgs]
+    first = [mfem.solve_multi(ctxs, xfs) for _ in range(3)]   # chunks of the default and the predicted lengths
+    ctxs[1].solve_batch(np.concatenate([cfgs[1]["xfs"]] * 3))
+    then = [mfem.solve_multi(ctxs, xfs) for _ in range(3)]
+    for outs, stats in first[1:] + then:
+        for i in range(2):
+            assert np.array_equal(outs[i], first[0][0][i])
+            assert [s["pcg_iters"] for s in stats[i]] == [s["pcg_iters"] for s in first[0][1][i]]
+    for c in ctxs:
+        c.close()
