@@ -537,19 +537,16 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
 int tile_of(const mfem_ctx* c) { return c->tile_rows ? c->tile_rows : kTileDefault; }
 int split_of(const mfem_ctx* c) { return c->spmv_split ? c->spmv_split : 1; }
 
-// Whether the problems inside PCG run in the resident kernel.
-bool fits_chip(mfem_ctx* c, std::vector<Group>& gs, int tile) {
-    auto fits = [&](auto zero, int prec) {
-        using T = decltype(zero);
-        std::vector<PcgDesc<T>> d;
-        std::vector<mfem_ctx*> owner;
-        int u = 0, uu = 0;
-        build_descs<T>(gs, tile, prec, d, u, uu, nullptr, &owner);
-        ResShape sh;
-        std::vector<ResJob> jobs;
-        return d.empty() || plan_resident<T>(c, d, owner, tile, sh, jobs);
-    };
-    return fits(0.f, 1) && fits(0.0, 0);
+// Whether run_pcg takes the problems of precision T inside PCG to the resident kernel.
+template <typename T>
+bool fits_chip(mfem_ctx* c, std::vector<Group>& gs, int tile, int prec) {
+    std::vector<PcgDesc<T>> d;
+    std::vector<mfem_ctx*> owner;
+    int u = 0, uu = 0;
+    build_descs<T>(gs, tile, prec, d, u, uu, nullptr, &owner);
+    ResShape sh;
+    std::vector<ResJob> jobs;
+    return d.empty() || plan_resident<T>(c, d, owner, tile, sh, jobs);
 }
 
 template <typename T>
@@ -809,6 +806,47 @@ mfem_status autotune_tile(mfem_ctx* lead, const Group& g) {
     return MFEM_OK;
 }
 
+// The first streamed PCG of calls that c leads: times the shapes (a resident solve has
+// none).  Decided on the table that run_pcg will see, every group's problems that start
+// now (`starts`) among it, before any of them is initialised; timed on the largest group
+// of a precision that is streamed.
+mfem_status search_shape(mfem_ctx* c, std::vector<Group>& gs, const std::vector<std::vector<int>>& starts,
+                         bool per_request) {
+    std::vector<std::vector<ProbHost>> keep(gs.size());
+    auto mark = [&](size_t gi, bool alone) {   // alone: without the problems already inside PCG
+        Group& g = gs[gi];
+        for (int b = 0; b < g.B; ++b) {
+            if (alone || starts[gi][b]) g.ph[b].in_pcg = starts[gi][b];
+            if (starts[gi][b]) g.ph[b].coarse = g.ctx->mesh.coarse_n > 0;
+        }
+    };
+    auto restore = [&]() {
+        for (size_t gi = 0; gi < gs.size(); ++gi) std::copy(keep[gi].begin(), keep[gi].end(), gs[gi].ph);
+    };
+    for (size_t gi = 0; gi < gs.size(); ++gi) {
+        keep[gi].assign(gs[gi].ph, gs[gi].ph + gs[gi].B);
+        mark(gi, false);
+    }
+    const int tile = c->tile_rows ? c->tile_rows : kTileDefault;
+    const bool streamed[2] = {per_request || !fits_chip<double>(c, gs, tile, 0),
+                              per_request || !fits_chip<float>(c, gs, tile, 1)};
+    restore();
+    size_t pick = gs.size();
+    int64_t most = 0;
+    for (size_t gi = 0; gi < gs.size(); ++gi) {
+        const int64_t rows = std::count(starts[gi].begin(), starts[gi].end(), 1) * (int64_t)gs[gi].ctx->plan.n;
+        if (!streamed[gs[gi].ctx->slot.prec] || rows <= most) continue;
+        most = rows;
+        pick = gi;
+    }
+    if (pick == gs.size()) return MFEM_OK;
+    mark(pick, true);
+    mfem_status st = upload_active(gs[pick].ctx, gs[pick].B, starts[pick]);
+    if (st == MFEM_OK) st = autotune_tile(c, gs[pick]);
+    restore();
+    return st;
+}
+
 }  // namespace
 
 namespace {
@@ -1026,9 +1064,13 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
         CK(cudaStreamSynchronize(s));
         synced(gs);
         int ran = 0;   // iterations of the resident solves read back now
-        for (auto& g : gs) {
+        std::vector<std::vector<int>> starts(gs.size());
+        for (size_t gi = 0; gi < gs.size(); ++gi) {
+            Group& g = gs[gi];
             mfem_ctx* gc = g.ctx;
-            std::vector<int> start(g.B, 0), redo;
+            std::vector<int>& start = starts[gi];
+            std::vector<int> redo;
+            start.assign(g.B, 0);
             for (int b = 0; b < g.B; ++b) {
                 ProbHost& p = g.ph[b];
                 if (!p.active || p.in_pcg) continue;
@@ -1082,24 +1124,16 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 p.need_hess = 0;
                 start[b] = 1;
             }
+        }
+        if (c->tile_rows == 0 || c->spmv_split == 0) {
+            mfem_status st = search_shape(c, gs, starts, per_request);
+            if (st != MFEM_OK) return st;
+        }
+        for (size_t gi = 0; gi < gs.size(); ++gi) {
+            Group& g = gs[gi];
+            mfem_ctx* gc = g.ctx;
+            const std::vector<int>& start = starts[gi];
             if (!any_of(start)) continue;
-            // first streamed PCG of this context: time the shapes (a resident one has
-            // none) on the problems that start now, the others' state untouched
-            if (c->tile_rows == 0 || c->spmv_split == 0) {
-                const std::vector<ProbHost> keep(g.ph, g.ph + g.B);
-                for (int b = 0; b < g.B; ++b) {
-                    g.ph[b].in_pcg = start[b];
-                    g.ph[b].coarse = gc->mesh.coarse_n > 0;
-                }
-                std::vector<Group> one{Group{gc, g.B, g.ph}};
-                mfem_status st = MFEM_OK;
-                if (per_request || !fits_chip(c, one, tile_of(c))) {
-                    st = upload_active(gc, g.B, start);
-                    if (st == MFEM_OK) st = autotune_tile(c, one[0]);
-                }
-                std::copy(keep.begin(), keep.end(), g.ph);
-                if (st != MFEM_OK) return st;
-            }
             // PCG target of this Newton step: cg_tol; where the Newton model is
             // trusted -- a quadratic energy (ARAP or corot with rig rotations:
             // Newton is iterative refinement of one linear solve) or a warm start

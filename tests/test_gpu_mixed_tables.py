@@ -15,7 +15,7 @@ def test_shape_search_on_a_later_group(lead, other):
     cfgs = [dict(figure_config(3000, seeds=[5]), model="snh"),
             dict(figure_config(60000, seeds=range(12)), model="corot")]
     opts = dict(spmv_split=1)
-    # one slot in the first context, twelve poses in the second: 12 x 25 blocks of 512 rows, past 152 SMs
+    # one slot in the first context, twelve poses in the second: 12 x 26 blocks of 512 rows, past 152 SMs
     ctxs = [mfem.Context.from_config(c, precision=p, max_batch=len(c["xfs"]), **opts)
             for c, p in zip(cfgs, (lead, other))]
     outs, stats = mfem.solve_multi(ctxs, [c["xfs"] for c in cfgs])
@@ -56,5 +56,27 @@ def test_second_context_grows_between_calls():
         for i in range(2):
             assert np.array_equal(outs[i], first[0][0][i])
             assert [s["pcg_iters"] for s in stats[i]] == [s["pcg_iters"] for s in first[0][1][i]]
+    for c in ctxs:
+        c.close()
+
+
+def test_search_when_only_the_whole_table_is_too_large(tmp_path, monkeypatch):
+    """Meshes that fit the chip one by one but not together run in the streamed kernels: their
+    shape is searched, on the larger group.  Together with a smaller one they fit: no search."""
+    from paper_2408_04066_gb300 import mfem
+    picks = tmp_path / "picks"
+    monkeypatch.setenv("MFEM_AUTOTUNE_CACHE", str(picks))
+    cfgs = [dict(figure_config(t, seeds=range(b)), model="corot") for t, b in ((3000, 1), (50000, 4), (60000, 5))]
+    ctxs = [mfem.Context.from_config(c, max_batch=len(c["xfs"]), spmv_split=1) for c in cfgs]
+    mfem.solve_multi(ctxs[:2], [c["xfs"] for c in cfgs[:2]])   # 1 x 2 + 4 x 22 blocks of 512 rows
+    assert not picks.exists()
+    outs, stats = mfem.solve_multi(ctxs[1:], [c["xfs"] for c in cfgs[1:]])   # 4 x 22 + 5 x 26, past 152 SMs
+    lines = picks.read_text().splitlines()
+    assert len(lines) == 1 and lines[0].split()[:2] == [str(ctxs[2].n), str(ctxs[2].m)]
+    for i, cfg in enumerate(cfgs[1:]):
+        alone = mfem.Context.from_config(cfg, max_batch=1, spmv_split=1, tile_rows=128)
+        for b in range(len(cfg["xfs"])):
+            assert np.array_equal(alone.solve_batch(cfg["xfs"][b:b + 1])[0][0], outs[i][b])
+        alone.close()
     for c in ctxs:
         c.close()
