@@ -99,7 +99,8 @@ __device__ __forceinline__ uint32_t cluster_rank() {
     return r;
 }
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 // FP32 at the same shared-memory offset in CTA `rank` of the cluster
 __device__ __forceinline__ float ld_cluster_f32(const float* local, uint32_t rank) {
@@ -180,13 +181,7 @@ __global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
         }
     }
     if (t < kTcProbs) dp[t] = nullptr;
-    if (warp == kFuThreads / 32 - 1) {
-        __syncwarp();
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                     "r"(kTcTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    if (warp == kFuThreads / 32 - 1) tmem_alloc(tslot, kTcTmemCols);
     __syncthreads();
     pdl_wait();
     pdl_trigger();
@@ -212,11 +207,7 @@ __global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
         if (t == 0)
             for (int c = 0; c < nst; ++c)
                 if (!mbar_wait(&full[c], 0)) atomicOr(err, 4u);
-        if (warp == 0) {
-            __syncwarp();
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols)
-                         : "memory");
-        }
+        if (warp == 0) tmem_free(tmem, kTcTmemCols);
         return;
     }
 
@@ -299,8 +290,7 @@ __global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
             float v[16];
 #pragma unroll
             for (int part = 0; part < 3; ++part) {
-                tmem_ld16(lane_addr + part * kTcProbs, v);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                tmem_ld(lane_addr + part * kTcProbs, v);
 #pragma unroll
                 for (int p = 0; p < kTcProbs; ++p) red[(part * kTcProbs + p) * kTcM + row] = v[p];
             }
@@ -326,9 +316,7 @@ __global__ void __launch_bounds__(kFuThreads, ST == kFuStagesMulti ? 2 : 1)
         es[r][p] = e;
     }
     cluster_sync();   // no CTA leaves or reuses its part while another reads it
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols)
-                     : "memory");
+    if (warp == 0) tmem_free(tmem, kTcTmemCols);
     if (e_out) {   // the product alone
         for (int i = t; i < 6 * kFuAggsCta * kTcProbs; i += kFuThreads) {
             const int r = i % (6 * kFuAggsCta), p = i / (6 * kFuAggsCta), row = 6 * a_cta + r;

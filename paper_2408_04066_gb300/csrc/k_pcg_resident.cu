@@ -89,15 +89,6 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
 __device__ __forceinline__ void red_release(unsigned* p) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
-// four consecutive FP32 columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
-    uint32_t r[4];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(taddr));
-#pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 // Exchange area of a cluster's CTA, at the same offset in each: the other CTAs
 // write its copies of the inner-product partials and of r_c, and read its u.
@@ -132,12 +123,6 @@ __device__ __forceinline__ void ld_cluster(uint32_t a, double (&q)[3]) {
     asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(q[2]) : "r"(a + 16) : "memory");
 }
 
-// eight 32-bit columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, uint4 a, uint4 b) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(a.x),
-                 "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
-                 : "memory");
-}
 // MMA with A in tensor memory
 __device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
                                              uint32_t accumulate) {
@@ -327,13 +312,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         ring_start();
         for (int i = 0; i < n_ring && i < sh.stages; ++i) load_next();
     }
-    if (has_cu && warp == 0) {
-        __syncwarp();
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem)),
-                     "r"(tm_cols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    if (has_cu && warp == 0) tmem_alloc(&S.tmem, tm_cols);
 
     // ---- the row's state
     T r[3] = {0, 0, 0}, pp[3] = {0, 0, 0}, ss[3] = {0, 0, 0}, dx[3] = {0, 0, 0}, zb[3] = {0, 0, 0}, di[kDinv];
@@ -371,10 +350,10 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                 for (int k = warp >> 2; k < kTcSteps; k += kThreads / 128) {
                     const uint4 x = __ldg(reinterpret_cast<const uint4*>(src + a_piece(arow, 2 * k)));
                     const uint4 y = __ldg(reinterpret_cast<const uint4*>(src + a_piece(arow, 2 * k + 1)));
-                    tmem_st8(tmem + lane0 + kResTmemD + i * kResTmemChunk + 8 * k, x, y);
+                    tmem_st(tmem + lane0 + kResTmemD + i * kResTmemChunk + 8 * k, x, y);
                 }
             }
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        tmem_st_wait();
         tc_fence_before();
     }
     const int voff = ul < kResUnits ? S.voff[ul] : -1;
@@ -427,11 +406,11 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                 asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(smem_u32(&S.fail), rk)), "r"(1) : "memory");
     };
     if (CLUSTER) {   // every CTA of the cluster runs before the first remote access
-        __syncwarp();
-        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        cluster_arrive();
+        cluster_wait();
         tell_fail();
-        __syncwarp();
-        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        cluster_arrive();
+        cluster_wait();
     }
     const bool go = CLUSTER ? !S.fail : landed;
     // FP64, one unit a CTA: an FP64 instruction holds a scheduler for 64 cycles and
@@ -451,8 +430,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
     // every write of the group's CTAs before arrive() is visible to their reads after wait()
     auto arrive = [&]() {
         if (CLUSTER) {
-            __syncwarp();
-            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+            cluster_arrive();
             return;
         }
         __syncthreads();
@@ -461,8 +439,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
     };
     auto wait = [&]() {
         if (CLUSTER) {
-            __syncwarp();
-            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+            cluster_wait();
             return;
         }
         if (t == 0) {
@@ -580,8 +557,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                 tc_fence_after();
                 if (warp < kTcM / 32) {
                     float v[4];
-                    tmem_ld4(tmem + ((uint32_t)(warp * 32) << 16), v);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    tmem_ld(tmem + ((uint32_t)(warp * 32) << 16), v);
                     const int lr = warp * 32 + lane, er = 6 * kFuAggsBlk * rb + lr;
                     if (lr < 6 * kFuAggsBlk && er < N) job.epart[(size_t)q * ld_e + er] = (v[0] + v[1]) + v[2];
                 }
@@ -899,9 +875,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         }
     }
     __syncthreads();
-    if (has_cu && warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tm_cols)
-                     : "memory");
+    if (has_cu && warp == 0) tmem_free(tmem, tm_cols);
 }
 
 template <typename T, bool CLUSTER, int U>
