@@ -327,6 +327,12 @@ mfem_status mfem_get_elem_static(mfem_ctx* ctx, double* s, double* lam);
  * MFEM_EINVAL if the context has no coarse space or B < 1. */
 mfem_status mfem_coarse_apply(mfem_ctx* ctx, const float* rc, int32_t B, float* e, int32_t product);
 
+/* For tests of the error path: in the next launch of the resident PCG kernel (problems
+ * that fit the chip) by a call that ctx leads, one thread block of every problem takes a
+ * wait of iteration `iteration` as run out; every wait itself ends as usual.  Negative:
+ * none.  Has no effect on the streamed kernels. */
+mfem_status mfem_expire_wait(mfem_ctx* ctx, int32_t iteration);
+
 /* Warm-start state (the last solution, host [n][3], caller order). */
 mfem_status mfem_get_state(const mfem_ctx* ctx, double* x);
 mfem_status mfem_set_state(mfem_ctx* ctx, const double* x);

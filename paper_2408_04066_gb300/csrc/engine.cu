@@ -632,6 +632,8 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
         int pe = count ? c->prof.begin(2, c->stream) : -1;
         if (resident) {
             rsh.iters = n_it;
+            rsh.expire = c->res_expire;
+            c->res_expire = -1;
             if (rsh.cluster == 0)
                 for (auto& g : gs)
                     if (g.ctx->slot.prec == prec)
@@ -1924,6 +1926,12 @@ mfem_status mfem_get_elem(mfem_ctx* c, double* s, double* lam) {
     if (s) CK(cudaMemcpyAsync(s, buf, sizeof(double) * 6 * m, cudaMemcpyDeviceToHost, c->stream));
     if (lam) CK(cudaMemcpyAsync(lam, buf + 6 * m, sizeof(double) * 9 * m, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    return MFEM_OK;
+}
+
+mfem_status mfem_expire_wait(mfem_ctx* c, int32_t iteration) {
+    if (!c) return ctx_fail(nullptr, MFEM_EINVAL, "null context");
+    c->res_expire = iteration;
     return MFEM_OK;
 }
 

@@ -114,6 +114,7 @@ struct mfem_ctx {
     double ahead_bytes = 0.0;
     bool graphs_off = false;   // capture failed once (e.g. a stream that cannot capture)
     mfem::ResLimits res_lim;   // what the device holds of the resident PCG kernel (sms = 0: not used)
+    int res_expire = -1;       // mfem_expire_wait: the next resident launch's `expire`
     mfem_profile last_profile{};
     std::string err;
     bool owned_by_server = false;

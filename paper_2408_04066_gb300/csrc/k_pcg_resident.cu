@@ -71,7 +71,8 @@ template <typename T>
 struct ResShared {
     uint64_t full[kResMaxStages], empty[kResMaxStages], done, vals;
     uint32_t tmem;
-    int fail;
+    int fail;                       // a wait of this CTA ran out
+    int gfail;                      // cluster: one of some CTA's did (written by that CTA between cluster barriers)
     int voff[kResUnits];            // byte offset of a unit's values in the value area, -1: read from global memory
     int slots[kResUnits];
     double wsum[kResMaxThreads / 32][3];
@@ -222,6 +223,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         mbar_init(&S.done, 1);
         mbar_init(&S.vals, 1);
         S.fail = 0;
+        S.gfail = 0;
         S.st = ResState{sc->rho, sc->alpha, sc->beta, sc->rr0, sc->rr, sc->tol2, sc->first, sc->iter, sc->maxit,
                         sc->state, 0.0, 0.0};
         if (!S.st.first) {
@@ -398,13 +400,16 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
 #pragma unroll
         for (int i = 0; i < NB; ++i)
             if (c0[i] >= 0) c0[i] = u_address(c0[i]);
-    // a failed wait is told to every CTA of the cluster before its next barrier, so
-    // that all leave together and none reads the memory of one that has left
+    // a failed wait is told to every CTA of the cluster before its next barrier and
+    // looked at after it, so that all leave together and none reads the memory of one
+    // that has left; S.fail itself is written by this CTA alone, so that its threads
+    // agree on it at a block barrier
     auto tell_fail = [&]() {
         if (CLUSTER && t == 0 && S.fail)
             for (int rk = 0; rk < G; ++rk)
-                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(smem_u32(&S.fail), rk)), "r"(1) : "memory");
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(smem_u32(&S.gfail), rk)), "r"(1) : "memory");
     };
+    auto failed = [&]() { return (CLUSTER ? S.gfail : S.fail) != 0; };   // after a group barrier
     if (CLUSTER) {   // every CTA of the cluster runs before the first remote access
         cluster_arrive();
         cluster_wait();
@@ -412,7 +417,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         cluster_arrive();
         cluster_wait();
     }
-    const bool go = CLUSTER ? !S.fail : landed;
+    const bool go = CLUSTER ? !failed() : landed;
     // FP64, one unit a CTA: an FP64 instruction holds a scheduler for 64 cycles and
     // the unit's two warps would use two of the four, so six warps form the product,
     // a component of w each (bar of 1536 tets: an iteration 19.8 -> 16.4 us)
@@ -456,6 +461,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
     bool active = true;
     for (int it = 0; go && it < sh.iters; ++it) {
         T u[3] = {zb[0], zb[1], zb[2]};
+        if (t == 0 && it == sh.expire && rank == G - 1) S.fail = 1;   // tests
         if (coarse) {
             // ---- coarse product: this CTA's units
             int a_at = 0;   // chunks issued this iteration (thread 0)
@@ -562,8 +568,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                     if (lr < 6 * kFuAggsBlk && er < N) job.epart[(size_t)q * ld_e + er] = (v[0] + v[1]) + v[2];
                 }
                 tc_fence_before();
-                __syncthreads();
-                if (S.fail) break;
+                if (__syncthreads_or(S.fail)) break;
             }
             // the last chunk's stage, for the next iteration
             if (t == 0 && !keep && !S.fail)
@@ -578,7 +583,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
             tell_fail();
             arrive();
             wait();
-            if (S.fail) break;
+            if (failed()) break;
             // ---- u = zb + Q_a P_i e_a, the parts of e_a added in part order
             float ev = 0.f;
             if (lane < 6 && ul < nu) {
@@ -608,7 +613,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         const Partial<T> d0 = dot3_partial(r[0], r[1], r[2], u[0], u[1], u[2]);
         const Partial<T> d2 = dot3_partial(r[0], r[1], r[2], r[0], r[1], r[2]);
         wait();
-        if (S.fail) break;
+        if (failed()) break;
         // ---- w = K u
         T a0 = 0, a1 = 0, a2 = 0;
         if (by_comp) {
@@ -687,7 +692,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         }
         arrive();
         wait();
-        if (S.fail) break;
+        if (failed()) break;
         double tot[3] = {0.0, 0.0, 0.0};   // valid in thread 0
         if (sizeof(T) == 8) {
             const int nw = sh.rtile / 32, n_tiles = (n + sh.rtile - 1) / sh.rtile, n_warps = (n + 31) / 32;
@@ -827,7 +832,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         }
         if (coarse) {
             wait();
-            if (S.fail) break;
+            if (failed()) break;
         }
     }
 
@@ -849,7 +854,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         if (k < N) coarse_b_store(d.bunit, d.bslot % kCoarseGroupSlots, k, d.rcp[k]);
     }
     if (t == 0) {
-        if (S.fail) {
+        if (S.fail || S.gfail) {
             sc->state = kFault;
         } else if (rank == 0) {
             sc->rho = S.st.rho;

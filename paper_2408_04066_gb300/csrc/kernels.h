@@ -187,6 +187,7 @@ struct ResShape {
     int units;           // most units a CTA owns: 4, 6 or 8 (the kernel's variant)
     int rtile;           // FP64: rows per tile of the streamed kernel's reduction
     int iters;           // most iterations of this launch
+    int expire = -1;     // iteration at which a CTA of every group takes a wait as run out (tests)
     int stages, b_chunks, v_bytes, smem;   // shared memory: A ring, B chunks, matrix values, all
 };
 struct ResLimits {

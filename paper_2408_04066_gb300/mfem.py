@@ -94,6 +94,7 @@ _SIGS = [
     ("mfem_get_elem_static", C.c_int32, [C.c_void_p, _dp, _dp]),
     ("mfem_coarse_apply", C.c_int32, [C.c_void_p, C.POINTER(C.c_float), C.c_int32, C.POINTER(C.c_float),
                                       C.c_int32]),
+    ("mfem_expire_wait", C.c_int32, [C.c_void_p, C.c_int32]),
     ("mfem_get_state", C.c_int32, [C.c_void_p, _dp]),
     ("mfem_set_state", C.c_int32, [C.c_void_p, _dp]),
     ("mfem_get_profile", C.c_int32, [C.c_void_p, C.POINTER(Profile)]),
@@ -360,6 +361,10 @@ class Context:
                                            COARSE_PRODUCTS[product] if isinstance(product, str) else product),
                self._ctx)
         return e
+
+    def expire_wait(self, iteration):
+        """mfem_expire_wait: a wait of the next resident PCG launch taken as run out (tests)."""
+        _check(self._lib.mfem_expire_wait(self._ctx, iteration), self._ctx)
 
     def get_state(self):
         x = np.empty((self.n, 3))
