@@ -28,7 +28,7 @@
 //     with Ahat = bf16(A_c^{-1}) (symmetric: rounding is entrywise), which
 //     keeps PCG's theory intact at any tolerance.
 //
-// Every wait on a copy or an MMA is bounded by the global timer; a wait that
+// Every wait on a copy or an MMA is bounded (mbar_wait); a wait that
 // runs out sets a bit of the mesh's error word (read by the host after the
 // solve), waits (bounded) for the copies it issued and frees its tensor memory.
 // The cluster barriers are reached by every CTA of a cluster on every path.

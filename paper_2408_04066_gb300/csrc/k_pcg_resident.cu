@@ -32,7 +32,7 @@
 // and an MMA whose A comes from tensor memory issues in 59 cycles instead of 165.
 //
 // Every wait is bounded, in global memory by a number of polls, on an mbarrier by
-// the global timer; one that runs out marks the problem (kFault) and the CTA leaves after its
+// the global timer and a number of polls; one that runs out marks the problem (kFault) and the CTA leaves after its
 // copies in flight have landed and its tensor memory is freed.  A CTA that has
 // left no longer counts in the cluster barrier.
 #include <cuda_bf16.h>

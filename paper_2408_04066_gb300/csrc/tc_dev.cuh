@@ -18,7 +18,8 @@ constexpr int kTcM = 128;                         // MMA M: rows of A_c^{-1} per
 constexpr int kTcSteps = kTcKC / 16;              // MMAs per chunk (K = 16 each)
 constexpr int kFuStepA = kTcM * 16 * 2;           // bytes of A per K step (4 KB)
 constexpr int kFuChunkA = kFuStepA * kTcSteps;    // 32 KB
-constexpr uint64_t kTcWaitNs = 200ull * 1000ull * 1000ull;   // 0.2 s per bounded wait
+constexpr uint64_t kTcWaitNs = 200ull * 1000ull * 1000ull;   // 0.2 s per bounded wait ...
+constexpr uint32_t kTcWaitPolls = 1u << 12;                  // ... and this many polls of it (under 1 ms of waiting)
 
 // Row blocks of an N x N inverse (runs of the mesh's aggregates)
 __host__ __device__ __forceinline__ int row_blocks(int N) { return (N / 6 + kFuAggsBlk - 1) / kFuAggsBlk; }
@@ -58,11 +59,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Wait for phase `parity` of the barrier to complete, at most kTcWaitNs.
+// Wait for phase `parity` of the barrier to complete; false if it has not after
+// kTcWaitNs and kTcWaitPolls polls.  The clock runs on while another process has the
+// GPU, the polls do not: a pause alone does not end a wait.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     const uint64_t t0 = global_ns();
-    while (!mbar_try_wait(bar, parity))
-        if (global_ns() - t0 > kTcWaitNs) return false;
+    for (uint32_t n = 0; !mbar_try_wait(bar, parity); ++n)
+        if (n >= kTcWaitPolls && global_ns() - t0 > kTcWaitNs) return mbar_try_wait(bar, parity);
     return true;
 }
 
