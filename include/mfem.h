@@ -330,7 +330,9 @@ mfem_status mfem_coarse_apply(mfem_ctx* ctx, const float* rc, int32_t B, float* 
 /* For tests of the error path: in the next launch of the resident PCG kernel (problems
  * that fit the chip) by a call that ctx leads, one thread block of every problem takes a
  * wait of iteration `iteration` as run out; every wait itself ends as usual.  Negative:
- * none.  Has no effect on the streamed kernels. */
+ * none.  Has no effect on the streamed kernels.  A Newton step whose resident solve ends
+ * this way is solved again, from the same x, by the streamed kernels, to the same result;
+ * they also take the context's next rounds. */
 mfem_status mfem_expire_wait(mfem_ctx* ctx, int32_t iteration);
 
 /* Warm-start state (the last solution, host [n][3], caller order). */

@@ -64,8 +64,7 @@ __device__ __forceinline__ void st3(T* rec, size_t np, int f, size_t row, T a, T
 }
 
 // Problem states (PCG)
-// (kFault: a bounded wait of the resident kernel ran out)
-enum : int { kIdle = 0, kActive = 1, kConverged = 2, kMaxIter = 3, kFault = 4 };
+enum : int { kIdle = 0, kActive = 1, kConverged = 2, kMaxIter = 3 };
 
 // Per-problem scalars.  Tickets are reset to 0 by the tile that completes them.
 struct ProbScal {
@@ -76,6 +75,7 @@ struct ProbScal {
     float alpha_f, beta_f;   // FP32 copies of alpha and beta for the FP32 kernels
     int iter, state, maxit, active;
     unsigned tk_a, tk_b, tk_g, tk_e, tk_s, tk_init, tk_c;
+    unsigned fault;   // a bounded wait of the resident kernel ran out: dx is no result (cleared by k_pcg_init)
     int first;   // the next reduction is the solve's first (beta = 0, alpha = (r,u) / (w,u))
 };
 

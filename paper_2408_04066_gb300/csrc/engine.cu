@@ -23,6 +23,7 @@ constexpr double kLsNoise = 1.0e-10; // predicted decrease below this * |E|: tak
 // 200k figure 71.5 / 69.5 / 69.1, 4 poses of the 800k figure 78.6 / 74.1 / 72.3.
 constexpr int kPcgTiles[2] = {128, 256};
 constexpr int kResIters = 1 << 13;   // most iterations of a batch's resident launch but one: ~0.15 s
+constexpr int kResRest = 256;        // PCG rounds streamed after a resident launch's wait ran out (some tens of calls)
 constexpr int kTileDefault = 256;               // until a streamed solve has been timed
 constexpr int kPcgChunk = 16;                   // PCG iterations enqueued between convergence checks (no history)
 constexpr int kPcgChunkMin = 16, kPcgChunkMax = 64;   // bounds of a predicted chunk (multiples of 8)
@@ -356,6 +357,12 @@ void build_descs(std::vector<Group>& gs, int tile, int prec, std::vector<PcgDesc
     }
 }
 
+bool any_of(const std::vector<int>& f) {
+    for (int v : f)
+        if (v) return true;
+    return false;
+}
+
 // Next free staging region; waits for the stream only when the ring is used up.
 mfem_status next_stage(mfem_ctx* c, int& pos) {
     if (c->ring_pos >= kStageRing) {
@@ -450,6 +457,13 @@ mfem_status launch_chunk(mfem_ctx* c, const PcgDesc<T>* dst, int nd, int units, 
     return MFEM_OK;
 }
 
+// A resident launch was cut short (ProbScal::fault): something else holds SMs for long.
+// The next rounds of every context of the table stay with the streamed kernels, which
+// wait for nothing.
+void rest_resident(std::vector<Group>& gs) {
+    for (auto& g : gs) g.ctx->res_rest = kResRest;
+}
+
 // Layout of the resident kernel (k_pcg_resident.cu) for the table, or false if
 // its problems do not fit the chip at once: every problem gets CTAs enough for
 // its rows (kResUnits units of 64 each).  If 16 CTAs
@@ -459,7 +473,7 @@ template <typename T>
 bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vector<mfem_ctx*>& owner, int tile,
                    ResShape& sh, std::vector<ResJob>& jobs) {
     const ResLimits& lim = c->res_lim;
-    if (lim.sms <= 0) return false;
+    if (lim.sms <= 0 || c->res_rest > 0) return false;
     sh = ResShape{};
     sh.rtile = tile;
     const size_t np = d.size();
@@ -562,6 +576,7 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
     ResShape rsh;
     std::vector<ResJob> rjobs;
     bool resident = max_iters <= 0 && one_chunk && plan_resident<T>(c, d, owner, tile, rsh, rjobs);
+    if (one_chunk && c->res_rest > 0) c->res_rest--;
     const int nj = (int)jobs.size();
     double coarse_bytes = 0.0;   // A_c^{-1} streamed once per iteration per mesh
     for (const auto& j : jobs) coarse_bytes += j.Abf ? 2.0 * j.N * j.N : 4.0 * j.N * coarse_ld(j.N);
@@ -710,18 +725,32 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
         CK(cudaStreamSynchronize(c->stream));
         synced(gs);
         for (auto& g : gs) {
-            if (g.ctx->slot.prec != prec) continue;
-            if (g.ctx->cerr_host && *g.ctx->cerr_host)
-                return ctx_fail(c, MFEM_ECUDA, "coarse product: a bounded wait in the tensor-core kernel ran out");
+            mfem_ctx* gc = g.ctx;
+            if (gc->slot.prec != prec) continue;
+            if (gc->cerr_host && *gc->cerr_host)
+                return ctx_fail(c, MFEM_ETIMEOUT, "coarse product: a bounded wait in the tensor-core kernel ran out");
+            std::vector<int> again(g.B, 0);   // cut short: from the start, in the streamed kernels
             for (int b = 0; b < g.B; ++b) {
                 ProbHost& p = g.ph[b];
                 if (!p.active || !p.in_pcg) continue;
-                const ProbScal& q = g.ctx->sc_host[b];
-                if (q.state == kFault) return ctx_fail(c, MFEM_ECUDA, "PCG: a bounded wait in the resident kernel ran out");
+                ProbScal& q = gc->sc_host[b];
+                if (q.fault) {
+                    again[b] = 1;
+                    q.state = kActive;
+                    p.pcg_launched = p.pcg_seen = 0;
+                    any = true;
+                    continue;
+                }
                 any |= q.state == kActive;
                 ran = std::max(ran, q.iter - p.pcg_seen);
                 p.pcg_seen = q.iter;
             }
+            if (!any_of(again)) continue;
+            rest_resident(gs);
+            mfem_status st = upload_active(gc, g.B, again, true);
+            if (st != MFEM_OK) return st;
+            launch_pcg_init(elem_args(gc), g.B, tile, 0.0, gc->opt.cg_max, gc->slot.tol2, gc->slot.coarse_on, c->stream);
+            gc->prof.launches++;
         }
         if (resident && count) {   // the iterations it ran, counted as the streamed kernels' launch pairs
             c->prof.pcg_launches += 2 * ran;
@@ -857,12 +886,6 @@ std::vector<int> mask_of(const Group& g, bool (*pred)(const ProbHost&)) {
     std::vector<int> f(g.B, 0);
     for (int b = 0; b < g.B; ++b) f[b] = pred(g.ph[b]) ? 1 : 0;
     return f;
-}
-
-bool any_of(const std::vector<int>& f) {
-    for (int v : f)
-        if (v) return true;
-    return false;
 }
 
 }  // namespace
@@ -1071,7 +1094,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
             Group& g = gs[gi];
             mfem_ctx* gc = g.ctx;
             std::vector<int>& start = starts[gi];
-            std::vector<int> redo;
+            std::vector<int> redo, cut(g.B, 0);
             start.assign(g.B, 0);
             for (int b = 0; b < g.B; ++b) {
                 ProbHost& p = g.ph[b];
@@ -1083,8 +1106,16 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 // a resident solve whose step was taken before its result was read
                 if (p.pend) {
                     p.pend = 0;
-                    if (gc->sc_host[b].state == kFault)
-                        return ctx_fail(c, MFEM_ECUDA, "PCG: a bounded wait in the resident kernel ran out");
+                    if (gc->sc_host[b].fault) {   // cut short; x was left as it was: the same step again, streamed
+                        cut[b] = 1;
+                        p.it--;
+                        p.pred = p.pend_pred;
+                        p.spec = p.expect_conv = p.need_hess = 0;
+                        p.gprev = p.gprev_back;
+                        p.eta_prev = p.eta_back;
+                        rest_resident(gs);
+                        continue;
+                    }
                     finish_pcg(gc, b, p, p.it - 1);
                     ran = std::max(ran, gc->sc_host[b].iter);
                     if (p.spec) p.spec_slope = gc->sc_host[b].slope;
@@ -1095,7 +1126,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
             if (sst != MFEM_OK) return sst;
             for (int b = 0; b < g.B; ++b) {
                 ProbHost& p = g.ph[b];
-                if (!p.active || p.in_pcg || redo[b]) continue;   // a rejected full step: element pass again
+                if (!p.active || p.in_pcg || redo[b] || cut[b]) continue;   // element pass again: a rejected full step, ...
                 if (!p.pred) {   // the predictor's gradient is not the SNH residual
                     const ProbScal& sc = gc->sc_host[b];
                     p.gn = std::sqrt(sc.gnorm2);
@@ -1173,6 +1204,8 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 if (start[b]) {
                     gc->tol2_host[b] = eta * eta;
                     p.expect_conv = last;
+                    p.gprev_back = p.gprev;
+                    p.eta_back = p.eta_prev;
                     if (!p.pred) {
                         p.gprev = p.gn;
                         p.eta_prev = eta;
@@ -1244,6 +1277,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 fin[gi][b] = 1;
                 any_fin = true;
                 p.pend = unread;
+                p.pend_pred = p.pred;
                 if (!unread) finish_pcg(g.ctx, b, p, p.it);
                 g.ctx->alpha_host[b] = 1.0;
             }
@@ -2044,7 +2078,7 @@ mfem_status mfem_coarse_apply(mfem_ctx* c, const float* rc, int32_t B, float* e,
     if (err == cudaSuccess) err = cudaStreamSynchronize(c->stream);
     cleanup();
     if (err != cudaSuccess) return cuda_check(c, err, "coarse apply");
-    if (werr) return ctx_fail(c, MFEM_ECUDA, "coarse product: a bounded wait in the tensor-core kernel ran out");
+    if (werr) return ctx_fail(c, MFEM_ETIMEOUT, "coarse product: a bounded wait in the tensor-core kernel ran out");
     if (tc) {   // e of every slot, complete
         std::memcpy(e, out.data(), sizeof(float) * (size_t)B * N);
         return MFEM_OK;

@@ -41,6 +41,8 @@ struct ProbHost {
     int pcg_launched = 0;   // PCG iterations launched in the current solve
     int pcg_seen = 0;       // its iteration count at the last readback
     int pend = 0;           // its result is still to be read (resident solve, step already taken)
+    int pend_pred = 0;      // ... and it was the predictor step
+    double gprev_back = -1.0, eta_back = 0.0;   // gprev and eta_prev before the current solve, if it has to start again
     int ref_pend = 0;       // the reference gradient is still to be read
 };
 
@@ -115,6 +117,7 @@ struct mfem_ctx {
     bool graphs_off = false;   // capture failed once (e.g. a stream that cannot capture)
     mfem::ResLimits res_lim;   // what the device holds of the resident PCG kernel (sms = 0: not used)
     int res_expire = -1;       // mfem_expire_wait: the next resident launch's `expire`
+    int res_rest = 0;          // PCG rounds that stay with the streamed kernels after a resident launch was cut short
     mfem_profile last_profile{};
     std::string err;
     bool owned_by_server = false;

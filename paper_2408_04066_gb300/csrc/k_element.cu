@@ -1039,7 +1039,7 @@ __global__ void k_warm_save(ElemArgs A) {
 // each free vertex's rest position clusters to, Q_h Q_h,prev^T dcorr_v.
 __global__ void k_warm_step(ElemArgs A, int apply) {
     const int b = blockIdx.y;
-    if (!A.slot.active[b]) return;
+    if (!A.slot.active[b] || A.slot.sc[b].fault) return;   // (as k_update)
     const MeshDev& M = A.mesh;
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= M.n) return;

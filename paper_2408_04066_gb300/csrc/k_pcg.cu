@@ -161,6 +161,7 @@ __global__ void k_pcg_init(ElemArgs A, double tol2, int maxit, const double* __r
         sc->alpha_f = 0.f;
         sc->beta_f = 0.f;
         sc->iter = 0;
+        sc->fault = 0u;
         sc->tol2 = tol2_b ? tol2_b[b] : tol2;
         sc->maxit = maxit;
         sc->state = (tot[0] > 0.0 && maxit > 0) ? kActive : kConverged;

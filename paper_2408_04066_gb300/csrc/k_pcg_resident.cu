@@ -32,9 +32,11 @@
 // and an MMA whose A comes from tensor memory issues in 59 cycles instead of 165.
 //
 // Every wait is bounded, in global memory by a number of polls, on an mbarrier by
-// the global timer and a number of polls; one that runs out marks the problem (kFault) and the CTA leaves after its
-// copies in flight have landed and its tensor memory is freed.  A CTA that has
-// left no longer counts in the cluster barrier.
+// the global timer and a number of polls; one that runs out marks the problem
+// (ProbScal::fault) and the CTA leaves after its copies in flight have landed and its
+// tensor memory is freed.  The host then leaves x where it was and solves that step
+// again with the streamed kernels: a CTA needs a whole SM, so another stream's long
+// kernel can keep a group's last CTAs from starting for longer than its first ones wait.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -854,8 +856,9 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         if (k < N) coarse_b_store(d.bunit, d.bslot % kCoarseGroupSlots, k, d.rcp[k]);
     }
     if (t == 0) {
+        // a word of its own: one block may fail and another of its group not
         if (S.fail || S.gfail) {
-            sc->state = kFault;
+            sc->fault = 1u;
         } else if (rank == 0) {
             sc->rho = S.st.rho;
             sc->alpha = S.st.alpha;

@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kRowTile) k_slope(ElemArgs A) {
 template <typename T>
 __global__ void k_update(ElemArgs A) {
     const int b = blockIdx.y;
-    if (!A.slot.active[b]) return;
+    if (!A.slot.active[b] || A.slot.sc[b].fault) return;   // a resident solve cut short: x stays, the host solves again
     const int n = A.mesh.n;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 3 * n) return;

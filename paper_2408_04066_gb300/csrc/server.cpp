@@ -254,7 +254,7 @@ void mfem_server::run() {
             if (st != MFEM_OK) err = gs[0].ctx->err;
         }
         if (st != MFEM_OK) {
-            fail_all_busy(st);
+            fail_all_busy(st == MFEM_ETIMEOUT ? MFEM_ECUDA : st);   // a wait's ETIMEOUT: still running
             continue;
         }
         // completion
