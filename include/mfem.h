@@ -133,9 +133,10 @@ typedef struct {
                             linear solve from any start); a state set by
                             mfem_set_state is used as it is */
     int32_t max_batch;   /* poses per mfem_solve_batch call allocated for (16) */
-    int32_t tile_rows;   /* SpMV rows per block: 64, 128 or 256; 0 = autotune (128 or
-                            256, timed on the first system solved by the streamed
-                            kernels) */
+    int32_t tile_rows;   /* SpMV rows per block: 64, 128 or 256; 0 (default) = 128 in
+                            FP64, whose sums show their order over the blocks in the
+                            results' last bits; mixed: 128 or 256, timed on the first
+                            table solved by the streamed kernels */
     int32_t diagnostics; /* 1: fill inverted/skew/angle fields of mfem_stats (0) */
     int32_t rotation;    /* MFEM_ROT_RIG (default): R_k is the rotation of the tet's
                             cluster handle (§3, Eq. 3; §3.1) -- the paper's method.
@@ -167,8 +168,10 @@ typedef struct {
                             the coarse space at most 6144 dof (6 per aggregate);
                             else a power of two >= 64, raised to that smallest size
                             if it is below it.  Other values: MFEM_EINVAL */
-    int32_t spmv_split;  /* SpMV threads per row: 1, 2 (two threads take a row's
-                            even and odd slots), 0 = autotune with tile_rows */
+    int32_t spmv_split;  /* SpMV threads per row: 1 (0, the default, is 1) or 2 (two
+                            threads take a row's even and odd slots, which rounds
+                            differently and was slower in every table timed; never in
+                            the resident kernel) */
     int32_t coarse_product; /* the coarse solve e = A_c^{-1} r_c of the two-level
                             preconditioner: MFEM_COARSE_TC (default) -- A_c^{-1}
                             rounded to BF16 (a fixed symmetric matrix) times r_c
@@ -282,8 +285,10 @@ mfem_status mfem_solve_batch(mfem_ctx* ctx, const double* xf, int32_t B, double*
  * (all host or all device, as `memory` says), stats[i] host [B[i]] (stats or
  * stats[i] may be NULL).  The contexts must be distinct and on one device; the
  * work runs on ctxs[0]'s stream (the others' streams are synchronised first and
- * restored after the call).  PCG tiles are ctxs[0]'s.  Each result equals the
- * same pose solved alone.  With init = MFEM_INIT_WARM, pose b of a mesh starts
+ * restored after the call).  PCG tiles and threads per row are ctxs[0]'s.  Each
+ * result equals the same pose solved alone with the same tile_rows and spmv_split
+ * (mixed: whatever tile_rows, as far as FP64 sums in another order round to the
+ * same FP32 step lengths).  With init = MFEM_INIT_WARM, pose b of a mesh starts
  * from the last solution held in that mesh's slot b (see mfem_options.init). */
 mfem_status mfem_solve_multi(mfem_ctx* const* ctxs, int32_t n_ctx, const double* const* xf,
                              const int32_t* B, double* const* out, int32_t memory,

@@ -18,13 +18,18 @@ thread_local std::string g_thread_err = "no error";
 constexpr double kLsC = 1.0e-4;      // Armijo constant
 constexpr int kLsMax = 20;           // halvings
 constexpr double kLsNoise = 1.0e-10; // predicted decrease below this * |E|: take the step
-// SpMV rows per block the autotuner times.  64 (still an option) is slower with one
-// thread per row: us per launched iteration at 64 / 128 / 256 rows, 16 poses of the
-// 200k figure 71.5 / 69.5 / 69.1, 4 poses of the 800k figure 78.6 / 74.1 / 72.3.
+// SpMV rows per block.  FP64: fixed, because the order of its sums over the blocks shows in
+// the results, which must not depend on a timing or on the calls before (and 128 is the
+// faster, us per iteration at 128 / 256 rows: 40 poses of 10k tets 71.0 / 72.3, 8 poses of
+// 50k 51.5 / 57.3, 8 of 200k 149.7 / 155.4).  Mixed: timed on the first streamed table;
+// 64 (still an option) is slower with one thread per row: us per launched iteration at
+// 64 / 128 / 256 rows, 16 poses of the 200k figure 71.5 / 69.5 / 69.1, 4 poses of the 800k
+// figure 78.6 / 74.1 / 72.3.
+constexpr int kTile64 = 128;
 constexpr int kPcgTiles[2] = {128, 256};
+constexpr int kTileDefault = 256;   // mixed, until a streamed solve has been timed
 constexpr int kResIters = 1 << 13;   // most iterations of a batch's resident launch but one: ~0.15 s
 constexpr int kResRest = 256;        // PCG rounds streamed after a resident launch's wait ran out (some tens of calls)
-constexpr int kTileDefault = 256;               // until a streamed solve has been timed
 constexpr int kPcgChunk = 16;                   // PCG iterations enqueued between convergence checks (no history)
 constexpr int kPcgChunkMin = 16, kPcgChunkMax = 64;   // bounds of a predicted chunk (multiples of 8)
 constexpr int kResStages = 4;                   // 32 KB chunks of A_c^{-1} the resident kernel's ring holds
@@ -118,6 +123,11 @@ size_t coarse_ks(const mfem_ctx* c) { return ((size_t)c->mesh.coarse_n + kCoarse
 
 // bytes of the control block of B problems (see alloc_slots)
 size_t ctl_bytes(size_t B) { return B * (2 * sizeof(int) + 2 * sizeof(double)); }
+
+// SpMV rows per block of the tables of one precision in the calls that c leads
+int tile_of(const mfem_ctx* c, int prec) {
+    return prec == 0 ? c->tile_rows64 : (c->tile_rows ? c->tile_rows : kTileDefault);
+}
 
 int part_tiles_for(const mfem_ctx* c) {
     int a = (c->plan.n + 31) / 32, b = (c->plan.m + kTetTile - 1) / kTetTile;
@@ -251,8 +261,8 @@ void end_profile(mfem_ctx* c) {
     P.coarse_launches = c->prof.coarse_launches;
     P.coarse_tc = c->mesh.coarse_n > 0 && c->mesh.coarse_tc ? 1 : 0;
     P.pcg_iters = c->prof.pcg_iters;
-    P.tile_rows = c->tile_rows ? c->tile_rows : kTileDefault;
-    P.spmv_split = c->spmv_split ? c->spmv_split : 1;
+    P.tile_rows = tile_of(c, c->slot.prec);
+    P.spmv_split = c->spmv_split;
     P.grid_blocks = c->grid_blocks;
     for (int i = 0; i < c->prof.used; ++i) {
         float ms = 0.f;
@@ -473,7 +483,8 @@ template <typename T>
 bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vector<mfem_ctx*>& owner, int tile,
                    ResShape& sh, std::vector<ResJob>& jobs) {
     const ResLimits& lim = c->res_lim;
-    if (lim.sms <= 0 || c->res_rest > 0) return false;
+    // two threads per row add a row's sum in two halves; the resident kernel does not
+    if (lim.sms <= 0 || c->res_rest > 0 || c->spmv_split == 2) return false;
     sh = ResShape{};
     sh.rtile = tile;
     const size_t np = d.size();
@@ -481,7 +492,7 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
     std::vector<size_t> bytes(np);
     int need = 0, most = 0;
     for (size_t i = 0; i < np; ++i) {
-        if (owner[i]->opt.spmv_split == 2 || (d[i].coarse && !d[i].ctc)) return false;
+        if (d[i].coarse && !d[i].ctc) return false;
         units[i] = (d[i].n_rows + kCoarseRows - 1) / kCoarseRows;
         bytes[i] = (size_t)owner[i]->plan.slice_ptr.back() * (9 * sizeof(T) + 4);
         g[i] = (units[i] + kResUnits - 1) / kResUnits;
@@ -548,19 +559,15 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
     return true;
 }
 
-int tile_of(const mfem_ctx* c) { return c->tile_rows ? c->tile_rows : kTileDefault; }
-int split_of(const mfem_ctx* c) { return c->spmv_split ? c->spmv_split : 1; }
-
-// Whether run_pcg takes the problems of precision T inside PCG to the resident kernel.
-template <typename T>
-bool fits_chip(mfem_ctx* c, std::vector<Group>& gs, int tile, int prec) {
-    std::vector<PcgDesc<T>> d;
+// Whether run_pcg takes the mixed path's problems inside PCG to the resident kernel.
+bool fits_chip(mfem_ctx* c, std::vector<Group>& gs, int tile) {
+    std::vector<PcgDesc<float>> d;
     std::vector<mfem_ctx*> owner;
     int u = 0, uu = 0;
-    build_descs<T>(gs, tile, prec, d, u, uu, nullptr, &owner);
+    build_descs<float>(gs, tile, 1, d, u, uu, nullptr, &owner);
     ResShape sh;
     std::vector<ResJob> jobs;
-    return d.empty() || plan_resident<T>(c, d, owner, tile, sh, jobs);
+    return d.empty() || plan_resident<float>(c, d, owner, tile, sh, jobs);
 }
 
 template <typename T>
@@ -762,13 +769,15 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
     return MFEM_OK;
 }
 
-// Pick the SpMV's shape -- rows per block (kPcgTiles) and threads per row
-// (1, 2) -- for calls that `lead` leads, by timing a fixed number of PCG iterations of
-// each candidate on the first assembled system of group g (results are discarded; PCG
-// is re-initialised afterwards).  g may belong to another context than `lead`: only
-// g's own buffers are written.  A shape fixed by the lead's options is not searched.
+// Pick the rows per block (kPcgTiles) of the mixed path's SpMV for calls that `lead`
+// leads, by timing a fixed number of PCG iterations of each candidate on the first
+// assembled system of group g (results are discarded; PCG is re-initialised afterwards).
+// g may belong to another context than `lead`: only g's own buffers are written.
 // MFEM_AUTOTUNE_CACHE names a file of earlier picks ("key tile split" lines; any
-// supported tile).
+// supported tile).  Threads per row are not searched: the split of a row's sum shows in
+// the results, and two were slower in every table timed, by 11% (one pose of 800k, FP32
+// coarse product) to 38% (24 poses of 20k); 16 poses of 200k, corot, 97.4 -> 125 us an
+// iteration, 8 FP64 ones 150 -> 205.
 mfem_status autotune_tile(mfem_ctx* lead, const Group& g) {
     mfem_ctx* c = g.ctx;
     std::vector<Group> gs{g};
@@ -776,11 +785,6 @@ mfem_status autotune_tile(mfem_ctx* lead, const Group& g) {
     char key[128];
     snprintf(key, sizeof key, "%d %d %lld %d %d", c->plan.n, c->plan.m, (long long)c->plan.nnz_blocks,
              c->slot.prec, g.B);
-    std::vector<int> tiles, splits;
-    if (lead->opt.tile_rows) tiles.push_back(lead->opt.tile_rows);
-    else tiles.assign(std::begin(kPcgTiles), std::end(kPcgTiles));
-    for (int sp = 1; sp <= 2; ++sp)
-        if (!lead->opt.spmv_split || sp == lead->opt.spmv_split) splits.push_back(sp);
     if (cache) {
         if (FILE* f = fopen(cache, "r")) {
             char line[256];
@@ -788,59 +792,52 @@ mfem_status autotune_tile(mfem_ctx* lead, const Group& g) {
                 int tile = 0, sp = 1;
                 size_t kl = strlen(key);
                 if (strncmp(line, key, kl) == 0 && sscanf(line + kl, " %d %d", &tile, &sp) >= 1 &&
-                    (lead->opt.tile_rows ? tile == lead->opt.tile_rows : pcg_tile_supported(tile)) &&
-                    std::find(splits.begin(), splits.end(), sp) != splits.end()) {
+                    pcg_tile_supported(tile) && sp == lead->spmv_split)
                     lead->tile_rows = tile;
-                    lead->spmv_split = sp;
-                }
             }
             fclose(f);
-            if (lead->tile_rows && lead->spmv_split) return MFEM_OK;
+            if (lead->tile_rows) return MFEM_OK;
         }
     }
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     float best = 1e30f;
-    int best_tile = tiles.back(), best_split = splits.front();
+    int best_tile = kTileDefault;
     for (int b = 0; b < g.B; ++b) g.ph[b].coarse = 0;   // timed with block Jacobi
     ElemArgs a = elem_args(c);
-    for (int tile : tiles)
-        for (int sp : splits)
-            for (int rep = 0; rep < 2; ++rep) {
-                launch_pcg_init(a, g.B, tile, 0.0, 1 << 30, nullptr, nullptr, c->stream);
-                CK(cudaEventRecord(e0, c->stream));
-                mfem_status st = c->slot.prec == 1 ? run_pcg<float>(c, gs, 1, tile, sp, 20, false)
-                                                   : run_pcg<double>(c, gs, 0, tile, sp, 20, false);
-                if (st != MFEM_OK) return st;
-                CK(cudaEventRecord(e1, c->stream));
-                CK(cudaEventSynchronize(e1));
-                c->ring_pos = 0;
-                float ms = 0.f;
-                cudaEventElapsedTime(&ms, e0, e1);
-                if (rep == 1 && ms < best) {
-                    best = ms;
-                    best_tile = tile;
-                    best_split = sp;
-                }
+    for (int tile : kPcgTiles)
+        for (int rep = 0; rep < 2; ++rep) {
+            launch_pcg_init(a, g.B, tile, 0.0, 1 << 30, nullptr, nullptr, c->stream);
+            CK(cudaEventRecord(e0, c->stream));
+            mfem_status st = run_pcg<float>(c, gs, 1, tile, lead->spmv_split, 20, false);
+            if (st != MFEM_OK) return st;
+            CK(cudaEventRecord(e1, c->stream));
+            CK(cudaEventSynchronize(e1));
+            c->ring_pos = 0;
+            float ms = 0.f;
+            cudaEventElapsedTime(&ms, e0, e1);
+            if (rep == 1 && ms < best) {
+                best = ms;
+                best_tile = tile;
             }
+        }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     lead->tile_rows = best_tile;
-    lead->spmv_split = best_split;
     if (cache) {
         if (FILE* f = fopen(cache, "a")) {
-            fprintf(f, "%s %d %d\n", key, best_tile, best_split);
+            fprintf(f, "%s %d %d\n", key, best_tile, lead->spmv_split);
             fclose(f);
         }
     }
     return MFEM_OK;
 }
 
-// The first streamed PCG of calls that c leads: times the shapes (a resident solve has
-// none).  Decided on the table that run_pcg will see, every group's problems that start
-// now (`starts`) among it, before any of them is initialised; timed on the largest group
-// of a precision that is streamed.
+// The first streamed mixed PCG of calls that c leads: times the shapes (a resident solve
+// has none).  Decided on the table that run_pcg will see, every group's problems that
+// start now (`starts`) among it, before any of them is initialised; timed on the largest
+// mixed group.
 mfem_status search_shape(mfem_ctx* c, std::vector<Group>& gs, const std::vector<std::vector<int>>& starts,
                          bool per_request) {
     std::vector<std::vector<ProbHost>> keep(gs.size());
@@ -858,15 +855,14 @@ mfem_status search_shape(mfem_ctx* c, std::vector<Group>& gs, const std::vector<
         keep[gi].assign(gs[gi].ph, gs[gi].ph + gs[gi].B);
         mark(gi, false);
     }
-    const int tile = c->tile_rows ? c->tile_rows : kTileDefault;
-    const bool streamed[2] = {per_request || !fits_chip<double>(c, gs, tile, 0),
-                              per_request || !fits_chip<float>(c, gs, tile, 1)};
+    const bool streamed = per_request || !fits_chip(c, gs, tile_of(c, 1));
     restore();
+    if (!streamed) return MFEM_OK;
     size_t pick = gs.size();
     int64_t most = 0;
     for (size_t gi = 0; gi < gs.size(); ++gi) {
         const int64_t rows = std::count(starts[gi].begin(), starts[gi].end(), 1) * (int64_t)gs[gi].ctx->plan.n;
-        if (!streamed[gs[gi].ctx->slot.prec] || rows <= most) continue;
+        if (gs[gi].ctx->slot.prec != 1 || rows <= most) continue;
         most = rows;
         pick = gi;
     }
@@ -1158,7 +1154,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 start[b] = 1;
             }
         }
-        if (c->tile_rows == 0 || c->spmv_split == 0) {
+        if (c->tile_rows == 0) {
             mfem_status st = search_shape(c, gs, starts, per_request);
             if (st != MFEM_OK) return st;
         }
@@ -1230,7 +1226,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                 launch_agg_rotations(elem_args(gc), g.B, s);
                 gc->prof.launches++;
             }
-            launch_pcg_init(elem_args(gc), g.B, tile_of(c), 0.0, gc->opt.cg_max, gc->slot.tol2,
+            launch_pcg_init(elem_args(gc), g.B, tile_of(c, gc->slot.prec), 0.0, gc->opt.cg_max, gc->slot.tol2,
                             gc->slot.coarse_on, s);
             gc->prof.launches++;
             for (int b = 0; b < g.B; ++b)
@@ -1257,9 +1253,9 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
             if (g.ctx->slot.prec == prec)
                 for (int b = 0; b < g.B; ++b) any |= g.ph[b].active && g.ph[b].in_pcg;
         if (!any) continue;
-        mfem_status st = prec == 1 ? run_pcg<float>(c, gs, 1, tile_of(c), split_of(c), 0, true, true, true,
+        mfem_status st = prec == 1 ? run_pcg<float>(c, gs, 1, tile_of(c, 1), c->spmv_split, 0, true, true, true,
                                                     per_request, &ahead[prec])
-                                   : run_pcg<double>(c, gs, 0, tile_of(c), split_of(c), 0, true, true, true,
+                                   : run_pcg<double>(c, gs, 0, tile_of(c, 0), c->spmv_split, 0, true, true, true,
                                                      per_request, &ahead[prec]);
         if (st != MFEM_OK) return st;
     }
@@ -1411,6 +1407,7 @@ mfem_ctx* ctx_slot_clone(mfem_ctx* src, int cap, cudaStream_t stream, mfem_statu
     c->mesh_shared = true;
     c->slot.prec = src->slot.prec;
     c->tile_rows = src->tile_rows;
+    c->tile_rows64 = src->tile_rows64;
     c->spmv_split = src->spmv_split;
     c->res_lim = src->res_lim;
     c->owned_by_server = true;
@@ -1623,7 +1620,8 @@ mfem_status mfem_create(const double* rest_verts, int32_t n, const int32_t* tets
     c->model = mat->model;
     c->slot.prec = o.precision == MFEM_MIXED ? 1 : 0;
     c->tile_rows = o.tile_rows;
-    c->spmv_split = o.spmv_split;
+    c->tile_rows64 = o.tile_rows ? o.tile_rows : kTile64;
+    c->spmv_split = o.spmv_split ? o.spmv_split : 1;
     const Plan& P = c->plan;
     if (cudaGetDevice(&c->device) != cudaSuccess) return fail(MFEM_ECUDA, "no CUDA device");
     if (cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking) != cudaSuccess)
