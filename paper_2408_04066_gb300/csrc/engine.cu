@@ -644,13 +644,8 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
         if (resident && !per_request) chunk = std::min(cap, kResIters) + 1;
     }
     for (int done = 0; done < cap; done += chunk) {
-        const int n_it = resident ? chunk : std::min(chunk, cap - done);
+        int n_it = resident ? chunk : std::min(chunk, cap - done);
         if (one_chunk && done > 0) break;
-        if (one_chunk)
-            for (auto& g : gs)
-                if (g.ctx->slot.prec == prec)
-                    for (int b = 0; b < g.B; ++b)
-                        if (g.ph[b].active && g.ph[b].in_pcg) g.ph[b].pcg_launched += n_it;
         int pe = count ? c->prof.begin(2, c->stream) : -1;
         if (resident) {
             rsh.iters = n_it;
@@ -665,14 +660,18 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
                 cudaGetLastError();
                 c->res_lim.sms = 0;   // the device cannot hold it: streamed kernels from now on
                 resident = false;
-                chunk = kPcgChunk;
+                n_it = std::min(kPcgChunk, cap);
             }
         }
         if (!resident) {
-            mfem_status lst = launch_chunk<T>(c, dst, (int)d.size(), units, units_u, tile, split,
-                                              std::min(n_it, kPcgChunkMax), jobs);
+            mfem_status lst = launch_chunk<T>(c, dst, (int)d.size(), units, units_u, tile, split, n_it, jobs);
             if (lst != MFEM_OK) return lst;
         }
+        if (one_chunk)
+            for (auto& g : gs)
+                if (g.ctx->slot.prec == prec)
+                    for (int b = 0; b < g.B; ++b)
+                        if (g.ph[b].active && g.ph[b].in_pcg) g.ph[b].pcg_launched += n_it;
         if (resident && count) {
             c->prof.end(pe, c->stream);
             c->prof.launches++;
@@ -718,8 +717,8 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
         // (one host round trip a Newton step instead of two)
         if (resident && !per_request && ahead && n_it > cap) {
             *ahead = true;
-            c->ahead_jobs = nj;
-            c->ahead_bytes = coarse_bytes;
+            c->ahead_jobs[prec] = nj;
+            c->ahead_bytes[prec] = coarse_bytes;
             return MFEM_OK;
         }
         bool any = false;
@@ -1084,7 +1083,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
     if (any_elem) {
         CK(cudaStreamSynchronize(s));
         synced(gs);
-        int ran = 0;   // iterations of the resident solves read back now
+        int ran[2] = {0, 0};   // iterations of the resident solves read back now, by precision
         std::vector<std::vector<int>> starts(gs.size());
         for (size_t gi = 0; gi < gs.size(); ++gi) {
             Group& g = gs[gi];
@@ -1113,7 +1112,7 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                         continue;
                     }
                     finish_pcg(gc, b, p, p.it - 1);
-                    ran = std::max(ran, gc->sc_host[b].iter);
+                    ran[gc->slot.prec] = std::max(ran[gc->slot.prec], gc->sc_host[b].iter);
                     if (p.spec) p.spec_slope = gc->sc_host[b].slope;
                     if (p.spec && !(-p.spec_slope > kLsNoise * std::fabs(p.spec_e0))) p.spec = 0;
                 }
@@ -1236,10 +1235,11 @@ mfem_status advance(std::vector<Group>& gs, bool per_request) {
                     g.ph[b].pcg_seen = 0;
                 }
         }
-        // counted as the streamed kernels' launch pairs
-        c->prof.pcg_launches += 2 * ran;
-        c->prof.coarse_launches += c->ahead_jobs * ran;
-        c->prof.pcg_bytes += c->ahead_bytes * ran;
+        for (int prec = 0; prec < 2; ++prec) {   // counted as the streamed kernels' launch pairs
+            c->prof.pcg_launches += 2 * ran[prec];
+            c->prof.coarse_launches += c->ahead_jobs[prec] * ran[prec];
+            c->prof.pcg_bytes += c->ahead_bytes[prec] * ran[prec];
+        }
     }
     // ---- a5: one chunk of PCG iterations over every problem inside PCG
     bool any_pcg = false;

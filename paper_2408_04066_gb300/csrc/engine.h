@@ -113,8 +113,8 @@ struct mfem_ctx {
     mfem::Profiler prof;
     // PCG chunks captured as CUDA graphs, keyed by the launch parameters
     std::map<std::string, cudaGraphExec_t> graphs;
-    int ahead_jobs = 0;          // coarse jobs and bytes an iteration of the resident solve not read yet
-    double ahead_bytes = 0.0;
+    int ahead_jobs[2] = {0, 0};   // by precision: coarse jobs and bytes an iteration of the resident solves not read yet
+    double ahead_bytes[2] = {0.0, 0.0};
     bool graphs_off = false;   // capture failed once (e.g. a stream that cannot capture)
     mfem::ResLimits res_lim;   // what the device holds of the resident PCG kernel (sms = 0: not used)
     int res_expire = -1;       // mfem_expire_wait: the next resident launch's `expire`

@@ -74,3 +74,23 @@ def test_search_when_only_the_whole_table_is_too_large(tmp_path, monkeypatch):
         alone.close()
     for c in ctxs:
         c.close()
+
+
+def test_profile_of_two_precisions_in_one_call():
+    """Resident solves of both precisions in one call are counted each by its own iterations and
+    coarse bytes: the call's sums are those of the meshes solved alone."""
+    from paper_2408_04066_gb300 import mfem
+    cfgs = [dict(figure_config(3000, seeds=[5]), model="corot"), dict(figure_config(30000, seeds=[6]), model="corot")]
+    ctxs = [mfem.Context.from_config(c, precision=p, max_batch=1, init="rigid")
+            for c, p in zip(cfgs, ("fp64", "mixed"))]
+    alone = []
+    for c, cfg in zip(ctxs, cfgs):
+        c.solve_batch(cfg["xfs"])
+        alone.append(c.profile())
+    mfem.solve_multi(ctxs, [c["xfs"] for c in cfgs])
+    both = [c.profile() for c in ctxs]
+    for k in ("pcg_launches", "coarse_launches", "pcg_iters", "pcg_bytes"):
+        a, b = sum(p[k] for p in alone), sum(p[k] for p in both)
+        assert abs(a - b) <= 1e-9 * a, k
+    for c in ctxs:
+        c.close()
