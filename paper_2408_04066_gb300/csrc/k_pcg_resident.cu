@@ -74,7 +74,7 @@ struct ResShared {
     uint64_t full[kResMaxStages], empty[kResMaxStages], done, vals;
     uint32_t tmem;
     int fail;                       // a wait of this CTA ran out
-    int gfail;                      // cluster: one of some CTA's did (written by that CTA between cluster barriers)
+    int gfail[2];                   // cluster: one of some CTA's did, in the set-up and in an iteration (tell_fail)
     int voff[kResUnits];            // byte offset of a unit's values in the value area, -1: read from global memory
     int slots[kResUnits];
     double wsum[kResMaxThreads / 32][3];
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         mbar_init(&S.done, 1);
         mbar_init(&S.vals, 1);
         S.fail = 0;
-        S.gfail = 0;
+        S.gfail[0] = S.gfail[1] = 0;
         S.st = ResState{sc->rho, sc->alpha, sc->beta, sc->rr0, sc->rr, sc->tol2, sc->first, sc->iter, sc->maxit,
                         sc->state, 0.0, 0.0};
         if (!S.st.first) {
@@ -402,24 +402,26 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
 #pragma unroll
         for (int i = 0; i < NB; ++i)
             if (c0[i] >= 0) c0[i] = u_address(c0[i]);
-    // a failed wait is told to every CTA of the cluster before its next barrier and
-    // looked at after it, so that all leave together and none reads the memory of one
-    // that has left; S.fail itself is written by this CTA alone, so that its threads
-    // agree on it at a block barrier
-    auto tell_fail = [&]() {
+    // A failed wait of a cluster's CTA is told to all of them before a barrier and looked
+    // at after that barrier only, so that all leave together and none reads the memory
+    // of one that has left.  The word of the set-up is written before the set-up's last
+    // barrier alone; that of the iterations before the coarse product's barrier, with two
+    // barriers more between a look at it and the next write.  (A look after any other
+    // barrier could meet the next iteration's write in some threads and not in others.)
+    // S.fail is written by its own CTA alone, between block barriers.
+    auto tell_fail = [&](int k) {
         if (CLUSTER && t == 0 && S.fail)
             for (int rk = 0; rk < G; ++rk)
-                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(smem_u32(&S.gfail), rk)), "r"(1) : "memory");
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(smem_u32(&S.gfail[k]), rk)), "r"(1) : "memory");
     };
-    auto failed = [&]() { return (CLUSTER ? S.gfail : S.fail) != 0; };   // after a group barrier
     if (CLUSTER) {   // every CTA of the cluster runs before the first remote access
         cluster_arrive();
         cluster_wait();
-        tell_fail();
+        tell_fail(0);
         cluster_arrive();
         cluster_wait();
     }
-    const bool go = CLUSTER ? !failed() : landed;
+    const bool go = CLUSTER ? !S.gfail[0] : landed;
     // FP64, one unit a CTA: an FP64 instruction holds a scheduler for 64 cycles and
     // the unit's two warps would use two of the four, so six warps form the product,
     // a component of w each (bar of 1536 tets: an iteration 19.8 -> 16.4 us)
@@ -463,7 +465,11 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
     bool active = true;
     for (int it = 0; go && it < sh.iters; ++it) {
         T u[3] = {zb[0], zb[1], zb[2]};
-        if (t == 0 && it == sh.expire && rank == G - 1) S.fail = 1;   // tests
+        if (it == sh.expire) {   // tests
+            __syncthreads();
+            if (t == 0 && rank == G - 1) S.fail = 1;
+            __syncthreads();
+        }
         if (coarse) {
             // ---- coarse product: this CTA's units
             int a_at = 0;   // chunks issued this iteration (thread 0)
@@ -582,10 +588,10 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                     }
                     load_next();
                 }
-            tell_fail();
+            tell_fail(1);
             arrive();
             wait();
-            if (failed()) break;
+            if (CLUSTER ? S.gfail[1] : S.fail) break;
             // ---- u = zb + Q_a P_i e_a, the parts of e_a added in part order
             float ev = 0.f;
             if (lane < 6 && ul < nu) {
@@ -615,7 +621,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         const Partial<T> d0 = dot3_partial(r[0], r[1], r[2], u[0], u[1], u[2]);
         const Partial<T> d2 = dot3_partial(r[0], r[1], r[2], r[0], r[1], r[2]);
         wait();
-        if (failed()) break;
+        if (!CLUSTER && S.fail) break;
         // ---- w = K u
         T a0 = 0, a1 = 0, a2 = 0;
         if (by_comp) {
@@ -694,7 +700,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         }
         arrive();
         wait();
-        if (failed()) break;
+        if (!CLUSTER && S.fail) break;
         double tot[3] = {0.0, 0.0, 0.0};   // valid in thread 0
         if (sizeof(T) == 8) {
             const int nw = sh.rtile / 32, n_tiles = (n + sh.rtile - 1) / sh.rtile, n_warps = (n + 31) / 32;
@@ -834,7 +840,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         }
         if (coarse) {
             wait();
-            if (failed()) break;
+            if (!CLUSTER && S.fail) break;
         }
     }
 
@@ -857,7 +863,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
     }
     if (t == 0) {
         // a word of its own: one block may fail and another of its group not
-        if (S.fail || S.gfail) {
+        if (S.fail || S.gfail[0] || S.gfail[1]) {
             sc->fault = 1u;
         } else if (rank == 0) {
             sc->rho = S.st.rho;

@@ -108,3 +108,20 @@ def test_cut_short_served_request():
         assert np.array_equal(x, ref[0][0])
         assert (st["newton_iters"], st["pcg_iters"]) == (ref[1][0]["newton_iters"], ref[1][0]["pcg_iters"])
     srv.close()
+
+
+def test_cut_short_at_any_iteration():
+    """One cluster of which a block without coarse units tells the others, at every iteration of
+    the first solve: it may run ahead of blocks that have not yet left the barrier before."""
+    from paper_2408_04066_gb300 import mfem
+    cfg = dict(config("fig3000"), model="corot")
+    xf = np.asarray(cfg["xfs"])[:1]
+    ref = None
+    for iteration in range(-1, 16):
+        ctx = mfem.Context.from_config(cfg, tile_rows=128, spmv_split=1, max_batch=1)
+        ctx.expire_wait(iteration)
+        x, st = ctx.solve_batch(xf)
+        if ref is None:
+            ref, st0 = x, st
+        assert np.array_equal(x, ref) and st[0]["pcg_iters"] == st0[0]["pcg_iters"], iteration
+        ctx.close()
