@@ -137,14 +137,16 @@ __device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, u
         : "memory");
 }
 
-// The neighbour records of up to NB slots of a row (-1: none): column ids into nb,
-// or, in a cluster, shared-memory addresses of the owning CTA's u
+// The neighbour records of up to NB slots of a row (kNone: none): column ids into nb,
+// or, in a cluster, shared-memory addresses (any but kNone, which is not aligned) of the
+// owning CTA's u
+constexpr int kNone = -1;
 template <typename T, int NB, bool CLUSTER>
 __device__ __forceinline__ void gather(const T* nb, const int (&c)[NB], T (&q)[NB][3]) {
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
         q[i][0] = q[i][1] = q[i][2] = (T)0;
-        if (c[i] < 0) continue;
+        if (c[i] == kNone) continue;
         if (CLUSTER) ld_cluster((uint32_t)c[i], q[i]);
         else ld4(nb + 4 * (size_t)c[i], q[i]);
     }
@@ -152,14 +154,14 @@ __device__ __forceinline__ void gather(const T* nb, const int (&c)[NB], T (&q)[N
 template <int NB>
 __device__ __forceinline__ void load_cols(const int* cp, int k, int w, int (&c)[NB]) {
 #pragma unroll
-    for (int i = 0; i < NB; ++i) c[i] = k + i < w ? cp[32 * (k + i)] : -1;
+    for (int i = 0; i < NB; ++i) c[i] = k + i < w ? cp[32 * (k + i)] : kNone;
 }
 // w_i += those slots' products, in slot order
 template <typename T, int NB>
 __device__ __forceinline__ void products(const T* vp, const int (&c)[NB], const T (&q)[NB][3], T& a0, T& a1, T& a2) {
 #pragma unroll
     for (int i = 0; i < NB; ++i)
-        if (c[i] >= 0) {
+        if (c[i] != kNone) {
             const T* vv = vp + 288 * i;
             a0 += vv[0] * q[i][0] + vv[32] * q[i][1] + vv[64] * q[i][2];
             a1 += vv[96] * q[i][0] + vv[128] * q[i][1] + vv[160] * q[i][2];
@@ -389,7 +391,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
         if (landed && in_smem)   // column ids -> addresses, once
             for (int k = 0; k < w; ++k) {
                 int* cp = reinterpret_cast<int*>(vmem + c_at) + 32 * k;
-                if (*cp >= 0) *cp = u_address(*cp);
+                if (*cp != kNone) *cp = u_address(*cp);
             }
         // the other CTAs' copies start from this launch's residual
         if (coarse && has_cu)
@@ -401,7 +403,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
     if (CLUSTER && !in_smem)
 #pragma unroll
         for (int i = 0; i < NB; ++i)
-            if (c0[i] >= 0) c0[i] = u_address(c0[i]);
+            if (c0[i] != kNone) c0[i] = u_address(c0[i]);
     // A failed wait of a cluster's CTA is told to all of them before a barrier and looked
     // at after that barrier only, so that all leave together and none reads the memory
     // of one that has left.  The word of the set-up is written before the set-up's last
@@ -637,7 +639,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                     gather<T, 4, CLUSTER>(d.nb, c, q);
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        if (c[i] >= 0) {
+                        if (c[i] != kNone) {
                             const T* vv = vp + 288 * (k + i);
                             a += vv[0] * q[i][0] + vv[32] * q[i][1] + vv[64] * q[i][2];
                         }
@@ -669,7 +671,7 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
                     if (CLUSTER)
 #pragma unroll
                         for (int i = 0; i < NB; ++i)
-                            if (c[i] >= 0) c[i] = u_address(c[i]);
+                            if (c[i] != kNone) c[i] = u_address(c[i]);
                     gather<T, NB, CLUSTER>(d.nb, c, q);
                     products<T, NB>(vg + 288 * (size_t)k, c, q, a0, a1, a2);
                 }
