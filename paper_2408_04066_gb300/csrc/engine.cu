@@ -510,9 +510,10 @@ bool plan_resident(mfem_ctx* c, const std::vector<PcgDesc<T>>& d, const std::vec
     };
     sh.smem = res_smem_max();
     if (most <= 16) {
-        // the largest cluster size that leaves no CTA without rows and runs every
-        // problem at once: a smaller one halves the SMs that read a problem's matrix
-        // (11k tets, 47 units, through L2: 16 us an iteration on 8 CTAs, 11 on 16)
+        // the largest cluster size at which fewer than half of the smallest problem's
+        // CTAs have no rows (9 units take 16) and every problem runs at once: a smaller
+        // one halves the SMs that read a problem's matrix (11k tets, 47 units, through
+        // L2: 16 us an iteration on 8 CTAs, 11 on 16)
         int least = 0;
         for (size_t i = 0; i < np; ++i) least = i ? std::min(least, units[i]) : units[i];
         for (int k = kResClusterSizes - 1, cl = 16; k >= 0 && sh.cluster == 0; --k, cl /= 2) {

@@ -1,5 +1,6 @@
 // Coarse solve and correction of the two-level preconditioner on the tensor
-// cores, fused into one kernel per mesh and PCG iteration.
+// cores, fused into one kernel: one launch per PCG iteration serves up to
+// kCoarseJobs meshes.
 //
 // u = zb + P e,  e = A_c^{-1} r_c  for every two-level problem of one mesh: the
 // product is the one dense contraction of the solve (the preconditioner's
@@ -47,7 +48,7 @@ namespace {
 // Shared-memory ring of A + B chunks: four stages, one CTA an SM; two stages and
 // two CTAs an SM where a launch of several meshes has more CTAs than the device
 // has SMs, so that none waits for a second wave (12 + 12 streams of the 200k and
-// 50k figures 80.9 -> 78.6 us an iteration, the 10k/50k/200k requests 18.2 -> 17.7
+// 50k figures 80.0 -> 78.9 us an iteration, the 10k/50k/200k requests 18.75 -> 17.7
 // ms; one mesh alone is slower with two: 72.0 -> 74.8 us, 16 poses of the 200k figure).
 constexpr int kFuStages = 4, kFuStagesMulti = 2;
 constexpr int kFuThreads = 320;                   // 10 warps: one per 32 vertex rows of 5 x 64

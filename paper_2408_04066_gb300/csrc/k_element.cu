@@ -968,7 +968,6 @@ __global__ void __launch_bounds__(kTetTile) k_energy_trial(ElemArgs A) {
     double en[1] = {0.0};
     if (k < m) {
         const double* x = A.slot.x + (size_t)b * n * 3;
-        // the dx field: 4 elements per vertex
         const T* dx = (const T*)A.slot.vec + ((size_t)b * kVecStride + kOffRec + kRecDX) * npad32(n);   // three planes
         double xa[4][3], G[4][3], Q[3][3], F[3][3], S[6], sig[6];
         gather_x<T>(x, dx, A.slot.alpha[b], M.tet[k], xa, npad32(n));

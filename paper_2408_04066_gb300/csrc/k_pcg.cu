@@ -191,7 +191,8 @@ __device__ __forceinline__ int unit_problem(const PcgDesc<T>* __restrict__ D, in
 // shuffle trees over empty lanes (200k figure, 16 poses: 117.8 -> 114.0 us an
 // iteration); FP32 takes its totals with a warp per value, the scalars are
 // loaded before they are needed, and two of its three divisions are the update's
-// (inv_rho, inv_alpha).  FP64 keeps the order of its sums and its divisions, which
+// (inv_rho, inv_alpha; beta and the denominator are then rounded twice in FP64, an ulp
+// where FP32 step lengths keep 2^-24).  FP64 keeps the order of its sums and its divisions, which
 // its results show.
 template <typename T, int NT>
 __device__ __forceinline__ void spmv_commit(const PcgDesc<T>& d, ProbScal* sc, int tile, double v) {

@@ -1,12 +1,11 @@
 // Element outputs without any device allocation.
 //
-// mfem_get_elem stages the per-element results through a device buffer that it
-// allocates and frees on every call, and cudaFree waits for the whole device.
-// Callers that may allocate device memory only while they set up -- a per-frame
-// animation loop or a host application's plugin running inside a fixed device
-// budget -- cannot pay that.  mfem_get_elem_static runs the same kernel but
-// stages through the fixed array below, so it calls no cudaMalloc, cudaFree or
-// allocating library routine.
+// mfem_get_elem stages the per-element results in the context's element blocks.
+// mfem_get_elem_static runs the same kernel for callers that may allocate device
+// memory only while they set up -- a per-frame animation loop or a host
+// application's plugin running inside a fixed device budget -- and touches none of
+// the context's buffers: it stages through the fixed array below and calls no
+// cudaMalloc, cudaFree or allocating library routine.
 #include <cuda_runtime.h>
 
 #include <mutex>
