@@ -101,7 +101,8 @@ mfem_status upload(mfem_ctx* c, U** dst, const U* src, size_t count) {
     if (count == 0) return MFEM_OK;
     CK(cudaMalloc((void**)dst, count * sizeof(U)));
     c->mesh_bytes += count * sizeof(U);
-    CK(cudaMemcpy(*dst, src, count * sizeof(U), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(*dst, src, count * sizeof(U), cudaMemcpyHostToDevice, c->stream));
+    CK(cudaStreamSynchronize(c->stream));   // src may be a temporary
     return MFEM_OK;
 }
 
@@ -198,16 +199,17 @@ mfem_status alloc_slots(mfem_ctx* c, int B) {
         AL(S.aggq, B * (size_t)c->mesh.n_agg * 9 * sizeof(float));
         AL(S.epart, B * (size_t)4 * coarse_ld(c->mesh.coarse_n) * sizeof(float));
         AL(S.bsplit, coarse_b_bytes(c->mesh.coarse_n, B));
-        CK(cudaMemset(S.bsplit, 0, coarse_b_bytes(c->mesh.coarse_n, B)));   // columns past N stay zero
+        CK(cudaMemsetAsync(S.bsplit, 0, coarse_b_bytes(c->mesh.coarse_n, B), c->stream));   // columns past N stay zero
     }
 #undef AL
-    CK(cudaMemset(S.sc, 0, B * sizeof(ProbScal)));
-    CK(cudaMemset(S.val, 0, B * slots * 9 * kt));   // padding slots stay zero
-    CK(cudaMemset(S.vec, 0, B * kVecStride * npad32((int)n) * kt));
+    // on the context's stream, which the legacy stream's work is not ordered with
+    CK(cudaMemsetAsync(S.sc, 0, B * sizeof(ProbScal), c->stream));
+    CK(cudaMemsetAsync(S.val, 0, B * slots * 9 * kt, c->stream));   // padding slots stay zero
+    CK(cudaMemsetAsync(S.vec, 0, B * kVecStride * npad32((int)n) * kt, c->stream));
     S.cap = B;
     // every slot starts at the rest shape (the WARM start without history)
     for (int b = 0; b < B; ++b)
-        CK(cudaMemcpy(S.x + (size_t)b * n * 3, c->mesh.X, n * 3 * 8, cudaMemcpyDeviceToDevice));
+        CK(cudaMemcpyAsync(S.x + (size_t)b * n * 3, c->mesh.X, n * 3 * 8, cudaMemcpyDeviceToDevice, c->stream));
     c->warm_kind.assign(B, 0);
     c->xpred_valid.assign(B, 0);
     c->pcg_hist.assign((size_t)B * kPcgHistSteps, 0);
@@ -1791,7 +1793,8 @@ mfem_status mfem_set_forces(mfem_ctx* c, const double* f, int32_t n_sets) {
         c->fext_sets = 0;
         CK(cudaMalloc((void**)&c->fext_dev, cnt * sizeof(double)));
     }
-    CK(cudaMemcpy(c->fext_dev, perm.data(), cnt * sizeof(double), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(c->fext_dev, perm.data(), cnt * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
     c->fext_sets = n_sets;
     return MFEM_OK;
 }
