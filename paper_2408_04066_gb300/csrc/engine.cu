@@ -50,6 +50,7 @@ mfem_status ctx_fail(mfem_ctx* c, mfem_status s, const std::string& msg) {
 
 mfem_status cuda_check(mfem_ctx* c, cudaError_t e, const char* what) {
     if (e == cudaSuccess) return MFEM_OK;
+    cudaGetLastError();   // reported here: not again by the next call's check
     std::string msg = std::string(what) + ": " + cudaGetErrorString(e);
     return ctx_fail(c, e == cudaErrorMemoryAllocation ? MFEM_ENOMEM : MFEM_ECUDA, msg);
 }
@@ -216,6 +217,8 @@ mfem_status alloc_slots(mfem_ctx* c, int B) {
     // pinned host staging
     if (c->sc_host) cudaFreeHost(c->sc_host);
     if (c->ctl_ring) cudaFreeHost(c->ctl_ring);
+    c->sc_host = nullptr;
+    c->ctl_ring = nullptr;
     CK(cudaMallocHost((void**)&c->sc_host, B * sizeof(ProbScal)));
     CK(cudaMallocHost((void**)&c->ctl_ring, kStageRing * ctl_bytes(B)));
     c->alpha_host.assign(B, 0.0);
@@ -226,6 +229,8 @@ mfem_status alloc_slots(mfem_ctx* c, int B) {
     if (dcap > c->descs_cap) {
         if (c->descs_dev) cudaFree(c->descs_dev);
         if (c->descs_host) cudaFreeHost(c->descs_host);
+        c->descs_dev = c->descs_host = nullptr;
+        c->descs_cap = 0;
         CK(cudaMalloc(&c->descs_dev, dcap));
         CK(cudaMallocHost(&c->descs_host, dcap));
         c->descs_cap = dcap;
@@ -240,7 +245,14 @@ size_t slot_bytes_for(const mfem_ctx* c, int B) { return bytes_per_slot(c) * (si
 mfem_status ensure_slots(mfem_ctx* c, int B) {
     if (B <= c->slot.cap) return MFEM_OK;
     free_slots(c);
-    return alloc_slots(c, B);
+    const mfem_status st = alloc_slots(c, B);
+    if (st != MFEM_OK) {   // none at all rather than some: the next call that needs slots allocates its own
+        const std::string why = c->err;
+        free_slots(c);
+        c->pose_set = false;
+        c->err = why;
+    }
+    return st;
 }
 
 void begin_profile(mfem_ctx* c) {
@@ -596,6 +608,8 @@ mfem_status run_pcg(mfem_ctx* c0, std::vector<Group>& gs, int prec, int tile, in
         CK(cudaStreamSynchronize(c->stream));
         if (c->descs_dev) cudaFree(c->descs_dev);
         if (c->descs_host) cudaFreeHost(c->descs_host);
+        c->descs_dev = c->descs_host = nullptr;
+        c->descs_cap = 0;
         CK(cudaMalloc(&c->descs_dev, 2 * bytes));
         CK(cudaMallocHost(&c->descs_host, 2 * bytes));
         c->descs_cap = 2 * bytes;
@@ -1761,6 +1775,7 @@ mfem_status mfem_set_pose(mfem_ctx* c, const double* xf, int32_t H) {
     if (c->owned_by_server) return ctx_fail(c, MFEM_EINVAL, "context belongs to a server");
     if (H != c->plan.H) return ctx_fail(c, MFEM_EINVAL, "pose has the wrong number of handles");
     mfem_status st = validate_pose(c, xf, H);
+    if (st == MFEM_OK) st = ensure_slots(c, 1);
     if (st != MFEM_OK) return st;
     CK(cudaMemcpyAsync(c->slot.xf, xf, sizeof(double) * 12 * H, cudaMemcpyHostToDevice, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -1952,6 +1967,7 @@ mfem_status mfem_solve_multi(mfem_ctx* const* ctxs, int32_t n_ctx, const double*
 mfem_status mfem_get_elem(mfem_ctx* c, double* s, double* lam) {
     if (!c) return ctx_fail(nullptr, MFEM_EINVAL, "null context");
     if (!s && !lam) return MFEM_OK;
+    if (c->slot.cap < 1) return ctx_fail(c, MFEM_EINVAL, kNoState);
     const size_t m = c->plan.m;
     // staged in the element blocks, which only live inside a Newton step (84 values
     // a tet, 15 needed): a buffer allocated and freed here took 0.2 ms a call
@@ -1974,6 +1990,7 @@ mfem_status mfem_expire_wait(mfem_ctx* c, int32_t iteration) {
 mfem_status mfem_get_state(const mfem_ctx* cc, double* x) {
     mfem_ctx* c = const_cast<mfem_ctx*>(cc);
     if (!c || !x) return ctx_fail(c, MFEM_EINVAL, "null argument");
+    if (c->slot.cap < 1) return ctx_fail(c, MFEM_EINVAL, kNoState);
     launch_unpermute(elem_args(c), 1, c->slot.outbuf, c->stream);
     CK(cudaMemcpyAsync(x, c->slot.outbuf, sizeof(double) * 3 * c->plan.n, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -1984,6 +2001,8 @@ mfem_status mfem_set_state(mfem_ctx* c, const double* x) {
     if (!c || !x) return ctx_fail(c, MFEM_EINVAL, "null argument");
     for (size_t i = 0; i < 3 * (size_t)c->plan.n; ++i)
         if (!std::isfinite(x[i])) return ctx_fail(c, MFEM_EINVAL, "non-finite state");
+    const mfem_status st = ensure_slots(c, 1);
+    if (st != MFEM_OK) return st;
     CK(cudaMemcpyAsync(c->slot.outbuf, x, sizeof(double) * 3 * c->plan.n, cudaMemcpyHostToDevice, c->stream));
     launch_permute_in(elem_args(c), 0, c->slot.outbuf, c->stream);
     CK(cudaStreamSynchronize(c->stream));

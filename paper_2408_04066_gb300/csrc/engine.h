@@ -128,6 +128,7 @@ struct mfem_ctx {
 namespace mfem {
 
 constexpr int kStageRing = 64;
+constexpr const char* kNoState = "the context holds no state: its slots could not be allocated";
 
 // One Newton group: B problems of one context.
 struct Group {

@@ -57,6 +57,7 @@ extern "C" mfem_status mfem_get_elem_static(mfem_ctx* c, double* s, double* lam)
     if (cudaGetDevice(&dev) != cudaSuccess || dev != c->device)
         return mfem::ctx_fail(c, MFEM_EINVAL, "the context's device must be current");
     if (!s && !lam) return MFEM_OK;
+    if (c->slot.cap < 1) return mfem::ctx_fail(c, MFEM_EINVAL, mfem::kNoState);
     double* scratch = nullptr;
     mfem_status st = scratch_for_current_device(c, &scratch);
     if (st != MFEM_OK) return st;
