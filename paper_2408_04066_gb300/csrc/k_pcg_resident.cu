@@ -882,7 +882,12 @@ __global__ void __launch_bounds__(kCoarseRows * U, 1)
             sc->iter = S.st.iter;
             sc->state = S.st.state;
         }
-        // copies in flight land before the memory is released
+        // copies in flight land, and after a failed wait the matrix values and the products
+        // issued last as well, before the memory is released (each bounded again)
+        if (S.fail) {
+            mbar_wait(&S.vals, 0);
+            mbar_wait(&S.done, done_ph ^ 1u);
+        }
         if (keep) {
             for (int i = 0; i < n_ring; ++i) mbar_wait(&S.full[i], 0);
         } else {
