@@ -372,7 +372,9 @@ const char* mfem_last_error(const mfem_ctx* ctx);
  * while others are on the GPU are admitted at the next Newton-step boundary as
  * slots and device memory allow; all admitted requests of all meshes advance
  * together (each PCG iteration launch serves every admitted request).
- * Each request's result equals the same pose solved alone by mfem_solve_batch. */
+ * Each request's result equals the same pose solved alone by mfem_solve_batch with the
+ * first mesh's tile_rows and spmv_split, which every mesh of a server takes (see
+ * mfem_solve_multi). */
 
 /* device_mem_budget: bytes the server may hold for request slots and warm
  * state (0 = no limit); max_slots: requests admitted at once across meshes.
